@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkmc.so")
-SOURCES = ["kmc_sweep.cu", "kmc_setup.cu", "kmc_capi.cu", "kmc_noalloc.cu", "kmc_batch.cu"]
+SOURCES = ["kmc_sweep.cu", "kmc_ions.cu", "kmc_setup.cu", "kmc_capi.cu", "kmc_noalloc.cu", "kmc_batch.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -45,7 +45,7 @@ def _stale(target: str, deps) -> bool:
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(INCLUDE, "kmc.h"))
     objs = []
     jobs = []

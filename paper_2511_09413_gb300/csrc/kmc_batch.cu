@@ -75,22 +75,20 @@ void drop_graph(kmc_batch *b)
 // Work list for a CTA size: one item per tile of 32/LPR * warps rails, larger
 // tiles (longer rails) first so that the dynamic schedule ends evenly.
 // Work items of a list of devices: every device's rails cut into tiles of
-// (32 / lanes per rail) x warps rails, grouped by kernel shape and, within a
+// (32 / its shape's lanes per rail) x warps rails, grouped by kernel shape and, within a
 // shape, longest tiles first.  Returns the items and the shape offsets.
-void make_items(const std::vector<const kmc_params *> &devs, const std::vector<int> &inst, int warps,
-                std::vector<BatchItem> &sorted, int *cls_off)
+void make_items(const std::vector<const kmc_params *> &devs, const std::vector<TileShape> &shapes,
+                const std::vector<int> &inst, int warps, std::vector<BatchItem> &sorted, int *cls_off)
 {
     std::vector<BatchItem> items;
     std::vector<int64_t> cost;
     for (size_t i = 0; i < devs.size(); ++i) {
         const kmc_params &p = *devs[i];
-        int wpl = 1;
-        const int lpr = sweep_pick_lpr(p.n_sites, &wpl);
-        const int64_t tile = (int64_t)(32 / lpr) * warps;
+        const int64_t tile = (int64_t)(32 / shapes[i].lpr) * warps;
         for (int64_t r0 = 0; r0 < p.n_rails; r0 += tile) {
             BatchItem it;
             it.inst = inst[i];
-            it.kind = sweep_kind(lpr, wpl);
+            it.kind = shapes[i].kind;
             it.tile_rail0 = r0;
             items.push_back(it);
             cost.push_back(std::min<int64_t>(tile, p.n_rails - r0) * p.n_sites);
@@ -120,26 +118,44 @@ int build_items(kmc_batch *b, int warps)
     float p0max = 0.0f;
     for (const kmc_handle *h : b->dev) p0max = std::max(p0max, h->args.P0f_scalar);
     const int acc = b->acc_req >= 0 ? b->acc_req : (p0max >= kAcceptAutoP0 ? 1 : 0);
-    // shared memory of each shape's CTAs: the largest of its devices' tiles
+    // each device's tile, its shared memory (of each shape's CTAs: the largest of
+    // its devices') and its arguments.  The devices share the GPU: their tiles'
+    // lanes per rail follow from all rails together.
     BatchPlan plan{};
     std::vector<const kmc_params *> devs;
+    std::vector<TileShape> shapes;
     std::vector<int> inst;
+    std::vector<SweepArgs> host(b->dev.size());
+    int64_t rails = 0;
+    for (const kmc_handle *h : b->dev) rails += h->p.n_rails;
     for (size_t i = 0; i < b->dev.size(); ++i) {
-        const kmc_params &p = b->dev[i]->p;
+        const kmc_handle *h = b->dev[i];
+        const kmc_params &p = h->p;
+        const TileShape t = pick_tile(rails, p.n_rails, p.n_sites, p.electrodes == 1, h->n_tot, h->n_max, acc != 0);
+        host[i] = h->args;
+        const size_t need = tile_args(host[i], t, p, h->P0site != nullptr, warps, acc != 0);
+        plan.smem[t.kind] = std::max(plan.smem[t.kind], need);
+        devs.push_back(&p);
+        shapes.push_back(t);
+        inst.push_back((int)i);
+    }
+    // the occupancy words of every device have to fit as well: the limit of a CTA
+    // size does not depend on the filling
+    for (size_t i = 0; i < b->dev.size(); ++i) {
+        const kmc_params &p = *devs[i];
         int wpl = 1;
         const int lpr = sweep_pick_lpr(p.n_sites, &wpl);
-        const int k = sweep_kind(lpr, wpl);
-        plan.smem[k] = std::max(plan.smem[k], sweep_smem_bytes(lpr, wpl, p.n_zones, p.n_sites, warps,
-                                                               b->flush, acc != 0));
-        devs.push_back(&p);
-        inst.push_back((int)i);
+        if (sweep_smem_bytes(lpr, wpl, p.n_zones, p.n_sites, warps, b->flush, acc != 0) + 1024 > (size_t)max_smem)
+            return fail(KMC_E_ARG, "batch: shared memory for this CTA size exceeds the device limit");
     }
     for (int k = 0; k < kShapeKinds; ++k)
         if (plan.smem[k] + 1024 > (size_t)max_smem)
             return fail(KMC_E_ARG, "batch: shared memory for this CTA size exceeds the device limit");
     std::vector<BatchItem> sorted;
     int cls_off[kShapeKinds + 1];
-    make_items(devs, inst, warps, sorted, cls_off);
+    make_items(devs, shapes, inst, warps, sorted, cls_off);
+    BCK(cudaMemcpyAsync(b->inst, host.data(), sizeof(SweepArgs) * host.size(), cudaMemcpyHostToDevice, b->user),
+        "copy device arguments");
     if (b->items) cudaFreeAsync(b->items, b->user);
     b->items = nullptr;
     BCK(cudaMallocAsync((void **)&b->items, sizeof(BatchItem) * std::max<size_t>(1, sorted.size()),
@@ -286,15 +302,11 @@ int kmc_batch_create(const kmc_params *params, int32_t n_inst, const double *con
         (e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming)) != cudaSuccess ||
         (e = batch_set_smem_limit()) != cudaSuccess)
         return bail(cuda_fail(e, "batch streams"));
-    std::vector<SweepArgs> host(n_inst);
-    for (int i = 0; i < n_inst; ++i) host[i] = b->dev[i]->args;
     if ((e = cudaMallocAsync((void **)&b->inst, sizeof(SweepArgs) * n_inst, b->user)) != cudaSuccess ||
         (e = cudaMallocAsync((void **)&b->work_ctr, sizeof(unsigned) * kShapeKinds, b->user)) != cudaSuccess ||
         (e = cudaMallocAsync((void **)&b->t0, sizeof(int64_t) * 2, b->user)) != cudaSuccess)
         return bail(cuda_fail(e, "batch allocation"));
-    if ((e = cudaMemcpyAsync(b->inst, host.data(), sizeof(SweepArgs) * n_inst, cudaMemcpyHostToDevice,
-                             b->user)) != cudaSuccess ||
-        (e = cudaMemsetAsync(b->work_ctr, 0, sizeof(unsigned) * kShapeKinds, b->user)) != cudaSuccess ||
+    if ((e = cudaMemsetAsync(b->work_ctr, 0, sizeof(unsigned) * kShapeKinds, b->user)) != cudaSuccess ||
         (e = cudaMemsetAsync(b->t0, 0, sizeof(int64_t) * 2, b->user)) != cudaSuccess)
         return bail(cuda_fail(e, "batch set-up"));
     rc = build_items(b, b->warps);
@@ -522,22 +534,25 @@ int kmc_batch_grad_all(kmc_batch *b, const double *const *dLoss_dJ, const double
         // work items grouped by shape, longest tiles first in each; one
         // persistent launch per shape, its shared memory the largest tile's
         std::vector<const kmc_params *> devs;
+        std::vector<TileShape> shapes;
         std::vector<int> inst;
         BatchPlan plan{};
         for (int i = 0; i < n_inst; ++i) {
             if (!active[(size_t)i]) continue;
             const kmc_params &p = b->dev[(size_t)i]->p;
-            int wpl = 1;
-            const int lpr = sweep_pick_lpr(p.n_sites, &wpl);
-            const int k = sweep_kind(lpr, wpl);
-            plan.smem[k] = std::max(plan.smem[k], grad_smem_bytes(lpr, wpl, p.n_zones, p.n_sites, warps));
+            TileShape t{};
+            t.lpr = sweep_pick_lpr(p.n_sites, &t.wpl);
+            t.kind = sweep_kind(t.lpr, t.wpl);
+            plan.smem[t.kind] = std::max(plan.smem[t.kind],
+                                         grad_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps));
             devs.push_back(&p);
+            shapes.push_back(t);
             inst.push_back(i);
         }
         std::vector<BatchItem> sorted;
         int cls_off[kShapeKinds + 1];
-        make_items(devs, inst, warps, sorted, cls_off);
-        for (int k = 0; k < kShapeKinds; ++k) {
+        make_items(devs, shapes, inst, warps, sorted, cls_off);
+        for (int k = 0; k < kWordKinds; ++k) {
             const int n = cls_off[k + 1] - cls_off[k];
             plan.grid[k] = n > 0 ? std::min(n, sms * batch_ctas_per_sm(k, 2, warps, plan.smem[k])) : 0;
         }

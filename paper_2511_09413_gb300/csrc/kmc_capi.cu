@@ -120,8 +120,13 @@ int pick_launch(kmc_handle *h)
 {
     const kmc_params &p = h->p;
     SweepLaunch l{};
-    l.lpr = sweep_pick_lpr(p.n_sites, &l.wpl);
-    const int G = 32 / l.lpr;
+    l.acc = h->accept_req >= 0 ? h->accept_req : (h->args.P0f_scalar >= kAcceptAutoP0 ? 1 : 0);
+    const TileShape t = pick_tile(p.n_rails, p.n_rails, p.n_sites, p.electrodes == 1, h->n_tot, h->n_max,
+                                  l.acc != 0);
+    l.ions = t.ions;
+    l.kind = t.kind;
+    l.lpr = t.lpr;
+    l.wpl = t.wpl;
     int flush = h->flush_req > 0 ? h->flush_req : 256;
     int warps = h->warps_req > 0 ? h->warps_req : 8;
     warps = std::min(warps, 8);
@@ -130,17 +135,11 @@ int pick_launch(kmc_handle *h)
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (max_smem <= 0) max_smem = 48 * 1024;
     max_smem = std::min(max_smem, 200 * 1024);
-    l.acc = h->accept_req >= 0 ? h->accept_req : (h->args.P0f_scalar >= kAcceptAutoP0 ? 1 : 0);
-    const bool acc = l.acc != 0;
-    while (warps > 1 && sweep_smem_bytes(l.lpr, l.wpl, p.n_zones, p.n_sites, warps, flush,
-                                         acc) > (size_t)max_smem)
-        warps >>= 1;
-    while (flush > 1 && sweep_smem_bytes(l.lpr, l.wpl, p.n_zones, p.n_sites, warps, flush,
-                                         acc) > (size_t)max_smem)
-        flush >>= 1;
+    auto smem_for = [&](int w) { return tile_args(h->args, t, p, h->P0site != nullptr, w, l.acc != 0); };
+    while (warps > 1 && smem_for(warps) > (size_t)max_smem) warps >>= 1;
     l.warps = warps;
-    l.smem = sweep_smem_bytes(l.lpr, l.wpl, p.n_zones, p.n_sites, warps, flush, acc);
-    const int64_t rails_per_cta = (int64_t)G * warps;
+    l.smem = smem_for(warps);
+    const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * warps;
     l.grid = (int)((p.n_rails + rails_per_cta - 1) / rails_per_cta);
     h->launch = l;
     h->args.flush = flush;
@@ -261,7 +260,10 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         std::lock_guard<std::mutex> lk(g_alloc_mu);
         h->al = g_alloc;
     }
-    std::call_once(g_attr_once, [] { g_attr_err = sweep_set_smem_limits(); });
+    std::call_once(g_attr_once, [] { 
+        g_attr_err = sweep_set_smem_limits();
+        if (g_attr_err == cudaSuccess) g_attr_err = ion_set_smem_limits();
+    });
     if (g_attr_err != cudaSuccess) return cuda_fail(g_attr_err, "cudaFuncSetAttribute");
 
     const kmc_params &p = h->p;
@@ -276,7 +278,7 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
     h->Zc = (unsigned long long *)h->alloc(sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1) *
                                            (size_t)Z);
     h->log = (kmc_log_entry *)h->alloc(sizeof(kmc_log_entry) * (size_t)h->log_cap);
-    h->misc = (unsigned long long *)h->alloc(sizeof(unsigned long long) * 8);
+    h->misc = (unsigned long long *)h->alloc(sizeof(unsigned long long) * 16);
     h->args_dev = (SweepArgs *)h->alloc(sizeof(SweepArgs));
     h->occ_init = (uint8_t *)h->alloc(occ_bytes);
     h->Jr = (int64_t *)h->alloc(sizeof(int64_t) * (size_t)R);
@@ -291,7 +293,7 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
             return fail(KMC_E_NOMEM, "device allocation failed (P0 table)");
     }
     cudaStream_t s = h->stream;
-    CK(cudaMemsetAsync(h->misc, 0, sizeof(unsigned long long) * 8, s), "memset");
+    CK(cudaMemsetAsync(h->misc, 0, sizeof(unsigned long long) * 16, s), "memset");
     CK(cudaMemsetAsync(h->J, 0, sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1), s), "memset");
     CK(cudaMemsetAsync(h->Zc, 0, sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1) * (size_t)Z, s),
        "memset");
@@ -314,7 +316,9 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         if (rc) return rc;
     }
     unsigned long long *bad = h->misc + 5;
-    CK(setup_row_counts(h->occ, h->stride, (int32_t)R, (int32_t)L, h->N0, bad, s), "row counts");
+    CK(setup_row_counts(h->occ, h->stride, (int32_t)R, (int32_t)L, h->N0, bad, h->misc + 8,
+                        s),
+       "row counts");
     CK(setup_background(h->N0, (int32_t)R, (int32_t)L, (int32_t)Z, h->K, h->bgd, s), "background");
     CK(cudaMemcpyAsync(h->occ_init, h->occ, occ_bytes, cudaMemcpyDeviceToDevice, s), "checkpoint");
 
@@ -329,7 +333,7 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
     }
     // check derived values
     DevConst kc;
-    unsigned long long flags[8];
+    unsigned long long flags[16];
     CK(cudaMemcpyAsync(&kc, h->K, sizeof(kc), cudaMemcpyDeviceToHost, s), "copy constants");
     CK(cudaMemcpyAsync(flags, h->misc, sizeof(flags), cudaMemcpyDeviceToHost, s), "copy flags");
     CK(cudaStreamSynchronize(s), "create");
@@ -341,7 +345,9 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         return fail(KMC_E_ARG, "initial occupancy has %llu bytes that are not 0 or 1", flags[5]);
     if (Ea && (int)(flags[6] & 0xffffffffu) != 0)
         return fail(KMC_E_PROB, "per-site base probability outside [0, 1] (check Ea_site)");
-    CK(cudaMemsetAsync(h->misc, 0, sizeof(unsigned long long) * 8, s), "memset");
+    CK(cudaMemsetAsync(h->misc, 0, sizeof(unsigned long long) * 16, s), "memset");
+    h->n_tot = (int64_t)flags[8];
+    h->n_max = (int64_t)flags[9];
     fill_args(h);
     h->args.P0f_scalar = kc.P0f;
     h->args.E_inf = kc.E_inf;
@@ -589,7 +595,8 @@ int kmc_step_n(kmc_handle *h, int64_t n_steps)
         const int64_t n = std::min<int64_t>(n_steps, 1 << 30);
         h->args.t0 = h->t;
         h->args.n_steps = (int32_t)n;
-        cudaError_t e = sweep_launch(h->args, h->launch, h->stream);
+        cudaError_t e = h->launch.ions ? ion_launch(h->args, h->launch, nullptr, h->stream)
+                                       : sweep_launch(h->args, h->launch, nullptr, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
         e = zone_scan(h->Zc, h->t, (int)n, h->p.n_zones, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "zone-count scan launch");
@@ -734,7 +741,8 @@ int kmc_grad(kmc_handle *h, const double *dLoss_dJ, const double *dLoss_dZc, dou
         SweepArgs ga;
         int rc = grad_prepare(h, dLoss_dJ, dLoss_dZc, &ga);
         if (rc) return rc;
-        SweepLaunch l = h->launch;
+        SweepLaunch l{};
+        l.lpr = sweep_pick_lpr((int)L, &l.wpl);
         int dev = 0, max_smem = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

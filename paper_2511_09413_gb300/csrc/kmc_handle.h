@@ -44,6 +44,7 @@ struct kmc_handle {
     unsigned long long *misc = nullptr;  // [0] log count, [1..3] counters, [4] scratch count
     kmc::SweepArgs *args_dev = nullptr;       // device copy of args for the kernels' rare paths
     int64_t log_cap = 4096;
+    int64_t n_tot = 0, n_max = 0;             // ions in all and on the fullest rail at step 0
     uint8_t *occ_init = nullptr;              // occupancy at step 0: the gradient pass's checkpoint
     int64_t *Jr = nullptr;                    // [R] per-rail net leftward crossings so far
 

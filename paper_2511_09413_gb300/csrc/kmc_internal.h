@@ -32,6 +32,19 @@ struct DevConst {
     int32_t bnd[kMaxZones + 1];  // zone boundaries floor(z L / Z), z = 0..Z
 };
 
+// Shared memory of the ion-list tile (kmc_ions.cu): the CTA's site table, then
+// one block per warp.  Sizes and offsets (within a warp's block) in bytes.
+struct IonLayout {
+    uint32_t tab;     // the site table, uint4 [L + 2]
+    uint32_t row;     // one rail's decision bounds (after the block's fixed part)
+    uint32_t zf;      // float4 [G][Z]: B/(1+B), 1/(1+B), band factors (per-site barriers)
+    uint32_t p0b;     // float2 [G][Z]: per-site P0 bounds of the zone (per-site barriers)
+    uint32_t pb;      // int [G][Z + 1]: ions below each zone boundary
+    uint32_t st;      // uint32 [slots][32]: each lane's state words
+    uint32_t col;     // uint32 [rcap][32]: each lane's entries
+    uint32_t bytes;   // one warp's block
+};
+
 // Everything one sweep launch needs.  Passed by value (kernel parameter space).
 struct SweepArgs {
     uint8_t *occ;              // [R][stride] occupancy bytes
@@ -68,6 +81,9 @@ struct SweepArgs {
     float P0f_scalar;             // scalar P0 in FP32 (host copy of DevConst::P0f)
     float E_inf, E_outf;          // electrode base probabilities in FP32
     int32_t rule;                 // 0 synchronous update, 1 brick-wall (even/odd bonds)
+    int32_t rcap;                 // ion lists: rows of a lane's column
+    uint32_t rcpZ;                // ion lists: i / Z = (i rcpZ) >> 16 for i < 1024
+    IonLayout iy;                 // ion lists: shared memory
 
     // likelihood-ratio gradient pass only (unused by the forward sweep)
     // With the forward's totals J_t, Zc_t and the leave-one-out divisor R - 1,
@@ -102,17 +118,29 @@ constexpr int kGradState = 5;
 // One work item of a batched launch: a tile of rails of one device.
 struct BatchItem {
     int32_t inst;        // device index in the batch
-    int32_t kind;        // kernel shape (shape_kind of the device's lanes per rail)
+    int32_t kind;        // kernel shape of the device (TileShape::kind)
     int64_t tile_rail0;  // first rail of the tile
 };
 
-// Kernel shapes of the tile body: lanes per rail 1, 2, 4, 8, 16, 32 with one
-// 32-bit word per lane (kinds 0-5), and 32 lanes of two words (kind 6).
-constexpr int kShapeKinds = 7;
+// Kernel shapes of the occupancy-word tile: lanes per rail 1, 2, 4, 8, 16, 32
+// with one 32-bit word per lane (kinds 0-5), and 32 lanes of two words (kind 6);
+// then those of the ion-list tile: 4, 8, 16, 32 lanes per rail with 32 rows of
+// bits, and 32 lanes with 64, each with blocking and with open electrodes.
+constexpr int kWordKinds = 7;
+constexpr int kShapeKinds = kWordKinds + 10;
 __host__ __device__ constexpr int shape_kind(int lpr, int wpl)
 {
     return wpl == 2 ? 6 : lpr == 1 ? 0 : lpr == 2 ? 1 : lpr == 4 ? 2 : lpr == 8 ? 3 : lpr == 16 ? 4 : 5;
 }
+
+// The tile that advances a device, and its shape.
+struct TileShape {
+    int ions;    // 1: ion-list tile, 0: occupancy-word tile
+    int lpr;     // lanes per rail
+    int wpl;     // words per lane (occupancy-word tile)
+    int kind;    // kernel shape
+    int rcap;    // ion lists: slots of a lane's column
+};
 
 // Per-shape launches of a batch: CTAs and dynamic shared memory of each
 // shape's persistent launch (grid 0: the batch has no items of that shape).
@@ -141,8 +169,10 @@ struct BatchArgs {
 
 // Launch configuration chosen on the host.
 struct SweepLaunch {
+    int ions;     // 1: ion-list tile (kmc_ions.cu), 0: occupancy-word tile (kmc_sweep.cu)
+    int kind;     // kernel shape
     int lpr;      // lanes per rail (1..32)
-    int wpl;      // 32-bit words per lane (1 or 2)
+    int wpl;      // 32-bit words per lane (1 or 2; occupancy-word tile)
     int warps;    // warps per CTA
     size_t smem;  // dynamic shared memory bytes
     int grid;
@@ -155,10 +185,28 @@ constexpr double kAcceptAutoP0 = 1.0 / 128.0;
 
 size_t sweep_smem_bytes(int lpr, int wpl, int Z, int L, int warps, int flush, bool acc);
 int sweep_pick_lpr(int L, int *wpl);
-cudaError_t sweep_launch(const SweepArgs &a, const SweepLaunch &l, cudaStream_t s);
+cudaError_t sweep_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s);
 // zone-count trace of steps [t0, t0 + n): per-step changes -> counts (after a sweep)
 cudaError_t zone_scan(unsigned long long *Zc, int64_t t0, int n, int Z, cudaStream_t s);
 cudaError_t sweep_set_smem_limits();
+
+// Ion-list tile (kmc_ions.cu).
+cudaError_t ion_set_smem_limits();
+// gate (may be null): a device flag; with a nonzero one the launch does nothing
+cudaError_t ion_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s);
+// The tile for a device: rails (of all devices that share its launches), sites,
+// electrodes, ions in all of the device's n_rails and at most n_max on a rail,
+// accept path.
+TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max, bool acc);
+// filling of the sites up to which the ion lists are the better tile
+float tile_max_fill(bool acc);
+// sets a.rcap and a.iy for the tile; shared memory of a CTA of `warps` warps
+size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool persite, int warps, bool acc);
+// the batch's kernels of ion-list kinds
+cudaError_t ion_batch_launch(const BatchArgs &b, int kind, int grid, int warps, size_t smem, bool acc,
+                             cudaStream_t s);
+int ion_batch_ctas_per_sm(int kind, bool acc, int warps, size_t smem);
+
 // gradient passes of a batch: one persistent launch per shape over its
 // (device, tile) items, whose per-device arguments (b.inst) are gradient-pass
 // arguments
@@ -190,8 +238,10 @@ cudaError_t setup_p0_table(const kmc_params &p, const double *Ea, double *P0, in
 cudaError_t setup_p0_bounds(const double *P0, int32_t R, int32_t L, int32_t Z, const DevConst *K,
                             float2 *out, cudaStream_t s);
 cudaError_t setup_p0_float(const double *P0, int64_t n, float *out, cudaStream_t s);
+// ions of each rail; with stats, also their total (stats[0]) and the largest (stats[1])
 cudaError_t setup_row_counts(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
-                             int32_t *N0, unsigned long long *bad, cudaStream_t s);
+                             int32_t *N0, unsigned long long *bad, unsigned long long *stats,
+                             cudaStream_t s);
 // bgd[r][z] = (N0[r] w_z / L in the oracle's FP64 order, D'_z): the background
 // of zone z of rail r and its part of Q_z - Qbar (S2.1.8 reading)
 cudaError_t setup_background(const int32_t *N0, int32_t R, int32_t L, int32_t Z, const DevConst *K,

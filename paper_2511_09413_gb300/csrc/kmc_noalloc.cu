@@ -70,6 +70,7 @@ int scratch_for_current_device(unsigned char **out)
         e = cudaGetSymbolAddress(&ptr, g_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(scratch)");
         e = sweep_set_smem_limits();
+        if (e == cudaSuccess) e = ion_set_smem_limits();
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         g_scratch_addr[dev] = ptr;
     }
@@ -81,10 +82,28 @@ bool finite_pos(double x) { return isfinite(x) && x > 0.0; }
 
 // Writes the launch arguments into the scratch array from the kernel's own
 // parameter space, so that no host buffer has to outlive the call (a copy
-// from host memory would read the caller's stack frame when it executes).
-__global__ void store_args_kernel(const SweepArgs a, SweepArgs *dst)
+// from host memory would read the caller's stack frame when it executes), and
+// chooses the tile: the filling is known only on the device, so both tiles are
+// launched and *words tells which of the two has the device (1: the occupancy
+// words, when more than max_fill of the sites of 32 rails spread over it are
+// occupied; an empty launch costs about 2 us).  One block of 1,024 threads, a
+// warp per sampled rail.  The choice changes no result.
+__global__ void __launch_bounds__(1024) store_args_kernel(const SweepArgs a, SweepArgs *dst, float max_fill,
+                                                          int *words)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *dst = a;
+    __shared__ int ions;
+    if (threadIdx.x == 0) {
+        *dst = a;
+        ions = 0;
+    }
+    __syncthreads();
+    const int64_t r = (int64_t)(threadIdx.x >> 5) * a.R / 32;
+    int n = 0;
+    for (int k = (int)(threadIdx.x & 31u); k < a.L; k += 32) n += a.occ[r * a.stride + k];
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31u) == 0u) atomicAdd(&ions, n);
+    __syncthreads();
+    if (threadIdx.x == 0) *words = (float)ions > max_fill * 32.0f * (float)a.L ? 1 : 0;
 }
 
 }  // namespace
@@ -155,7 +174,7 @@ extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t 
     if ((e = setup_constants(*p, K, s)) != cudaSuccess) return cuda_fail(e, "constants launch");
     const int32_t *N0 = N0_dev_or_null;
     if (!N0) {
-        if ((e = setup_row_counts(occ_dev, row_stride, R, L, N0s, misc + 5, s)) != cudaSuccess)
+        if ((e = setup_row_counts(occ_dev, row_stride, R, L, N0s, misc + 5, nullptr, s)) != cudaSuccess)
             return cuda_fail(e, "row counts launch");
         N0 = N0s;
     }
@@ -216,36 +235,46 @@ extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t 
     a.E_inf = (float)E_in;
     a.E_outf = (float)E_out;
 
-    // ---- launch shape: as many warps per CTA (up to 8) as shared memory allows
-    SweepLaunch l{};
-    l.lpr = sweep_pick_lpr(L, &l.wpl);
+    // ---- launch shapes: as many warps per CTA (up to 8) as shared memory allows
     int dev = 0, max_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (max_smem <= 0) max_smem = 48 * 1024;
     max_smem = std::min(max_smem, 200 * 1024);
-    int warps = 8, flush = 256;
-    l.acc = P0 >= kAcceptAutoP0 ? 1 : 0;
-    const bool acc = l.acc != 0;
-    while (warps > 1 &&
-           sweep_smem_bytes(l.lpr, l.wpl, Z, L, warps, flush, acc) > (size_t)max_smem)
-        warps >>= 1;
-    while (flush > 1 &&
-           sweep_smem_bytes(l.lpr, l.wpl, Z, L, warps, flush, acc) > (size_t)max_smem)
-        flush >>= 1;
-    l.warps = warps;
-    l.smem = sweep_smem_bytes(l.lpr, l.wpl, Z, L, warps, flush, acc);
-    const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * warps;
-    l.grid = (int)((R + rails_per_cta - 1) / rails_per_cta);
-    a.flush = flush;
+    const bool acc = P0 >= kAcceptAutoP0;
+    a.flush = 256;
+    auto shape = [&](const TileShape &t) {
+        SweepLaunch l{};
+        l.ions = t.ions;
+        l.kind = t.kind;
+        l.lpr = t.lpr;
+        l.wpl = t.wpl;
+        l.acc = acc ? 1 : 0;
+        l.warps = 8;
+        while (l.warps > 1 && tile_args(a, t, *p, false, l.warps, acc) > (size_t)max_smem) l.warps >>= 1;
+        l.smem = tile_args(a, t, *p, false, l.warps, acc);
+        const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * l.warps;
+        l.grid = (int)((R + rails_per_cta - 1) / rails_per_cta);
+        return l;
+    };
+    // a quarter of the sites full, but room for any number of ions
+    const TileShape lists = pick_tile(R, R, L, p->electrodes == 1, (int64_t)R * L / 4, L, acc);
+    const SweepLaunch li = shape(lists);
+    TileShape wt{};
+    wt.lpr = sweep_pick_lpr(L, &wt.wpl);
+    wt.kind = sweep_kind(wt.lpr, wt.wpl);
+    const SweepLaunch lw = shape(wt);
+    int *gate = (int *)(misc + 7);
 
-    store_args_kernel<<<1, 32, 0, s>>>(a, args_dev);
+    store_args_kernel<<<1, 1024, 0, s>>>(a, args_dev, tile_max_fill(acc), gate);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "argument store launch");
     int64_t left = n_steps;
     while (left > 0) {
         const int64_t n = std::min<int64_t>(left, 1 << 30);
         a.n_steps = (int32_t)n;
-        if ((e = sweep_launch(a, l, s)) != cudaSuccess) return cuda_fail(e, "sweep launch");
+        if (li.ions && (e = ion_launch(a, li, gate, s)) != cudaSuccess) return cuda_fail(e, "sweep launch");
+        if ((e = sweep_launch(a, lw, li.ions ? gate : nullptr, s)) != cudaSuccess)
+            return cuda_fail(e, "sweep launch");
         if ((e = zone_scan(a.Zc, a.t0, (int)n, Z, s)) != cudaSuccess)
             return cuda_fail(e, "zone-count scan launch");
         a.t0 += n;

@@ -123,7 +123,7 @@ __global__ void p0_float_kernel(const double *P0, int64_t n, float *out)
 
 // One warp per rail: ion count, and a count of bytes that are not 0 or 1.
 __global__ void row_counts_kernel(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
-                                  int32_t *N0, unsigned long long *bad)
+                                  int32_t *N0, unsigned long long *bad, unsigned long long *stats)
 {
     const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -138,6 +138,10 @@ __global__ void row_counts_kernel(const uint8_t *occ, int64_t stride, int32_t R,
     b = __reduce_add_sync(0xffffffffu, b);
     if (lane == 0) {
         N0[r] = c;
+        if (stats) {
+            atomicAdd(stats, (unsigned long long)c);
+            atomicMax(stats + 1, (unsigned long long)c);
+        }
         if (b) atomicAdd(bad, (unsigned long long)b);
     }
 }
@@ -266,11 +270,12 @@ cudaError_t setup_background(const int32_t *N0, int32_t R, int32_t L, int32_t Z,
 }
 
 cudaError_t setup_row_counts(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
-                             int32_t *N0, unsigned long long *bad, cudaStream_t s)
+                             int32_t *N0, unsigned long long *bad, unsigned long long *stats,
+                             cudaStream_t s)
 {
     const int warps = 8;
     row_counts_kernel<<<(unsigned)((R + warps - 1) / warps), warps * 32, 0, s>>>(occ, stride, R, L,
-                                                                                N0, bad);
+                                                                                N0, bad, stats);
     return cudaGetLastError();
 }
 

@@ -35,63 +35,19 @@
 #include <stdint.h>
 #include <type_traits>
 
+#include "kmc_device.cuh"
 #include "kmc_internal.h"
 
 namespace kmc {
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
 constexpr int kDeferCap = 64;           // deferred (exact-path) candidates per warp and step
 // Philox blocks in flight per lane per iteration of the draw loop.  One is
 // fastest on both loops: the kernel gains more from resident warps than from
 // ILP (the accept-table loop at 4 CTAs per SM, the reject-only loop at 5).
 constexpr int kDrawIlpAcc = 1;
 constexpr int kDrawIlpReject = 1;
-
-// Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): per round two 32x32->64
-// multiplies; the high halves are xor-ed with the other counter words and the
-// round key.  The ten round keys are precomputed on the host.
-__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                        const uint32_t *rk0, const uint32_t *rk1)
-{
-#pragma unroll
-    for (int i = 0; i < 10; ++i) {
-        // one widening multiply per product (both halves at once): 1 % faster
-        // in the sweep and 2.5 % in the Philox-only probe than separate
-        // low and high multiplies
-        uint64_t p0, p1;
-        asm("mul.wide.u32 %0, %1, %2;" : "=l"(p0) : "r"(c0), "r"(0xD2511F53u));
-        asm("mul.wide.u32 %0, %1, %2;" : "=l"(p1) : "r"(c2), "r"(0xCD9E8D57u));
-        const uint32_t lo0 = (uint32_t)p0, hi0 = (uint32_t)(p0 >> 32);
-        const uint32_t lo1 = (uint32_t)p1, hi1 = (uint32_t)(p1 >> 32);
-        c0 = hi1 ^ c1 ^ rk0[i];
-        c1 = lo1;
-        c2 = hi0 ^ c3 ^ rk1[i];
-        c3 = lo0;
-    }
-    return make_uint4(c0, c1, c2, c3);
-}
-
-// 16 occupancy bytes (values 0/1) -> 16 bits; byte i -> bit i.
-__device__ __forceinline__ uint32_t pack4(uint32_t v)
-{
-    return (((v & 0x01010101u) * 0x00204081u) >> 21) & 0xFu;
-}
-__device__ __forceinline__ uint32_t pack16(uint4 q)
-{
-    return pack4(q.x) | (pack4(q.y) << 4) | (pack4(q.z) << 8) | (pack4(q.w) << 12);
-}
-// 4 bits -> 4 bytes of 0/1
-__device__ __forceinline__ uint32_t unpack4(uint32_t n)
-{
-    return (n * 0x00204081u) & 0x01010101u;
-}
-__device__ __forceinline__ uint4 unpack16(uint32_t b)
-{
-    return make_uint4(unpack4(b & 0xF), unpack4((b >> 4) & 0xF), unpack4((b >> 8) & 0xF),
-                      unpack4((b >> 12) & 0xF));
-}
 
 // Site masks of the 32-site word starting at site s0 of an L-site rail: the
 // sites that exist, site 0, site L-1.  Recomputed where needed rather than
@@ -106,24 +62,10 @@ __device__ __forceinline__ uint32_t last_mask(int s0, int L)
     return (L - 1 >= s0 && L - 1 < s0 + 32) ? (1u << (L - 1 - s0)) : 0u;
 }
 
-// Conservative integer thresholds on the high 32 bits h of a 64-bit draw w
-// (u = (w >> 11) 2^-53):  h < acc_thr(p_lo) implies u <= p;  h > rej_thr(p_hi)
-// implies u > p, for any p in [p_lo, p_hi].
-__device__ __forceinline__ uint32_t acc_thr(float p_lo)
-{
-    const uint32_t f = __float2uint_rd(p_lo * 4294967296.0f);
-    return f > 0u ? f - 1u : 0u;
-}
-__device__ __forceinline__ uint32_t rej_thr(float p_hi)
-{
-    return __float2uint_ru(p_hi * 4294967296.0f);
-}
-
 // ---------------------------------------------------------------- shared memory
 // One warp's block: a fixed part whose offsets are compile-time constants and a
 // part that scales with G * Z (offsets from one runtime stride), so that the
 // kernel keeps only a base address and that stride in registers.
-__host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 template <int LPR, int WPL>
 struct Layout {
@@ -236,62 +178,6 @@ struct WarpSmem {
     __device__ int32_t *gPb() const { return (int32_t *)(gbase() + 10 * gzq + align16(128 * Ly::G)); }
 };
 
-// --------------------------------------------------------- exact FP64 path
-// Exact FP64 zone quantities (B_z, 1/(1+B_z)) for zone zt of one rail, with
-// the operation order of the oracle: excess C_z, enclosed charge Q_z, mean
-// Qbar, dV_z (S2.1.8), dE_z (Eq. 3), B_z (Eq. 4).  Every operation is an
-// explicitly rounded intrinsic so that no contraction changes the result.
-__device__ __forceinline__ void exact_zone(const int32_t *Pb, const DevConst *Kp, int Z, int L,
-                                        int32_t n0, const double2 *bgd, double V, int zt, double *B,
-                                        double *inv)
-{
-    const DevConst &K = *Kp;
-    const double Ld = (double)L;
-    double run = 0.0, acc = 0.0, Qt = 0.0;
-    for (int z = 0; z < Z; ++z) {
-        const int w = K.bnd[z + 1] - K.bnd[z];
-        const int Nz = Pb[z + 1] - Pb[z];
-        // background N0 w_z / L: the rail's precomputed row when there is one
-        const double bz = bgd ? bgd[z].x : __ddiv_rn(__dmul_rn((double)n0, (double)w), Ld);
-        const double C = __dsub_rn((double)Nz, bz);
-        const double Q = __dadd_rn(run, __dmul_rn(0.5, C));
-        run = __dadd_rn(run, C);
-        acc = __dadd_rn(acc, __dmul_rn((double)w, Q));
-        if (z == zt) Qt = Q;
-    }
-    const double Qbar = __ddiv_rn(acc, Ld);
-    const double dV = __dsub_rn(V, __dmul_rn(K.ka, __dsub_rn(Qt, Qbar)));
-    const double dE = __ddiv_rn(__dmul_rn(dV, K.d), K.t_dev);
-    const double b = exp(__ddiv_rn(-dE, K.kT));
-    *B = b;
-    *inv = __ddiv_rn(1.0, __dadd_rn(1.0, b));
-}
-
-// Exact decision u <= p for the 64-bit word w, with near-threshold logging.
-__device__ __forceinline__ bool exact_trial(uint64_t w, double p, kmc_log_entry *log,
-                                         unsigned long long *log_count, int64_t log_cap,
-                                         int32_t rail, uint32_t step, int32_t site, int32_t dir,
-                                         int32_t kind)
-{
-    const double u = __dmul_rn((double)(w >> 11), 0x1.0p-53);
-    const double diff = __dsub_rn(u, p);
-    if (fabs(diff) < 1e-12) {
-        const unsigned long long slot = atomicAdd(log_count, 1ull);
-        if ((int64_t)slot < log_cap) {
-            kmc_log_entry e;
-            e.rail = rail;
-            e.step = step;
-            e.site = site;
-            e.dir = dir;
-            e.kind = kind;
-            e.pad = 0;
-            e.diff = diff;
-            log[slot] = e;
-        }
-    }
-    return u <= p;
-}
-
 // ------------------------------------------------------------ one decision
 // Bounded decision of one candidate from the step-start state kept in shared
 // memory: dR, dL in {0 reject (or direction blocked), 1 accept, 2 undecided},
@@ -304,12 +190,6 @@ struct Decision {
     int idx;
     uint32_t bit;
 };
-
-// Band factors: p_lo = p flo, p_hi = p fhi bracket the exact p.
-__device__ __forceinline__ int bounded(uint32_t h, float p, float flo, float fhi)
-{
-    return h < acc_thr(p * flo) ? 1 : (h > rej_thr(p * fhi) ? 0 : 2);
-}
 
 template <int LPR, int WPL>
 __device__ __forceinline__ Decision decide(const WarpSmem<LPR, WPL> &S, const SweepArgs *g,
@@ -1457,9 +1337,10 @@ template <int LPR, int WPL, bool ACC>
 // any one pipe, and the extra resident warps outweigh the spills (mostly on
 // the slow and exact paths) that the caps cause.  With 80 registers and 3 CTAs
 // the hysteresis device runs 4.5 % slower.
-__global__ void __launch_bounds__(256, ACC ? 4 : 5) sweep_kernel(const SweepArgs a)
+__global__ void __launch_bounds__(256, ACC ? 4 : 5) sweep_kernel(const SweepArgs a, const int *gate)
 {
     extern __shared__ __align__(16) uint8_t smem[];
+    if (gate && *gate == 0) return;     // the ion-list tile advances this device
     const int64_t tile_rail0 = (int64_t)blockIdx.x * (blockDim.x >> 5) * (32 / LPR);
     sweep_tile<LPR, WPL, ACC>(a, a.rk0, a.rk1, a.t0, a.n_steps, a.flush, tile_rail0, smem);
 }
@@ -1670,10 +1551,10 @@ __global__ void batch_advance_kernel(int64_t *t0, unsigned *work, int n_steps)
 }
 
 template <int LPR, int WPL>
-cudaError_t launch_t(const SweepArgs &a, const SweepLaunch &l, cudaStream_t s)
+cudaError_t launch_t(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s)
 {
-    if (l.acc) sweep_kernel<LPR, WPL, true><<<l.grid, l.warps * 32, l.smem, s>>>(a);
-    else sweep_kernel<LPR, WPL, false><<<l.grid, l.warps * 32, l.smem, s>>>(a);
+    if (l.acc) sweep_kernel<LPR, WPL, true><<<l.grid, l.warps * 32, l.smem, s>>>(a, gate);
+    else sweep_kernel<LPR, WPL, false><<<l.grid, l.warps * 32, l.smem, s>>>(a, gate);
     return cudaGetLastError();
 }
 
@@ -1783,7 +1664,7 @@ cudaError_t with_shape(int k, F &&f)
 
 cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, int warps, cudaStream_t s)
 {
-    for (int k = 0; k < kShapeKinds; ++k) {
+    for (int k = 0; k < kWordKinds; ++k) {
         if (plan.grid[k] <= 0) continue;
         const cudaError_t e = with_shape(k, [&](auto lpr, auto wpl) {
             constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
@@ -1797,6 +1678,7 @@ cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, int war
 
 int batch_ctas_per_sm(int kind, int mode, int warps, size_t smem)
 {
+    if (kind >= kWordKinds) return ion_batch_ctas_per_sm(kind, mode == 1, warps, smem);
     int n = 0;
     const cudaError_t e = with_shape(kind, [&](auto lpr, auto wpl) {
         constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
@@ -1858,7 +1740,7 @@ int sweep_kind(int lpr, int wpl)
 
 cudaError_t batch_set_smem_limit()
 {
-    for (int k = 0; k < kShapeKinds; ++k) {
+    for (int k = 0; k < kWordKinds; ++k) {
         const cudaError_t e = with_shape(k, [](auto lpr, auto wpl) {
             constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
             const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -1878,7 +1760,9 @@ cudaError_t batch_launch(const BatchArgs &b, const BatchPlan &plan, int warps, b
     cudaError_t e;
     for (int k = 0; k < kShapeKinds; ++k) {
         if (plan.grid[k] <= 0) continue;
-        e = with_shape(k, [&](auto lpr, auto wpl) {
+        if (k >= kWordKinds) e = ion_batch_launch(b, k, plan.grid[k], warps, plan.smem[k], acc, s);
+        else
+            e = with_shape(k, [&](auto lpr, auto wpl) {
             constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
             if (acc) sweep_batch_kernel<true, P, Q><<<plan.grid[k], warps * 32, plan.smem[k], s>>>(b);
             else sweep_batch_kernel<false, P, Q><<<plan.grid[k], warps * 32, plan.smem[k], s>>>(b);
@@ -1899,16 +1783,16 @@ cudaError_t zone_scan(unsigned long long *Zc, int64_t t0, int n, int Z, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t sweep_launch(const SweepArgs &a, const SweepLaunch &l, cudaStream_t s)
+cudaError_t sweep_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s)
 {
-    if (l.wpl == 2) return launch_t<32, 2>(a, l, s);
+    if (l.wpl == 2) return launch_t<32, 2>(a, l, gate, s);
     switch (l.lpr) {
-    case 1: return launch_t<1, 1>(a, l, s);
-    case 2: return launch_t<2, 1>(a, l, s);
-    case 4: return launch_t<4, 1>(a, l, s);
-    case 8: return launch_t<8, 1>(a, l, s);
-    case 16: return launch_t<16, 1>(a, l, s);
-    default: return launch_t<32, 1>(a, l, s);
+    case 1: return launch_t<1, 1>(a, l, gate, s);
+    case 2: return launch_t<2, 1>(a, l, gate, s);
+    case 4: return launch_t<4, 1>(a, l, gate, s);
+    case 8: return launch_t<8, 1>(a, l, gate, s);
+    case 16: return launch_t<16, 1>(a, l, gate, s);
+    default: return launch_t<32, 1>(a, l, gate, s);
     }
 }
 

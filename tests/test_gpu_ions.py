@@ -1,0 +1,94 @@
+"""The ion-list tile (kmc_ions.cu) against the oracle, bit for bit, at the sizes
+where its shapes change: lanes per rail follow from the number of rails and of
+ions, 32 rows of bits end at 32 entries a lane, and open rails grow, shrink and
+have their entries dealt out again."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kmc():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_09413_gb300 import build, kmc as K
+    build.build()
+    K.load()
+    torch.cuda.init()
+    return K
+
+
+def _dev(**kw):
+    d = dict(R=48, L=100, Z=10, electrodes=0, d=1.0, dt=5e-7, T=300.0, Ea=0.40, nu=1e12,
+             alpha=0.2, kappa=1.0, k_e=0.0, rho_e=0.0, seed=33, instance=2)
+    d.update(kw)
+    return d
+
+
+def _check(K, dev, V, fill, chunks):
+    occ0 = oracle.init_occupancy(dev, 1, fill=fill)
+    sim = K.Sim(dev, V, 2, occ0=occ0)
+    orc = oracle.OracleSim(dev, V, occ0, None)
+    for c in chunks:
+        sim.step_n(c)
+    n = sum(chunks)
+    Jo, Zo = orc.step_n(n)
+    Jg, Zg = sim.traces()
+    assert np.array_equal(Zg, Zo), "zone-count traces differ"
+    assert np.array_equal(Jg, Jo), "current traces differ"
+    assert np.array_equal(sim.occupancy(), orc.occ), "occupancy differs"
+    assert np.array_equal(sim.rail_current(), orc.J_rail), "per-rail current differs"
+    sim.close()
+
+
+# (rails, sites): 4, 8, 16 and 32 lanes per rail, each at the last number of
+# sites whose full rails fit 32 rows and one beyond, the fewest sites, and 64 rows
+@pytest.mark.parametrize("R,L", [(49153, 8), (19201, 128), (19201, 129), (24001, 256), (24001, 257),
+                                 (12289, 512), (12289, 513), (300, 1024), (300, 1025), (64, 2048)])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_shapes_of_the_lists(kmc, R, L, electrodes, dt):
+    Z = min(L, 10 if R % 2 else 32)
+    k = 1.0 / dt if electrodes else 0.0
+    dev = _dev(R=R, L=L, Z=Z, electrodes=electrodes, k_e=k, rho_e=0.3, dt=dt)
+    n = 7 if R * L > 1000000 else 40
+    V = np.where(np.arange(n) % 6 < 3, 1.0, -0.5)
+    _check(kmc, dev, V, 0.25, [n // 3, n - n // 3])
+
+
+# open rails that fill up from empty, drain from half full, and swap their ions
+# at a high rate: entries come and go at both ends
+@pytest.mark.parametrize("L", [8, 33, 64, 200])
+@pytest.mark.parametrize("fill,rho", [(0.0, 0.95), (0.4, 0.0), (0.3, 0.5)])
+@pytest.mark.parametrize("rule", [0, 1])
+def test_open_rails_grow_and_shrink(kmc, L, fill, rho, rule):
+    dev = _dev(R=70, L=L, Z=min(L, 7), electrodes=1, k_e=4e6, rho_e=rho, dt=2e-6, rule=rule)
+    V = 2.0 * np.sin(np.arange(500) / 40.0)
+    _check(kmc, dev, V, fill, [500])
+
+
+# a batch chooses its tiles from all rails together: the same devices alone
+# and together give the same results, lists and words side by side
+def test_batch_of_lists_and_words(kmc):
+    devs, fills = [], []
+    for i, (R, L, f, e) in enumerate([(30000, 40, 0.2, 0), (20000, 130, 0.3, 1), (9000, 300, 0.25, 0),
+                                      (500, 1500, 0.2, 1), (3000, 100, 0.9, 0), (4000, 4, 0.4, 0),
+                                      (200, 900, 0.1, 0)]):
+        devs.append(_dev(R=R, L=L, Z=min(L, 10), electrodes=e, k_e=1e6 if e else 0.0, rho_e=f, instance=i))
+        fills.append(f)
+    V = np.where(np.arange(48) % 20 < 9, 0.8, 0.0)
+    b = kmc.Batch(devs, [V] * len(devs), [1] * len(devs), fills=fills)
+    b.set_launch(8, 16)
+    b.step_n(40)
+    for i, (d, f) in enumerate(zip(devs, fills)):
+        s = kmc.Sim(d, V, 1, fill=f)
+        s.step_n(40)
+        for x, y in zip((*b.traces(i), b.occupancy(i), b.rail_current(i)),
+                        (*s.traces(), s.occupancy(), s.rail_current())):
+            assert np.array_equal(x, y)
+        s.close()
+    b.close()
