@@ -75,16 +75,16 @@ void drop_graph(kmc_batch *b)
 // Work list for a CTA size: one item per tile of 32/LPR * warps rails, larger
 // tiles (longer rails) first so that the dynamic schedule ends evenly.
 // Work items of a list of devices: every device's rails cut into tiles of
-// (32 / its shape's lanes per rail) x warps rails, grouped by kernel shape and, within a
+// (32 / its shape's lanes per rail) x (its launch's warps) rails, grouped by kernel shape and, within a
 // shape, longest tiles first.  Returns the items and the shape offsets.
 void make_items(const std::vector<const kmc_params *> &devs, const std::vector<TileShape> &shapes,
-                const std::vector<int> &inst, int warps, std::vector<BatchItem> &sorted, int *cls_off)
+                const std::vector<int> &inst, const int *warps, std::vector<BatchItem> &sorted, int *cls_off)
 {
     std::vector<BatchItem> items;
     std::vector<int64_t> cost;
     for (size_t i = 0; i < devs.size(); ++i) {
         const kmc_params &p = *devs[i];
-        const int64_t tile = (int64_t)(32 / shapes[i].lpr) * warps;
+        const int64_t tile = (int64_t)(32 / shapes[i].lpr) * warps[shapes[i].kind];
         for (int64_t r0 = 0; r0 < p.n_rails; r0 += tile) {
             BatchItem it;
             it.inst = inst[i];
@@ -153,7 +153,8 @@ int build_items(kmc_batch *b, int warps)
             return fail(KMC_E_ARG, "batch: shared memory for this CTA size exceeds the device limit");
     std::vector<BatchItem> sorted;
     int cls_off[kShapeKinds + 1];
-    make_items(devs, shapes, inst, warps, sorted, cls_off);
+    for (int k = 0; k < kShapeKinds; ++k) plan.warps[k] = warps;
+    make_items(devs, shapes, inst, plan.warps, sorted, cls_off);
     BCK(cudaMemcpyAsync(b->inst, host.data(), sizeof(SweepArgs) * host.size(), cudaMemcpyHostToDevice, b->user),
         "copy device arguments");
     if (b->items) cudaFreeAsync(b->items, b->user);
@@ -515,46 +516,45 @@ int kmc_batch_grad_all(kmc_batch *b, const double *const *dLoss_dJ, const double
         ++n_active;
     }
     if (n_active > 0) {
-        // CTA size: 8 warps unless some device's tile needs less shared memory
-        int warps = 8;
-        auto smem_for = [&](int w) {
-            size_t m = 0;
-            for (int i = 0; i < n_inst; ++i)
-                if (active[(size_t)i]) {
-                    const kmc_params &p = b->dev[(size_t)i]->p;
-                    int wpl = 1;
-                    const int lpr = sweep_pick_lpr(p.n_sites, &wpl);
-                    m = std::max(m, grad_smem_bytes(lpr, wpl, p.n_zones, p.n_sites, w));
-                }
-            return m;
-        };
-        while (warps > 1 && smem_for(warps) > (size_t)max_smem) warps >>= 1;
-        if (smem_for(warps) > (size_t)max_smem)
-            return fail(KMC_E_ARG, "batched gradient pass: shared memory exceeds the device limit");
-        // work items grouped by shape, longest tiles first in each; one
-        // persistent launch per shape, its shared memory the largest tile's
+        // every device's tile, and of every shape the CTA size and shared memory
         std::vector<const kmc_params *> devs;
         std::vector<TileShape> shapes;
         std::vector<int> inst;
-        BatchPlan plan{};
+        int64_t rails = 0;
+        for (int i = 0; i < n_inst; ++i)
+            if (active[(size_t)i]) rails += b->dev[(size_t)i]->p.n_rails;
         for (int i = 0; i < n_inst; ++i) {
             if (!active[(size_t)i]) continue;
-            const kmc_params &p = b->dev[(size_t)i]->p;
-            TileShape t{};
-            t.lpr = sweep_pick_lpr(p.n_sites, &t.wpl);
-            t.kind = sweep_kind(t.lpr, t.wpl);
-            plan.smem[t.kind] = std::max(plan.smem[t.kind],
-                                         grad_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps));
-            devs.push_back(&p);
-            shapes.push_back(t);
+            const kmc_handle *h = b->dev[(size_t)i];
+            devs.push_back(&h->p);
+            shapes.push_back(pick_grad_tile(rails, h->p.n_rails, h->p.n_sites, h->p.electrodes == 1, h->n_tot,
+                                            h->n_max));
             inst.push_back(i);
         }
+        BatchPlan plan{};
+        for (int k = 0; k < kShapeKinds; ++k) plan.warps[k] = k < kWordKinds ? 8 : 16;
+        for (size_t i = 0; i < devs.size(); ++i) {
+            size_t most = 0, total = 0;
+            grad_smem_limits(&most, &total, shapes[i].ions != 0);
+            plan.warps[shapes[i].kind] = std::min(plan.warps[shapes[i].kind],
+                                                  grad_warps(shapes[i], *devs[i], most - 1024, total, rails, sms));
+        }
+        for (size_t i = 0; i < devs.size(); ++i) {
+            const int k = shapes[i].kind;
+            size_t most = 0, total = 0;
+            grad_smem_limits(&most, &total, shapes[i].ions != 0);
+            plan.smem[k] = std::max(plan.smem[k], grad_tile_args(gargs[(size_t)inst[i]], shapes[i], *devs[i], plan.warps[k]));
+            if (plan.smem[k] > most)
+                return fail(KMC_E_ARG, "batched gradient pass: shared memory exceeds the device limit");
+        }
+        // work items grouped by shape, longest tiles first in each; one
+        // persistent launch per shape, its shared memory the largest tile's
         std::vector<BatchItem> sorted;
         int cls_off[kShapeKinds + 1];
-        make_items(devs, shapes, inst, warps, sorted, cls_off);
-        for (int k = 0; k < kWordKinds; ++k) {
+        make_items(devs, shapes, inst, plan.warps, sorted, cls_off);
+        for (int k = 0; k < kShapeKinds; ++k) {
             const int n = cls_off[k + 1] - cls_off[k];
-            plan.grid[k] = n > 0 ? std::min(n, sms * batch_ctas_per_sm(k, 2, warps, plan.smem[k])) : 0;
+            plan.grid[k] = n > 0 ? std::min(n, sms * batch_ctas_per_sm(k, 2, plan.warps[k], plan.smem[k])) : 0;
         }
         SweepArgs *ginst = nullptr;
         BatchItem *gitems = nullptr;
@@ -574,7 +574,7 @@ int kmc_batch_grad_all(kmc_batch *b, const double *const *dLoss_dJ, const double
             (e = cudaMemcpyAsync(gitems, sorted.data(), sizeof(BatchItem) * sorted.size(),
                                  cudaMemcpyHostToDevice, b->user)) == cudaSuccess &&
             (e = cudaMemsetAsync(b->work_ctr, 0, sizeof(unsigned) * kShapeKinds, b->user)) == cudaSuccess &&
-            (e = batch_grad_launch(a, plan, warps, b->user)) == cudaSuccess)
+            (e = batch_grad_launch(a, plan, b->user)) == cudaSuccess)
             // re-arm for the forward
             e = cudaMemsetAsync(b->work_ctr, 0, sizeof(unsigned) * kShapeKinds, b->user);
         cudaFreeAsync(gitems, b->user);

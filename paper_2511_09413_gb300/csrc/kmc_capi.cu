@@ -390,7 +390,10 @@ int kmc::grad_prepare(kmc_handle *h, const double *dLoss_dJ, const double *dLoss
         h->g_out = (double *)h->alloc(sizeof(double) * 8);
         h->g_misc = (unsigned long long *)h->alloc(sizeof(unsigned long long) * 8);
         h->g_args_dev = (SweepArgs *)h->alloc(sizeof(SweepArgs));
-        if (!h->g_occ || !h->g_state || !h->g_wJ || !h->g_fJab || !h->g_fZa || !h->g_fZb || !h->g_fZr ||
+        h->g_bgN = (double2 *)h->alloc(sizeof(double2) * (size_t)((L + 1) * Z));
+        if (h->g_bgN)
+            CK(setup_background_by_count((int32_t)L, (int32_t)Z, h->K, h->g_bgN, s), "backgrounds");
+        if (!h->g_bgN || !h->g_occ || !h->g_state || !h->g_wJ || !h->g_fJab || !h->g_fZa || !h->g_fZb || !h->g_fZr ||
             !h->g_out || !h->g_misc || !h->g_args_dev)
             return fail(KMC_E_NOMEM, "device allocation failed (gradient pass)");
     }
@@ -479,6 +482,7 @@ int kmc::grad_prepare(kmc_handle *h, const double *dLoss_dJ, const double *dLoss
     ga.fZb = dLoss_dZc ? h->g_fZb : nullptr;
     ga.fZr = dLoss_dZc ? h->g_fZr : nullptr;
     ga.gstate = h->g_state;
+    ga.bgN = h->g_bgN;
     ga.alpha = p.alpha_V;
     const double kT = 8.6173e-5 * p.T_K;
     ga.tdev_kT = ((double)L * p.site_spacing_nm) * kT;
@@ -741,23 +745,23 @@ int kmc_grad(kmc_handle *h, const double *dLoss_dJ, const double *dLoss_dZc, dou
         SweepArgs ga;
         int rc = grad_prepare(h, dLoss_dJ, dLoss_dZc, &ga);
         if (rc) return rc;
+        const TileShape ts = pick_grad_tile(R, R, (int)L, p.electrodes == 1, h->n_tot, h->n_max);
         SweepLaunch l{};
-        l.lpr = sweep_pick_lpr((int)L, &l.wpl);
-        int dev = 0, max_smem = 0;
+        l.kind = ts.kind;
+        l.lpr = ts.lpr;
+        l.wpl = ts.wpl;
+        size_t most = 0, total = 0;
+        grad_smem_limits(&most, &total, ts.ions != 0);
+        int dev = 0, sms = 0;
         cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (max_smem <= 0) max_smem = 48 * 1024;
-        max_smem = std::min(max_smem, 200 * 1024);
-        int warps = 8;
-        while (warps > 1 && grad_smem_bytes(l.lpr, l.wpl, (int)Z, (int)L, warps) > (size_t)max_smem)
-            warps >>= 1;
-        if (grad_smem_bytes(l.lpr, l.wpl, (int)Z, (int)L, warps) > (size_t)max_smem)
-            return fail(KMC_E_ARG, "gradient pass: shared memory exceeds the device limit");
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int warps = grad_warps(ts, p, most, total, R, sms);
+        l.smem = grad_tile_args(ga, ts, p, warps);
+        if (l.smem > most) return fail(KMC_E_ARG, "gradient pass: shared memory exceeds the device limit");
         l.warps = warps;
-        l.smem = grad_smem_bytes(l.lpr, l.wpl, (int)Z, (int)L, warps);
         const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * warps;
         l.grid = (int)((R + rails_per_cta - 1) / rails_per_cta);
-        CK(grad_launch(ga, l, s), "gradient pass launch");
+        CK(ts.ions ? ion_grad_launch(ga, l, s) : grad_launch(ga, l, s), "gradient pass launch");
         rc = grad_reduce_out(h, out);
         if (rc) return rc;
         CK(cudaStreamSynchronize(s), "gradient pass");

@@ -60,6 +60,7 @@ struct kmc_handle {
     kmc::SweepArgs *g_args_dev = nullptr;
     double *g_etab = nullptr;                 // exp tables of the zone sums (1024 + nH doubles)
     int32_t g_etM = -1;                       // their range, or -1 when not built
+    double2 *g_bgN = nullptr;                 // backgrounds by ion count
 
     kmc::SweepArgs args{};
     kmc::SweepLaunch launch{};

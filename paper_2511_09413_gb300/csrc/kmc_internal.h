@@ -41,6 +41,7 @@ struct IonLayout {
     uint32_t p0b;     // float2 [G][Z]: per-site P0 bounds of the zone (per-site barriers)
     uint32_t pb;      // int [G][Z + 1]: ions below each zone boundary
     uint32_t st;      // uint32 [slots][32]: each lane's state words
+    uint32_t g;       // gradient pass: its sums, counts and factors (IonView)
     uint32_t col;     // uint32 [rcap][32]: each lane's entries
     uint32_t bytes;   // one warp's block
 };
@@ -107,6 +108,9 @@ struct SweepArgs {
     const double *etH;                   // [2 etM / 1024 + 1]
     int32_t etM;
     int32_t et_pad;
+    // ion lists: background D'_z of a rail of n ions and exp(xV kappa alpha D'_z),
+    // xV V = ln B_z without space charge; [n_sites + 1][Z]
+    const double2 *bgN;
 };
 
 // Per-rail state of the gradient pass: cumulative inner-trial weight W (the
@@ -146,6 +150,7 @@ struct TileShape {
 // shape's persistent launch (grid 0: the batch has no items of that shape).
 struct BatchPlan {
     int grid[kShapeKinds];
+    int warps[kShapeKinds];
     size_t smem[kShapeKinds];
 };
 
@@ -205,12 +210,26 @@ size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool per
 // the batch's kernels of ion-list kinds
 cudaError_t ion_batch_launch(const BatchArgs &b, int kind, int grid, int warps, size_t smem, bool acc,
                              cudaStream_t s);
-int ion_batch_ctas_per_sm(int kind, bool acc, int warps, size_t smem);
+int ion_batch_ctas_per_sm(int kind, int mode, int warps, size_t smem);
+// the same for the gradient pass
+TileShape pick_grad_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max);
+// shared memory of a CTA at most, and of an SM, for the gradient pass
+void grad_smem_limits(size_t *most, size_t *total, bool ions);
+constexpr int kGradSmem = 226 * 1024;   // dynamic shared memory of a gradient CTA at most
+constexpr int kGradWarps = 20;          // warps of a gradient CTA at most (102 registers)
+cudaError_t ion_batch_set_smem_limits();
+cudaError_t ion_grad_set_smem_limits();
+int ion_grad_ctas_per_sm(int kind, int warps, size_t smem);
+int grad_warps(const TileShape &t, const kmc_params &p, size_t most, size_t total, int64_t rails, int sms);
+size_t grad_tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, int warps);
+cudaError_t ion_grad_launch(const SweepArgs &a, const SweepLaunch &l, cudaStream_t s);
+cudaError_t ion_batch_grad_launch(const BatchArgs &b, int kind, int grid, int warps, size_t smem,
+                                  cudaStream_t s);
 
 // gradient passes of a batch: one persistent launch per shape over its
 // (device, tile) items, whose per-device arguments (b.inst) are gradient-pass
 // arguments
-cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, int warps, cudaStream_t s);
+cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, cudaStream_t s);
 // resident CTAs per SM of a shape's batched kernel (mode 0 forward, 1 forward
 // with the accept path, 2 gradient pass) at this CTA size and shared memory
 int batch_ctas_per_sm(int kind, int mode, int warps, size_t smem);
@@ -253,6 +272,8 @@ cudaError_t setup_count_keys(const kmc_params &p, uint64_t key_bound, int mode, 
                              unsigned long long *count, cudaStream_t s);
 cudaError_t setup_mark_smallest(const kmc_params &p, uint64_t key_star, int64_t idx_star,
                                 int select_none, uint8_t *occ, int64_t stride, cudaStream_t s);
+// out[n][z] = (D'_z of a rail of n <= L ions, exp(xV kappa alpha D'_z))
+cudaError_t setup_background_by_count(int32_t L, int32_t Z, const DevConst *K, double2 *out, cudaStream_t s);
 // exp(cm (j 1024 - M)) for j < nH into etH and exp(cm i) for i < 1024 into etL
 cudaError_t setup_exp_tables(double cm, int32_t M, double *etL, double *etH, int32_t nH,
                              cudaStream_t s);

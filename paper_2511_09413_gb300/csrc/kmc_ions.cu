@@ -1,889 +1,16 @@
-// kmc_ions.cu -- the per-time-step sweep (arXiv 2511.09413, Supplementary
-// S2.1.2 - S2.1.7) over ordered ion lists, hand-written for sm_103a.
-//
-// The state of a rail is the list of its ions' sites.  Ions never pass one
-// another (S2.1.6), so the list stays ordered and an ion's neighbours are its
-// predecessor and successor: exclusion is a gap of one site, a conflict a gap
-// of two with both ions moving inward.  P lanes share a rail, 32 / P rails a
-// warp; a lane holds consecutive ions in a column of shared memory that only
-// it touches.  Against the occupancy words of kmc_sweep.cu nothing is rebuilt
-// when an ion moves (no popcount scan, free-neighbour masks or compaction of
-// candidates): every lane draws for its next ion in every iteration.  Ions
-// with both neighbours occupied draw in vain, so fuller rails stay with the
-// occupancy words (pick_tile).
-//
-//  * Zone sums.  The number of ions below each zone boundary, P_b, and
-//    F = sum_b P_b w_b are updated when an ion crosses a boundary, and the
-//    field of S2.1.8 and the decision bounds of Eqs. 3-6 are evaluated again
-//    only then (or when a voltage window starts).
-//  * Open electrodes.  The first entry of an open rail's list is at site 0 or,
-//    when that site is empty, at the virtual site -1; an injection is its hop
-//    to site 0 and an extraction the hop back, so the exchange (the most
-//    frequent event of an open rail) moves an entry like any other hop.  Site
-//    L - 1 mirrors this with the virtual site L.  The list grows or shrinks
-//    only when an ion hops between a boundary site and its inner neighbour.
-//  * Decisions are those of kmc_sweep.cu: integer bounds on the draw's high
-//    word that provably enclose the FP64 probability, an FP64 band for the
-//    draws between them and the exact evaluation for the last 1e-11.
+// kmc_ions.cu -- single-device launches of the ion-list tile (kmc_ions.cuh) and the
+// choice of a device's tile.
 #include <cuda_runtime.h>
-#include <math.h>
 #include <stdint.h>
+
 #include <algorithm>
 #include <type_traits>
 
-#include "kmc_device.cuh"
-#include "kmc_internal.h"
+#include "kmc_ions.cuh"
 
 namespace kmc {
 
 namespace {
-
-constexpr uint32_t kM0 = 0xD2511F53u, kM1 = 0xCD9E8D57u;   // Philox multipliers
-
-__device__ __forceinline__ uint64_t mul_wide(uint32_t x, uint32_t m)
-{
-    uint64_t p;
-    asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(x), "r"(m));
-    return p;
-}
-
-// The words x1, x3 of one Philox4x32-10 block (the high words of the right and
-// left draws).  The first two rounds split into a part of (step, rail) alone,
-// formed once per step in (u1, u2, u3), and one multiply each of the site's;
-// the last round needs only the low halves of its products.
-struct StepDraw {
-    uint32_t u1, u2, u3;
-};
-__device__ __forceinline__ StepDraw step_draw(uint32_t t, uint32_t rail, const uint32_t *rk0,
-                                              const uint32_t *rk1)
-{
-    const uint64_t a = mul_wide(t, kM1);
-    const uint32_t c0 = (uint32_t)(a >> 32) ^ rail ^ rk0[0];
-    const uint64_t b = mul_wide(c0, kM0);
-    StepDraw d;
-    d.u1 = (uint32_t)a ^ rk0[1];
-    d.u2 = (uint32_t)(b >> 32) ^ rk1[1];
-    d.u3 = (uint32_t)b;
-    return d;
-}
-// The site's part of the first two rounds: three words that depend on the site
-// and the instance only.
-__device__ __forceinline__ uint3 site_words(uint32_t site, uint32_t kc)
-{
-    const uint64_t a = mul_wide(site, kM0);
-    const uint64_t b = mul_wide((uint32_t)(a >> 32) ^ kc, kM1);
-    return make_uint3((uint32_t)(b >> 32), (uint32_t)b, (uint32_t)a);
-}
-__device__ __forceinline__ void site_draw(const StepDraw &d, uint32_t w0, uint32_t w1, uint32_t w2,
-                                          const uint32_t *rk0, const uint32_t *rk1, uint32_t &xy, uint32_t &xw)
-{
-    uint32_t c0 = w0 ^ d.u1, c1 = w1;
-    uint32_t c2 = w2 ^ d.u2, c3 = d.u3;
-#pragma unroll
-    for (int i = 2; i < 9; ++i) {
-        const uint64_t p0 = mul_wide(c0, kM0), p1 = mul_wide(c2, kM1);
-        c0 = (uint32_t)(p1 >> 32) ^ c1 ^ rk0[i];
-        c1 = (uint32_t)p1;
-        c2 = (uint32_t)(p0 >> 32) ^ c3 ^ rk1[i];
-        c3 = (uint32_t)p0;
-    }
-    xy = c2 * kM1;
-    xw = c0 * kM0;
-}
-
-// The site table (per CTA, one uint4 per position -1 .. L): the three words of
-// site_words, and the position's entry, as the lists hold it: 16 times
-// (position + 1), its own byte offset in the table, in the low 16 bits, above
-// them the byte offset of its row of decision bounds.  Rows: one per zone, of
-// an open rail four more for positions -1, 0, L - 1, L, and a dead row (nothing
-// accepted) for the unused slots of a column.  Looking the words up takes two of
-// the draw's 16 widening multiplies off the pipe that bounds the loop.
-constexpr int kStep = 16;          // an entry's difference between neighbouring positions
-__device__ __forceinline__ int pos_of(uint32_t e) { return (int)((e & 0xFFFFu) / kStep) - 1; }
-__device__ __forceinline__ uint4 site_at(const uint8_t *tab, uint32_t e) { return *(const uint4 *)(tab + (e & 0xFFFFu)); }
-// zone code of a row: z + 1, and 0 / Z + 1 for the virtual sites -1 / L
-__device__ __forceinline__ int code_of_row(int row, int Z)
-{
-    return row < Z ? row + 1 : (row < Z + 2 ? row - Z : (row == Z + 2 ? Z : Z + 1));
-}
-
-// A warp's block: header of 64 bytes (band factor and mid voltage of the voltage
-// window float [2], the largest column, the step up to which draws are counted),
-// int [G] each of F, N0 and the sum of positions that the per-rail current
-// counts from, then the bounds.
-constexpr uint32_t kIonHead = 64u;
-__host__ __device__ constexpr uint32_t ion_fixed(int P) { return kIonHead + (uint32_t)align16(12u * (32u / (uint32_t)P)); }
-// per-lane words ([kIonSlots][32]): entries of the column; distances from its
-// first entry to the one before (low half) and from its last to the one after
-// (high half), on the neighbouring lanes or the rail's ends; moves since the
-// last flush
-enum { kSlotN = 0, kSlotGaps = 1, kSlotMoves = 2, kIonSlots = 3 };
-
-// The thread index, read anew.  Each phase of a step forms its addresses from
-// it and takes its state from shared memory, so that no phase's registers are
-// held through another: with one set of pointers for the whole launch the draw
-// loop ran on spilled values.
-__device__ __forceinline__ uint32_t tid_here()
-{
-    uint32_t v;
-    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(v));
-    return v;
-}
-// A lane's view of its warp's shared memory.
-template <int P>
-struct IonView {
-    static constexpr int G = 32 / P;
-    const SweepArgs &a;
-    uint32_t tid;
-    uint8_t *sb;
-    __device__ __forceinline__ IonView(const SweepArgs &args, uint8_t *smem) : a(args)
-    {
-        tid = tid_here();
-        sb = smem + a.iy.tab + (tid >> 5) * a.iy.bytes;
-    }
-    __device__ __forceinline__ int lane() const { return (int)(tid & 31u); }
-    __device__ __forceinline__ int seg() const { return (int)(tid & 31u) / P; }
-    __device__ __forceinline__ int sl() const { return (int)(tid & (P - 1)); }
-    __device__ __forceinline__ int64_t rail(int64_t tile_rail0) const { return tile_rail0 + (int64_t)(tid >> 5) * G + seg(); }
-    __device__ __forceinline__ float4 &band() const { return *(float4 *)sb; }
-    __device__ __forceinline__ int &kmax() const { return *(int *)(sb + 16); }
-    __device__ __forceinline__ int &mark() const { return *(int *)(sb + 20); }
-    // [0] F, [G] N0, [2 G] sum of positions
-    __device__ __forceinline__ int32_t *Fs(int sg) const { return (int32_t *)(sb + kIonHead) + sg; }
-    __device__ __forceinline__ int32_t *Fs() const { return Fs(seg()); }
-    __device__ __forceinline__ uint8_t *bounds(int sg) const { return sb + ion_fixed(P) + sg * (int)a.iy.row; }
-    __device__ __forceinline__ uint8_t *bounds() const { return bounds(seg()); }
-    __device__ __forceinline__ uint32_t *words() const { return (uint32_t *)(sb + ion_fixed(P)); }
-    __device__ __forceinline__ float4 *zf(int sg) const { return (float4 *)(sb + a.iy.zf) + sg * a.Z; }
-    __device__ __forceinline__ float2 *p0b(int sg) const { return (float2 *)(sb + a.iy.p0b) + sg * a.Z; }
-    __device__ __forceinline__ int32_t *Pb(int sg) const { return (int32_t *)(sb + a.iy.pb) + sg * (a.Z + 1); }
-    __device__ __forceinline__ uint32_t &slot(int k) const { return ((uint32_t *)(sb + a.iy.st))[k * 32 + lane()]; }
-    __device__ __forceinline__ uint32_t *col() const { return (uint32_t *)(sb + a.iy.col); }
-    __device__ __forceinline__ uint32_t *colp() const { return col() + lane(); }
-};
-__device__ __forceinline__ int gap_first(uint32_t w) { return (int)(w & 0xFFFFu); }
-__device__ __forceinline__ int gap_last(uint32_t w) { return (int)(w >> 16); }
-
-// Bits of a lane's rows: 32 or 64.
-__device__ __forceinline__ int count_bits(uint32_t m) { return __popc(m); }
-__device__ __forceinline__ int count_bits(uint64_t m) { return __popcll(m); }
-__device__ __forceinline__ int first_bit(uint32_t m) { return __ffs(m) - 1; }
-__device__ __forceinline__ int first_bit(uint64_t m) { return __ffsll(m) - 1; }
-template <class M>
-__device__ __forceinline__ M low_bits(int n)      // n in [0, bits of M]
-{
-    return n < (int)(8 * sizeof(M)) ? (M(1) << n) - M(1) : ~M(0);
-}
-
-// Row j of a lane's column (n entries): the distances to its step-start
-// neighbours and which of its trials are open (the neighbouring site free, or
-// an open electrode; under the even/odd rule only across the active bond).
-struct IonEntry {
-    uint32_t e;
-    int x, gL, gR;
-    bool fL, fR;
-};
-__device__ __forceinline__ IonEntry ion_entry(const uint32_t *colp, int j, int n, uint32_t gaps, int rule,
-                                              uint32_t t)
-{
-    IonEntry q;
-    q.e = colp[j * 32];
-    q.x = pos_of(q.e);
-    q.gL = j > 0 ? q.x - pos_of(colp[(j - 1) * 32]) : gap_first(gaps);
-    q.gR = j + 1 < n ? pos_of(colp[(j + 1) * 32]) - q.x : gap_last(gaps);
-    q.fR = j < n && q.gR > 1;
-    q.fL = j < n && q.gL > 1;
-    if (rule != 0) {
-        // the bond right of x is active when x = t (mod 2)
-        const bool odd = ((q.x ^ (int)t) & 1) != 0;
-        q.fR = q.fR && !odd;
-        q.fL = q.fL && odd;
-    }
-    return q;
-}
-
-// A draw within the FP32 band of its probability: the FP64 band, then the exact
-// path.  d* in: 2 for a trial to decide, else 0 or 1; out: 0 or 1.
-template <int P>
-__device__ __forceinline__ void ion_exact(const IonView<P> &c, int sg, int64_t r2, int pos, int zone,
-                                          uint32_t t, int &dR, int &dL)
-{
-    constexpr int G = 32 / P;
-    const SweepArgs &a = c.a;
-    const int L = a.L, Z = a.Z;
-    const DevConst *K = a.K;
-    const int site = min(max(pos, 0), L - 1);
-    const bool open = a.electrodes == 1;
-    const int kindR = pos < 0 ? 1 : (open && pos == L - 1 ? 2 : 0);
-    const int kindL = pos >= L ? 1 : (open && pos == 0 ? 2 : 0);
-    const uint4 x = philox((uint32_t)site, a.rail_base + (uint32_t)r2, t, a.instance, a.rk0, a.rk1);
-    const double V = a.V[t];
-    const double P0k = a.P0bnd != nullptr ? a.P0site[r2 * L + site] : K->P0;
-    const double baseR = kindR == 1 ? K->E_in : (kindR == 2 ? K->E_out : P0k);
-    const double baseL = kindL == 1 ? K->E_in : (kindL == 2 ? K->E_out : P0k);
-    const uint64_t wR = ((uint64_t)x.y << 32) | x.x, wL = ((uint64_t)x.w << 32) | x.z;
-    const int32_t *Pb = c.Pb(sg);
-    const int32_t *Fs = c.Fs(sg);
-    unsigned ne = 0;
-    // FP64 band (kmc_sweep.cu, slow_candidate): p to 1e-13 relative, so a draw
-    // more than 1e-11 from it is decided.  m_z does not change when every P_b
-    // is shifted by the same count, as an open rail's are.
-    if (a.bgd) {
-        const int m = (int)((uint32_t)L * (uint32_t)(Pb[zone] + Pb[zone + 1]) - (uint32_t)Fs[0]);
-        const double dq = __fma_rn((double)m, K->half_invL, -a.bgd[r2 * Z + zone].y);
-        const double xx = __dmul_rn(__fma_rn(-K->ka, dq, V), K->xs);
-        if (fabs(xx) < 600.0) {
-            const double Bf = exp(xx);
-            const double invf = 1.0 / (1.0 + Bf);
-            if (dR == 2) {
-                const double d = __dsub_rn(__dmul_rn((double)(wR >> 11), 0x1.0p-53),
-                                           __dmul_rn(__dmul_rn(baseR, invf), Bf));
-                if (fabs(d) > 1e-11) {
-                    dR = d <= 0.0 ? 1 : 0;
-                    ++ne;
-                }
-            }
-            if (dL == 2) {
-                const double d = __dsub_rn(__dmul_rn((double)(wL >> 11), 0x1.0p-53),
-                                           __dmul_rn(baseL, invf));
-                if (fabs(d) > 1e-11) {
-                    dL = d <= 0.0 ? 1 : 0;
-                    ++ne;
-                }
-            }
-        }
-    }
-    if (dR == 2 || dL == 2) {
-        double B, inv;
-        exact_zone(Pb, K, Z, L, Fs[G], a.bgd ? a.bgd + r2 * Z : nullptr, V, zone, &B, &inv);
-        const int32_t rg = (int32_t)(a.rail_base + (uint32_t)r2);
-        if (dR == 2) {
-            const double p = __dmul_rn(__dmul_rn(baseR, inv), B);   // Eq. 6
-            dR = exact_trial(wR, p, a.log, a.log_count, a.log_cap, rg, t, site, 0, kindR) ? 1 : 0;
-            ++ne;
-        }
-        if (dL == 2) {
-            const double p = __dmul_rn(baseL, inv);                  // Eq. 5
-            dL = exact_trial(wL, p, a.log, a.log_count, a.log_cap, rg, t, site, 1, kindL) ? 1 : 0;
-            ++ne;
-        }
-    }
-    atomicAdd(&a.counters[1], (unsigned long long)ne);
-}
-
-// Distances across the lanes of a rail, for the columns as they stand (n entries
-// on this lane).  wallL, wallR: the positions beyond a rail's ends.
-template <int P>
-__device__ __forceinline__ void ion_refresh(const IonView<P> &c, int n, int wallL, int wallR)
-{
-    const uint32_t *colp = c.colp();
-    const int xF = n > 0 ? pos_of(colp[0]) : wallR;
-    const int xL = n > 0 ? pos_of(colp[(n - 1) * 32]) : wallR;
-    int up = __shfl_up_sync(FULL, xL, 1, P), dn = __shfl_down_sync(FULL, xF, 1, P);
-    if (c.sl() == 0) up = wallL;
-    if (c.sl() == P - 1) dn = wallR;
-    c.slot(kSlotGaps) = (uint32_t)(xF - up) | (uint32_t)(dn - xL) << 16;
-}
-
-// Deals a warp's entries out evenly from the occupancy words (staged where the
-// bounds are): M / P to a lane and one more to the first M % P lanes; the other
-// slots are dead.  Sets the lane's state words and the largest column.
-template <int P, bool OPEN>
-__device__ __forceinline__ void ion_build(const IonView<P> &c, const uint8_t *tab, bool active)
-{
-    const SweepArgs &a = c.a;
-    const int L = a.L, W = (L + 31) >> 5, C = (W + P - 1) / P, sl = c.sl();
-    const int w0 = min(sl * C, W), w1 = min(w0 + C, W);
-    const uint32_t *words = c.words() + c.seg() * W;
-    uint32_t *col = c.col();
-    const uint32_t dead = (a.iy.row - 16u) << 16 | (uint32_t)kStep;
-    for (int r = 0; r < a.rcap; ++r) col[r * 32 + c.lane()] = dead;
-    int cnt = 0;
-    for (int w = w0; w < w1; ++w) cnt += __popc(words[w]);
-    int incl = cnt;
-#pragma unroll
-    for (int off = 1; off < P; off <<= 1) {
-        const int v = __shfl_up_sync(FULL, incl, off, P);
-        if (sl >= off) incl += v;
-    }
-    const int total = __shfl_sync(FULL, incl, P - 1, P);
-    int vl = 0, vr = 0;
-    if (OPEN && active) {
-        vl = (words[0] & 1u) ? 0 : 1;
-        vr = ((words[(L - 1) >> 5] >> ((L - 1) & 31)) & 1u) ? 0 : 1;
-    }
-    const int M = total + vl + vr;
-    const int base = M / P, rem = M - base * P;
-    __syncwarp();
-    auto place = [&](int i, int xb) {
-        int l, r;
-        if (i < rem * (base + 1)) {
-            l = i / (base + 1);
-            r = i - l * (base + 1);
-        } else {
-            const int i2 = i - rem * (base + 1);
-            l = i2 / base;      // base > 0: M > rem (base + 1) here
-            r = i2 - l * base;
-            l += rem;
-        }
-        col[r * 32 + c.seg() * P + l] = site_at(tab, (uint32_t)xb * kStep).w;
-    };
-    int i = incl - cnt + vl;
-    for (int w = w0; w < w1; ++w) {
-        uint32_t m = words[w];
-        while (m) {
-            place(i++, 32 * w + __ffs(m));      // position + 1
-            m &= m - 1;
-        }
-    }
-    if (sl == 0 && vl) place(0, 0);
-    if (sl == P - 1 && vr) place(M - 1, L + 1);
-    __syncwarp();
-    const int n = base + (sl < rem ? 1 : 0);
-    if (sl == 0) *(uint4 *)(c.bounds() + a.iy.row - 16u) = make_uint4(0u, 0u, 0u, 0u);
-    c.slot(kSlotN) = (uint32_t)n;
-    const int km = __reduce_max_sync(FULL, n);
-    if (c.lane() == 0) c.kmax() = km;
-    ion_refresh<P>(c, n, OPEN ? -2 : -1, OPEN ? L + 1 : L);
-    __syncwarp();
-}
-
-// The sum of the positions of a rail's entries (on all of its lanes).
-template <int P>
-__device__ __forceinline__ int ion_sum(const IonView<P> &c)
-{
-    const uint32_t *colp = c.colp();
-    const int n = (int)c.slot(kSlotN);
-    int v = 0;
-    for (int r = 0; r < n; ++r) v += pos_of(colp[r * 32]);
-#pragma unroll
-    for (int off = P / 2; off >= 1; off >>= 1) v += __shfl_xor_sync(FULL, v, off, P);
-    return v;
-}
-
-// The occupancy words of the lists (staged where the bounds are).
-template <int P>
-__device__ __forceinline__ void ion_to_words(const IonView<P> &c)
-{
-    const int L = c.a.L, W = (L + 31) >> 5;
-    uint32_t *words = c.words();
-    const uint32_t *colp = c.colp();
-    __syncwarp();
-    for (int i = c.lane(); i < 32 / P * W; i += 32) words[i] = 0u;
-    __syncwarp();
-    const int n = (int)c.slot(kSlotN);
-    for (int r = 0; r < n; ++r) {
-        const int x = pos_of(colp[r * 32]);
-        if (x >= 0 && x < L) atomicOr(&words[c.seg() * W + (x >> 5)], 1u << (x & 31));
-    }
-    __syncwarp();
-}
-
-// Entry e at *at moves by m: its new entry, and when it crosses a zone boundary
-// b the counts P_b and F, which lose (rightward) or gain one ion, and the zone
-// counts of the next step, zc[b - 1] and zc[b] (null after the launch's last
-// step).  Returns whether it crossed one.
-template <int P>
-__device__ __forceinline__ bool ion_commit(const IonView<P> &c, const uint8_t *tab, uint32_t *at, uint32_t e,
-                                           int m, unsigned long long *zc)
-{
-    const SweepArgs &a = c.a;
-    const uint32_t en = site_at(tab, (e & 0xFFFFu) + (uint32_t)(kStep * m)).w;
-    *at = en;
-    if (((e ^ en) >> 16) == 0u) return false;
-    const int k0 = code_of_row((int)(e >> 20), a.Z), k1 = code_of_row((int)(en >> 20), a.Z);
-    if (k0 == k1) return false;
-    const int b = max(k0, k1) - 1;
-    atomicAdd(&c.Pb(c.seg())[b], -m);
-    atomicAdd(c.Fs(), -m * a.wsum[b]);
-    if (zc) {
-        if (b > 0) atomicAdd(zc + (b - 1), (unsigned long long)(long long)(-m));
-        if (b < a.Z) atomicAdd(zc + b, (unsigned long long)(long long)m);
-    }
-    return true;
-}
-
-// The field of S2.1.8, Eqs. 3-6 and the decision bounds of the zones of the rail
-// slots in `dirty` (bits), for step s.  Bounds: p lies within a factor 1 +- eps
-// of its FP32 value, times [1 / eh, eh] over a voltage window.  With u = 2^-24,
-// every one of the twelve roundings that lead to the exponent x is relative to
-// at most S = (|V| + |kappa alpha| (P_z + P_z+1 + F / L + N0)) / (L kT), so x is
-// off by less than 16 u S, and Eqs. 5-6 move by that relatively (their
-// logarithmic derivatives with respect to x are at most 1); __expf adds
-// (2 + 1.2 |x|) ulp, the division two, the other operations three.
-template <int P, bool OPEN>
-__device__ __forceinline__ void ion_zones(const IonView<P> &c, int64_t t0, int s, int n_steps, bool window,
-                                          uint32_t dirty, int &wend)
-{
-    constexpr int VWIN = 32;              // steps per voltage window of the bounds
-    constexpr int G = 32 / P;
-    const SweepArgs &a = c.a;
-    const int Z = a.Z;
-    if (window) {
-        // A window: steps from s on, at most VWIN, whose voltage stays near the
-        // first one's.  Evaluating at the window's mid voltage changes B/(1+B)
-        // and 1/(1+B) by a factor within [e^-h, e^h] (logarithmic derivatives at
-        // most 1); a jump (a pulse's edge) would widen the bounds by several per
-        // cent for all of the window's steps, so it starts the next one.
-        const int left = min(VWIN, n_steps - s);
-        const double v = a.V[t0 + s + min(c.lane(), left - 1)];
-        const float v0 = __shfl_sync(FULL, (float)v, 0);
-        const uint32_t far = __ballot_sync(FULL, fabsf((float)v - v0) * a.inv_LkT > 2e-3f);
-        const int len = min(left, far ? __ffs(far) - 1 : VWIN);
-        float vlo = __double2float_rd(v), vhi = __double2float_ru(v);
-        if (c.lane() >= len) vlo = vhi = v0;
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            vlo = fminf(vlo, __shfl_xor_sync(FULL, vlo, off));
-            vhi = fmaxf(vhi, __shfl_xor_sync(FULL, vhi, off));
-        }
-        const float h = 0.5f * (vhi - vlo) * a.inv_LkT;
-        if (c.lane() == 0) {
-            float4 &b = c.band();
-            b.x = __expf(h) * (1.0f + 4e-6f + 2e-6f * h);
-            b.y = 0.5f * (vlo + vhi);
-        }
-        wend = s + len;
-    }
-    __syncwarp();
-    const float eh = c.band().x, Vf = c.band().y;
-    const int items = __popc(dirty) * Z;
-    for (int i = c.lane(); i < items; i += 32) {
-        const int k = (int)(((uint32_t)i * a.rcpZ) >> 16), z = i - k * Z;    // i / Z for i < 1024
-        uint32_t m = dirty;
-        for (int q = 0; q < k; ++q) m &= m - 1;
-        const int sg = G == 1 ? 0 : __ffs(m) - 1;
-        const int32_t *Pb = c.Pb(sg), *Fs = c.Fs(sg);
-        uint8_t *rm = c.bounds(sg);
-        // an open rail's counts are relative to its first boundary
-        const int p0 = OPEN ? Pb[0] : 0;
-        const int Pz = Pb[z] - p0, Pz1 = Pb[z + 1] - p0;
-        const int F = OPEN ? (int)((uint32_t)Fs[0] - (uint32_t)p0 * (uint32_t)(2 * a.L)) : Fs[0];
-        const float Ff = (float)F * a.inv_L, Nf = (float)Fs[G], Pf = (float)(Pz + Pz1);
-        const float qd = 0.5f * (Pf - Ff) - Nf * a.cz[z];
-        const float x = -(Vf - a.ka_f * qd) * a.inv_LkT;
-        const float S = (fabsf(Vf) + fabsf(a.ka_f) * (Pf + Ff + Nf)) * a.inv_LkT;
-        const float eps = 4e-6f + 5e-7f * fabsf(x) + 1.2e-6f * S;
-        const bool ok = fabsf(x) <= 40.0f && eps < 0.25f;
-        // no bounds: every draw of the zone goes to the FP64 paths
-        uint4 b = make_uint4(FULL, FULL, 0u, 0u);
-        float inv = 0.0f, sR = 0.0f, flo = 0.0f, fhi = 0.0f;
-        if (ok) {
-            const float B = __expf(x);
-            inv = __fdividef(1.0f, 1.0f + B);
-            sR = inv * B;
-            flo = __fdividef(1.0f - eps, eh);
-            fhi = (1.0f + eps) * eh;
-            float blo = a.P0f_scalar, bhi = a.P0f_scalar;
-            if (a.P0bnd != nullptr) {
-                const float2 pp = c.p0b(sg)[z];
-                blo = pp.x;
-                bhi = pp.y;
-            }
-            b.x = rej_thr(bhi * sR * fhi);
-            b.y = rej_thr(bhi * inv * fhi);
-            b.z = acc_thr(blo * sR * flo);
-            b.w = acc_thr(blo * inv * flo);
-        }
-        *(uint4 *)(rm + z * 16) = b;
-        if (a.P0bnd != nullptr) c.zf(sg)[z] = make_float4(sR, inv, flo, fhi);
-        if (OPEN && (z == 0 || z == Z - 1)) {
-            // electrode positions: outward trials are extractions, the virtual
-            // sites' inward trials injections
-            const float Ein = a.E_inf, Eout = a.E_outf;
-            if (z == 0) {
-                uint4 e = b, q = b;
-                if (ok) {
-                    e.x = rej_thr(Ein * sR * fhi);
-                    e.z = acc_thr(Ein * sR * flo);
-                    q.y = rej_thr(Eout * inv * fhi);
-                    q.w = acc_thr(Eout * inv * flo);
-                }
-                *(uint4 *)(rm + Z * 16) = e;
-                *(uint4 *)(rm + Z * 16 + 16) = q;
-            }
-            if (z == Z - 1) {
-                uint4 e = b, q = b;
-                if (ok) {
-                    e.y = rej_thr(Ein * inv * fhi);
-                    e.w = acc_thr(Ein * inv * flo);
-                    q.x = rej_thr(Eout * sR * fhi);
-                    q.z = acc_thr(Eout * sR * flo);
-                }
-                *(uint4 *)(rm + Z * 16 + 32) = q;
-                *(uint4 *)(rm + Z * 16 + 48) = e;
-            }
-        }
-    }
-    __syncwarp();
-}
-
-// The list ends of open rails after a step's moves: the first entry stays at
-// site -1 or 0, the last at L - 1 or L.  Returns (warp-uniform) whether the
-// bounds were overwritten.
-template <int P>
-__device__ __forceinline__ bool ion_ends(const IonView<P> &c, const uint8_t *tab, int s, bool active,
-                                         uint32_t &draws)
-{
-    const SweepArgs &a = c.a;
-    const int L = a.L, sl = c.sl();
-    const uint32_t dead = (a.iy.row - 16u) << 16 | (uint32_t)kStep;
-    uint32_t *colp = c.colp();
-    const uint32_t gaps = c.slot(kSlotGaps);
-    const int n0 = (int)c.slot(kSlotN);
-    int n = n0;
-    if (n > 0 && sl == 0) {
-        const int xF = pos_of(colp[0]);
-        if (xF > 0) {
-            for (int r = n; r > 0; --r) colp[r * 32] = colp[(r - 1) * 32];
-            colp[0] = site_at(tab, 0u).w;
-            ++n;
-            atomicAdd(&c.Fs()[2 * (32 / P)], -1);     // entries that come and go are no moves
-        } else if (xF < 0) {
-            const int x2 = n > 1 ? pos_of(colp[32]) : xF + gap_last(gaps);
-            if (x2 == 0) {
-                --n;
-                for (int r = 0; r < n; ++r) colp[r * 32] = colp[(r + 1) * 32];
-                colp[n * 32] = dead;
-                atomicAdd(&c.Fs()[2 * (32 / P)], 1);
-            }
-        }
-    }
-    const int xe = n > 0 ? pos_of(colp[(n - 1) * 32]) : 0;
-    if (n > 0 && (sl == P - 1 || xe + gap_last(gaps) == L + 1)) {        // the lane of the last entry
-        if (xe < L - 1) {
-            colp[n * 32] = site_at(tab, (uint32_t)(L + 1) * kStep).w;
-            ++n;
-            atomicAdd(&c.Fs()[2 * (32 / P)], L);
-        } else if (xe == L) {
-            const int x2 = n > 1 ? pos_of(colp[(n - 2) * 32]) : xe - gap_first(gaps);
-            if (x2 == L - 1) {
-                --n;
-                colp[n * 32] = dead;
-                atomicAdd(&c.Fs()[2 * (32 / P)], -L);
-            }
-        }
-    }
-    if (!__any_sync(FULL, n != n0)) return false;
-    // draws so far were of the old columns
-    draws = __reduce_add_sync(FULL, (uint32_t)n0) * (uint32_t)(s + 1 - c.mark());
-    __syncwarp();
-    if (c.lane() == 0) c.mark() = s + 1;
-    c.slot(kSlotN) = (uint32_t)n;
-    // deal the entries out again when a lane ran empty, holds more than one
-    // above its even share or has outgrown its bits
-    int M = n;
-#pragma unroll
-    for (int off = P / 2; off >= 1; off >>= 1) M += __shfl_xor_sync(FULL, M, off, P);
-    if (__any_sync(FULL, (n0 > 0 && n == 0) || n > min((M + P - 1) / P + 1, a.rcap - 2))) {
-        ion_to_words<P>(c);
-        ion_build<P, true>(c, tab, active);
-        return true;
-    }
-    const int km = __reduce_max_sync(FULL, n);
-    if (c.lane() == 0) c.kmax() = km;
-    ion_refresh<P>(c, n, -2, L + 1);
-    __syncwarp();
-    return false;
-}
-
-// One CTA's tile of rails advanced through steps [t0, t0 + n_steps): rails
-// [tile_rail0, tile_rail0 + G * warps).  The draw loop only compares each
-// entry's two words with its bounds and keeps the outcomes as bits of M, one
-// per row.  With ACC (hop probabilities of order 1e-2 and above, several
-// accepted draws per warp and step) it also compares with the lower bounds and
-// keeps which neighbours are one and two sites away, so that exclusion and
-// conflicts are a few operations on bits; without, the entries with a word
-// below its upper bound are looked at one by one.
-template <int P, bool ACC, bool OPEN, class M>
-__device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0, const uint32_t *rk1,
-                                         int64_t t0, int n_steps, int flush, int64_t tile_rail0,
-                                         uint8_t *smem)
-{
-    constexpr int G = 32 / P;
-    using View = IonView<P>;
-    uint8_t *tab = smem;    // site table of the CTA
-
-    {
-        const View c(a, smem);
-        const int L = a.L, Z = a.Z, sl = c.sl();
-        const int64_t rail = c.rail(tile_rail0);
-        const bool active = rail < a.R;
-        // ---- site table of the CTA
-        for (int i = (int)c.tid; i < L + 2; i += blockDim.x) {
-            const int k = min(max(i - 1, 0), L - 1);
-            int row = 0;
-            while (a.bnd[row + 1] <= k) ++row;
-            if (OPEN && i <= 1) row = Z + i;
-            if (OPEN && i >= L) row = Z + 2 + (i - L);
-            const uint3 w = site_words((uint32_t)k, a.instance ^ rk1[0]);
-            ((uint4 *)tab)[i] = make_uint4(w.x, w.y, w.z, (uint32_t)(i * kStep) | (uint32_t)(row * 16) << 16);
-        }
-        // ---- occupancy words of the warp's rails, read once from HBM
-        const int W = (L + 31) >> 5;          // words per rail
-        const int C = (W + P - 1) / P;        // words per lane
-        const int w0 = min(sl * C, W), w1 = min(w0 + C, W);
-        uint32_t *words = c.words() + c.seg() * W;
-        for (int w = w0; w < w1; ++w) {
-            uint32_t bits = 0;
-            if (active) {
-                const uint8_t *row = a.occ + rail * a.stride + 32 * w;
-                bits = pack16(*(const uint4 *)row);
-                if (32 * w + 16 < a.stride) bits |= pack16(*(const uint4 *)(row + 16)) << 16;
-                if (32 * w + 32 > L) bits &= (1u << (L - 32 * w)) - 1u;
-            }
-            words[w] = bits;
-        }
-        if (sl == 0) c.Fs()[G] = active ? a.N0[rail] : 0;
-        if (a.P0bnd != nullptr)
-            for (int z = sl; z < Z; z += P)
-                c.p0b(c.seg())[z] = active ? a.P0bnd[rail * Z + z] : make_float2(0.0f, 0.0f);
-        c.slot(kSlotMoves) = 0u;
-        if (c.lane() == 0) c.mark() = 0;
-        __syncthreads();
-        if (rail - c.seg() >= a.R) return;
-        // ---- ions below each zone boundary and F
-        for (int b = sl; b <= Z; b += P) {
-            const int e = a.bnd[b];
-            int m = 0;
-            for (int w = 0; w < (e >> 5); ++w) m += __popc(words[w]);
-            if (e & 31) m += __popc(words[e >> 5] & ((1u << (e & 31)) - 1u));
-            c.Pb(c.seg())[b] = m;
-        }
-        __syncwarp();
-        if (sl == 0) {
-            int f = 0;
-            for (int b = 0; b <= Z; ++b) f += c.Pb(c.seg())[b] * a.wsum[b];
-            c.Fs()[0] = f;
-        }
-        // zone counts of the launch's first step (the changes of later ones follow)
-        for (int z = sl; z < Z; z += P) {
-            const int nz = c.Pb(c.seg())[z + 1] - c.Pb(c.seg())[z];
-            if (nz != 0) atomicAdd(&a.Zc[t0 * Z + z], (unsigned long long)(long long)nz);
-        }
-        ion_build<P, OPEN>(c, tab, active);
-        const int sum = ion_sum<P>(c);
-        if (sl == 0) c.Fs()[2 * G] = sum;
-        __syncwarp();
-    }
-
-    int wend = 0;          // first step after the voltage window of the bounds
-    uint32_t dirty = 0u;   // rail slots whose zone sums changed since their bounds were evaluated
-    for (int c0 = 0; c0 < n_steps; c0 += flush) {
-        const int c1 = min(n_steps, c0 + flush);
-        for (int s = c0; s < c1; ++s) {
-            const uint32_t t = (uint32_t)(t0 + s);
-
-            if (dirty != 0u || s == wend) {
-                const View c(a, smem);
-                ion_zones<P, OPEN>(c, t0, s, n_steps, s == wend,
-                                   s == wend ? (uint32_t)((1ull << G) - 1u) : dirty, wend);
-            }
-            dirty = 0u;
-
-            // ---- draws: accepted trials aR, aL (M bits per row), entries with a
-            //      draw still to be decided, and rows whose successor is two
-            //      sites away
-            M aR = 0, aL = 0, und = 0, two = 0;
-            {
-                const View c(a, smem);
-                const StepDraw sd = step_draw(t, a.rail_base + (uint32_t)c.rail(tile_rail0), rk0, rk1);
-                const uint8_t *rm = c.bounds();
-                const uint32_t *cp = c.colp();
-                const uint32_t *const end = cp + c.kmax() * 32;
-                M bit = 1;
-                if constexpr (ACC) {
-                    M sR = 0, sL = 0, one = 0;
-                    uint32_t e = *cp;
-#pragma unroll 4
-                    while (cp != end) {
-                        cp += 32;
-                        const uint32_t en = *cp;        // the column has one slot more than rows in use
-                        const uint32_t gap = (en & 0xFFFFu) - (e & 0xFFFFu);
-                        const uint4 w = site_at(tab, e);
-                        uint32_t xy, xw;
-                        site_draw(sd, w.x, w.y, w.z, rk0, rk1, xy, xw);
-                        const uint4 th = *(const uint4 *)(rm + (e >> 16));
-                        if (xy <= th.x) aR |= bit;
-                        if (xw <= th.y) aL |= bit;
-                        if (xy < th.z) sR |= bit;
-                        if (xw < th.w) sL |= bit;
-                        if (gap == 1u * kStep) one |= bit;
-                        if (gap == 2u * kStep) two |= bit;
-                        bit <<= 1;
-                        e = en;
-                    }
-                    const int n = (int)c.slot(kSlotN);
-                    const uint32_t gaps = c.slot(kSlotGaps);
-                    // the last entry's successor is on the next lane
-                    const M last = n > 0 ? M(1) << (n - 1) : M(0), valid = low_bits<M>(n);
-                    one = (one & (valid >> 1)) | (gap_last(gaps) == 1 ? last : 0);
-                    two = (two & (valid >> 1)) | (gap_last(gaps) == 2 ? last : 0);
-                    aR &= valid & ~one;
-                    aL &= valid & ~(one << 1 | (gap_first(gaps) == 1 ? 1u : 0u));
-                    if (a.rule != 0) {
-                        M odd = 0;
-                        for (int r = 0; r < n; ++r)
-                            if ((pos_of(c.colp()[r * 32]) ^ (int)t) & 1) odd |= M(1) << r;
-                        aR &= ~odd;
-                        aL &= odd;
-                    }
-                    und = (aR & ~sR) | (aL & ~sL);
-                } else {
-#pragma unroll 4
-                    while (cp != end) {
-                        const uint32_t e = *cp;
-                        cp += 32;
-                        const uint4 w = site_at(tab, e);
-                        uint32_t xy, xw;
-                        site_draw(sd, w.x, w.y, w.z, rk0, rk1, xy, xw);
-                        const uint2 th = *(const uint2 *)(rm + (e >> 16));
-                        if (xy <= th.x || xw <= th.y) und |= bit;
-                        bit <<= 1;
-                    }
-                }
-            }
-            if (!__any_sync(FULL, (aR | aL | und) != 0)) continue;
-
-            // ---- draws between their bounds (without ACC every draw that may be
-            //      accepted): the site's own base probability in the FP32 band
-            if (__any_sync(FULL, und != 0)) {
-                M left = 0;
-                {
-                    const View c(a, smem);
-                    const int64_t rail = c.rail(tile_rail0);
-                    const StepDraw sd = step_draw(t, a.rail_base + (uint32_t)rail, rk0, rk1);
-                    const int n = (int)c.slot(kSlotN);
-                    const uint32_t gaps = c.slot(kSlotGaps);
-                    for (; und; und &= und - 1) {
-                        const M bit = und & (M(0) - und);
-                        const IonEntry q = ion_entry(c.colp(), first_bit(und), n, gaps, a.rule, t);
-                        const uint32_t site = (uint32_t)min(max(q.x, 0), a.L - 1);
-                        const uint4 w = site_at(tab, q.e);
-                        uint32_t xy, xw;
-                        site_draw(sd, w.x, w.y, w.z, rk0, rk1, xy, xw);
-                        const uint4 th = *(const uint4 *)(c.bounds() + (q.e >> 16));
-                        int dR = q.fR && xy <= th.x ? (xy < th.z ? 1 : 2) : 0;
-                        int dL = q.fL && xw <= th.y ? (xw < th.w ? 1 : 2) : 0;
-                        if (a.P0bnd != nullptr && (dR == 2 || dL == 2)) {
-                            // inner trials (electrode trials have one base probability)
-                            const int row = (int)(q.e >> 20);
-                            const float4 z = c.zf(c.seg())[min(max(code_of_row(row, a.Z) - 1, 0), a.Z - 1)];
-                            if (z.y > 0.0f) {
-                                const float P0 = __ldg(a.P0f + rail * a.L + site);
-                                if (dR == 2 && row != a.Z && row != a.Z + 2) dR = bounded(xy, P0 * z.x, z.z, z.w);
-                                if (dL == 2 && row != a.Z + 1 && row != a.Z + 3) dL = bounded(xw, P0 * z.y, z.z, z.w);
-                            }
-                        }
-                        aR = dR == 1 ? aR | bit : aR & ~bit;
-                        aL = dL == 1 ? aL | bit : aL & ~bit;
-                        if (q.gR == 2) two |= bit;
-                        if (dR == 2 || dL == 2) left |= bit;
-                    }
-                }
-                // ---- draws within the band: FP64
-                if (__any_sync(FULL, left != 0)) {
-                    const View c(a, smem);
-                    for (; left; left &= left - 1) {
-                        const M bit = left & (M(0) - left);
-                        const IonEntry q = ion_entry(c.colp(), first_bit(left), (int)c.slot(kSlotN),
-                                                     c.slot(kSlotGaps), a.rule, t);
-                        int dR = q.fR ? 2 : 0, dL = q.fL ? 2 : 0;
-                        ion_exact<P>(c, c.seg(), c.rail(tile_rail0), q.x,
-                                     min(max(code_of_row((int)(q.e >> 20), a.Z) - 1, 0), a.Z - 1), t, dR, dL);
-                        aR = dR == 1 ? aR | bit : aR & ~bit;
-                        aL = dL == 1 ? aL | bit : aL & ~bit;
-                    }
-                }
-            }
-
-            // ---- moves and the current: both trials accepted, the ion stays; two
-            //      ions entering the site between them are both cancelled
-            bool crossed = false;
-            {
-                const M both = aR & aL;
-                aR ^= both;
-                aL ^= both;
-                if (!__any_sync(FULL, (aR | aL) != 0)) continue;
-                const View c(a, smem);
-                const int n = (int)c.slot(kSlotN), sl = c.sl();
-                const uint32_t gaps = c.slot(kSlotGaps);
-                const M clash = aR & (aL >> 1) & two;
-                aR ^= clash;
-                aL ^= clash << 1;
-                // across lanes: the last entry's hop right and the next lane's first left
-                const int lastR = n > 0 ? (int)(aR >> (n - 1)) & 1 : 0, firstL = (int)aL & 1;
-                const int up = __shfl_up_sync(FULL, lastR, 1, P), dn = __shfl_down_sync(FULL, firstL, 1, P);
-                if (sl > 0 && up && firstL && gap_first(gaps) == 2) aL ^= M(1);
-                if (sl < P - 1 && dn && lastR && gap_last(gaps) == 2) aR ^= M(1) << (n - 1);
-                const int nR = count_bits(aR), nL = count_bits(aL);
-                uint32_t *colp = c.colp();
-                for (M todo = aR | aL; todo; todo &= todo - 1) {
-                    const int j = first_bit(todo);
-                    crossed |= ion_commit<P>(c, tab, colp + j * 32, colp[j * 32], (aR >> j) & 1 ? 1 : -1,
-                                             s + 1 < n_steps ? a.Zc + (t0 + s + 1) * a.Z : nullptr);
-                }
-                c.slot(kSlotMoves) += (uint32_t)(nR + nL);
-                const int Jw = __reduce_add_sync(FULL, nL - nR);
-                if (c.lane() == 0 && Jw != 0) atomicAdd(&a.J[t0 + s], (unsigned long long)(long long)Jw);
-                ion_refresh<P>(c, n, OPEN ? -2 : -1, OPEN ? a.L + 1 : a.L);
-            }
-            if (OPEN) {
-                const View c(a, smem);
-                uint32_t draws = 0u;
-                crossed |= ion_ends<P>(c, tab, s, c.rail(tile_rail0) < a.R, draws);
-                if (draws != 0u && c.lane() == 0) atomicAdd(&a.counters[0], (unsigned long long)draws);
-            }
-            // lanes to rail slots
-            const uint32_t cm = __ballot_sync(FULL, crossed);
-            if (G == 1) dirty = cm != 0u ? 1u : 0u;
-            else
-#pragma unroll
-                for (int q = 0; q < G; ++q)
-                    if ((cm >> (q * P)) & ((1u << (P & 31)) - 1u)) dirty |= 1u << q;
-        }
-        // ---- flush this warp's counters and per-rail current
-        {
-            const View c(a, smem);
-            __syncwarp();
-            const uint32_t nd = __reduce_add_sync(FULL, c.slot(kSlotN)) * (uint32_t)(c1 - c.mark());
-            const uint32_t nv = __reduce_add_sync(FULL, c.slot(kSlotMoves));
-            // a rail's net leftward crossings: the decrease of its positions' sum
-            const int sum = ion_sum<P>(c);
-            __syncwarp();
-            if (c.lane() == 0) {
-                if (nd) atomicAdd(&a.counters[0], (unsigned long long)nd);
-                if (nv) atomicAdd(&a.counters[2], (unsigned long long)nv);
-                c.mark() = c1;
-            }
-            c.slot(kSlotMoves) = 0u;
-            const int64_t rail = c.rail(tile_rail0);
-            if (c.sl() == 0) {
-                const int v = c.Fs()[2 * G] - sum;
-                c.Fs()[2 * G] = sum;
-                if (a.Jr && rail < a.R && v != 0) a.Jr[rail] += v;
-            }
-            __syncwarp();
-        }
-    }
-
-    // ---- write the rails back
-    {
-        const View c(a, smem);
-        ion_to_words<P>(c);
-        const int W = (a.L + 31) >> 5, C = (W + P - 1) / P;
-        const int w0 = min(c.sl() * C, W), w1 = min(w0 + C, W);
-        const uint32_t *words = c.words() + c.seg() * W;
-        const int64_t rail = c.rail(tile_rail0);
-        if (rail < a.R)
-            for (int w = w0; w < w1; ++w) {
-                const uint32_t o = words[w];
-                uint8_t *row = a.occ + rail * a.stride + 32 * w;
-                *(uint4 *)row = unpack16(o & 0xFFFFu);
-                if (32 * w + 16 < a.stride) *(uint4 *)(row + 16) = unpack16(o >> 16);
-            }
-    }
-}
 
 // 4 CTAs of 256 threads per SM (64 registers).  With 5 (48 registers) the
 // replicated 512-site device ran 4-11 % slower, with 3 (80) 4 % slower.
@@ -896,68 +23,24 @@ __global__ void __launch_bounds__(256, 4) ion_kernel(const __grid_constant__ Swe
     ion_tile<P, ACC, OPEN, M>(a, a.rk0, a.rk1, a.t0, a.n_steps, a.flush, tile_rail0, smem);
 }
 
-// The batch's persistent launch of one shape (as sweep_batch_kernel).
-template <int P, bool ACC, bool OPEN, class M>
-__global__ void __launch_bounds__(256, 4) ion_batch_kernel(const __grid_constant__ BatchArgs b, int kind)
-{
-    extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ SweepArgs ia;
-    __shared__ int s_item;
-    const int64_t t0 = *b.t0;
-    const int first = b.cls_off[kind], end = b.cls_off[kind + 1];
-    for (;;) {
-        if (threadIdx.x == 0) s_item = first + (int)atomicAdd(b.work + kind, 1u);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= end) break;
-        const BatchItem it = b.items[item];
-        const uint32_t *src = (const uint32_t *)&b.inst[it.inst];
-        for (int i = threadIdx.x; i < (int)(sizeof(SweepArgs) / 4); i += blockDim.x)
-            ((uint32_t *)&ia)[i] = src[i];
-        __syncthreads();
-        ion_tile<P, ACC, OPEN, M>(ia, b.rk0, b.rk1, t0, b.n_steps, b.flush, it.tile_rail0, smem);
-        __syncthreads();
-    }
-}
-
-// Calls f(lanes per rail, accept path, open electrodes, type of the row bits)
-// for an ion-list kind.
-template <class F>
-cudaError_t with_ions(int kind, bool acc, F &&f)
-{
-    using std::integral_constant;
-    using T = integral_constant<bool, true>;
-    using N = integral_constant<bool, false>;
-    const int k = kind - kWordKinds;
-    const bool open = (k & 1) != 0;
-    auto go = [&](auto p, auto m) {
-        if (acc) return open ? f(p, T(), T(), m) : f(p, T(), N(), m);
-        return open ? f(p, N(), T(), m) : f(p, N(), N(), m);
-    };
-    switch (k >> 1) {
-    case 0: return go(integral_constant<int, 4>(), uint32_t());
-    case 1: return go(integral_constant<int, 8>(), uint32_t());
-    case 2: return go(integral_constant<int, 16>(), uint32_t());
-    case 3: return go(integral_constant<int, 32>(), uint32_t());
-    default: return go(integral_constant<int, 32>(), uint64_t());
-    }
-}
-
 // Slots of a lane's column, two more than the rows its bits can count (one that
 // the draw loop reads ahead, one that an end entry may take before the entries
 // are dealt out again): blocking rails keep their ion counts (at most n_max), an
 // open rail holds at most one entry per site.  0: more rows than bits.
-int ion_rows(int P, int L, bool open, int64_t n_max)
+int ion_rows(int P, int L, bool open, int64_t n_max, int bits)
 {
     const int even = (int)(((open ? (int64_t)L : n_max) + P - 1) / P);   // a lane's even share
-    const int bits = P == 32 ? 64 : 32;
     if (even > bits) return 0;
     return std::min(even + (open ? 2 : 0), even <= 32 ? 32 : bits) + 2;
+}
+int ion_rows(int P, int L, bool open, int64_t n_max)
+{
+    return ion_rows(P, L, open, n_max, P == 32 ? 64 : 32);
 }
 
 }  // namespace
 
-IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap)
+IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, bool grad)
 {
     const uint32_t G = 32u / (uint32_t)P, rows = (uint32_t)Z + (open ? 5u : 1u);
     const uint32_t words = G * (uint32_t)((L + 31) >> 5) * 4u;   // occupancy words, staged in the bounds
@@ -970,7 +53,8 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap)
     y.p0b = y.zf + (persite ? 16u * gz : 0u);
     y.pb = y.p0b + (persite ? (uint32_t)align16(8u * gz) : 0u);
     y.st = y.pb + pz;
-    y.col = y.st + 128u * kIonSlots;
+    y.g = y.st + 128u * kIonSlots;
+    y.col = y.g + (grad ? 2688u + 64u * G + (uint32_t)align16(8u * G * (uint32_t)(Z + 1)) + 48u * gz : 0u);
     y.bytes = y.col + (uint32_t)rcap * 128u;
     return y;
 }
@@ -1024,7 +108,76 @@ size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool per
     if (!t.ions) return sweep_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps, 0, acc);
     a.rcap = t.rcap;
     a.rcpZ = 65536u / (uint32_t)p.n_zones + 1u;
-    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, persite, t.rcap);
+    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, persite, t.rcap, false);
+    return a.iy.tab + (size_t)warps * a.iy.bytes;
+}
+
+// The gradient pass's tile.  An FP64 warp instruction takes the SM's FP64 pipe for
+// 16 cycles whatever the number of lanes at work, so the fewest lanes per rail are
+// the best: a rail's zones then fill the lanes (10 zones on 4 lanes: 10 of 12) and
+// its sums are formed once for 8 rails (65,536 x 512 rails: 56 us a step on 4
+// lanes, 70 on 8, 91 on 16, 155 on 32).  More lanes only where fewer than 1,200
+// warps would be left (4,096 rails: 9.0 us on 4, 7.3 on 8, 6.7 on 16, 11 on 32).
+TileShape pick_grad_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max)
+{
+    TileShape t{};
+    if (L >= 8 && (double)n_tot <= tile_max_fill(true) * (double)n_rails * (double)L) {
+        int P = 32;
+        while (P > 4 && rails * (P / 2) / 32 >= 1200 && ion_rows(P / 2, L, open, n_max, 64) > 0) P >>= 1;
+        t.ions = 1;
+        t.lpr = P;
+        t.rcap = ion_rows(P, L, open, n_max, 64);
+        t.kind = kWordKinds + 2 * (P == 4 ? 0 : P == 8 ? 1 : P == 16 ? 2 : 3) + (open ? 1 : 0);
+        return t;
+    }
+    t.lpr = sweep_pick_lpr(L, &t.wpl);
+    t.kind = sweep_kind(t.lpr, t.wpl);
+    return t;
+}
+
+void grad_smem_limits(size_t *most, size_t *total, bool ions)
+{
+    int dev = 0, cta = 0, sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&cta, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (cta <= 0) cta = 48 * 1024;
+    if (sm < cta) sm = cta;
+    *most = (size_t)std::min(cta, ions ? kGradSmem : 200 * 1024);
+    *total = (size_t)sm;
+}
+
+// Warps per CTA of a shape's gradient launch over `rails` rails: as many resident
+// on an SM as its shared memory (`total` bytes, `most` to a CTA, which costs 1 KB
+// more than it asks for) allows, of equals the smaller CTA; when all warps are
+// resident at once, the same number on every SM (16,384 x 512 rails on 4 lanes,
+// 13.5 warps an SM: 14.4 us a step in one wave of 14, 20.4 us in CTAs of 8).
+int grad_warps(const TileShape &t, const kmc_params &p, size_t most, size_t total, int64_t rails, int sms)
+{
+    SweepArgs a;
+    int best = 1, resident = 0, largest = 1;
+    for (int w = 1; w <= (t.ions ? kGradWarps : 8); ++w) {
+        const size_t m = grad_tile_args(a, t, p, w);
+        if (m > most) break;
+        if (!t.ions && (w & (w - 1))) continue;
+        largest = w;
+        const int n = t.ions ? w * std::min<int>((int)(total / (m + 1024)), kGradWarps / w) : w;
+        if (n > resident) {
+            resident = n;
+            best = w;
+        }
+    }
+    const int64_t even = (rails * t.lpr / 32 + sms - 1) / std::max(1, sms);
+    if (t.ions && even <= std::min(resident, largest)) return (int)std::max<int64_t>(1, even);
+    return best;
+}
+
+size_t grad_tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, int warps)
+{
+    if (!t.ions) return grad_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps);
+    a.rcap = t.rcap;
+    a.rcpZ = 65536u / (uint32_t)p.n_zones + 1u;
+    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, false, t.rcap, true);
     return a.iy.tab + (size_t)warps * a.iy.bytes;
 }
 
@@ -1034,16 +187,14 @@ cudaError_t ion_set_smem_limits()
     for (int k = kWordKinds; k < kShapeKinds; ++k)
         for (int acc = 0; acc < 2; ++acc) {
             const cudaError_t r = with_ions(k, acc != 0, [](auto p, auto ac, auto open, auto m) {
-                constexpr int P = decltype(p)::value;
-                constexpr bool A = decltype(ac)::value, O = decltype(open)::value;
-                const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-                const cudaError_t q = cudaFuncSetAttribute(ion_kernel<P, A, O, decltype(m)>, attr, 200 * 1024);
-                return q != cudaSuccess
-                           ? q : cudaFuncSetAttribute(ion_batch_kernel<P, A, O, decltype(m)>, attr, 200 * 1024);
+                return cudaFuncSetAttribute(
+                    ion_kernel<decltype(p)::value, decltype(ac)::value, decltype(open)::value, decltype(m)>,
+                    cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
             });
             if (r != cudaSuccess) e = r;
         }
-    return e;
+    const cudaError_t b = ion_batch_set_smem_limits(), g = ion_grad_set_smem_limits();
+    return e != cudaSuccess ? e : b != cudaSuccess ? b : g;
 }
 
 cudaError_t ion_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s)
@@ -1053,27 +204,6 @@ cudaError_t ion_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate
             <<<l.grid, l.warps * 32, l.smem, s>>>(a, gate);
         return cudaGetLastError();
     });
-}
-
-cudaError_t ion_batch_launch(const BatchArgs &b, int kind, int grid, int warps, size_t smem, bool acc,
-                             cudaStream_t s)
-{
-    return with_ions(kind, acc, [&](auto p, auto ac, auto open, auto m) {
-        ion_batch_kernel<decltype(p)::value, decltype(ac)::value, decltype(open)::value, decltype(m)>
-            <<<grid, warps * 32, smem, s>>>(b, kind);
-        return cudaGetLastError();
-    });
-}
-
-int ion_batch_ctas_per_sm(int kind, bool acc, int warps, size_t smem)
-{
-    int n = 0;
-    const cudaError_t e = with_ions(kind, acc, [&](auto p, auto ac, auto open, auto m) {
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &n, ion_batch_kernel<decltype(p)::value, decltype(ac)::value, decltype(open)::value, decltype(m)>,
-            warps * 32, smem);
-    });
-    return e == cudaSuccess && n > 0 ? n : 1;
 }
 
 }  // namespace kmc

@@ -193,6 +193,31 @@ __global__ void exp_table_kernel(double cm, int32_t M, double *etL, double *etH,
     if (i < nH) etH[i] = exp(__dmul_rn(cm, (double)((int64_t)i * 1024 - M)));
 }
 
+// The background of a rail of n ions (one thread per n) for the gradient pass:
+// D'_z as background_kernel forms it, and its factor exp(xV kappa alpha D'_z) of
+// B_z, xV = -d / (t_dev kT).
+__global__ void background_by_count_kernel(int32_t L, int32_t Z, const DevConst *K, double2 *out)
+{
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n > L) return;
+    const double xV = -(K->d / K->t_dev) / K->kT;
+    double2 *o = out + (int64_t)n * Z;
+    double run = 0.0, acc = 0.0;
+    for (int z = 0; z < Z; ++z) {
+        const int w = K->bnd[z + 1] - K->bnd[z];
+        const double cz = ((double)n * (double)w) / (double)L;
+        const double D = run + 0.5 * cz;
+        run += cz;
+        acc += (double)w * D;
+        o[z].x = D;
+    }
+    const double mean = acc / (double)L;
+    for (int z = 0; z < Z; ++z) {
+        const double D = o[z].x - mean;
+        o[z] = make_double2(D, exp(__dmul_rn(__dmul_rn(xV, K->ka), D)));
+    }
+}
+
 // Background of each zone of each rail for the FP64 decision paths (one
 // thread per rail): c_z = N0 w_z / L, an exact product rounded once by the
 // division, as the exact path uses it, and D'_z = D_z - sum_z' w_z' D_z' / L
@@ -259,6 +284,12 @@ cudaError_t setup_exp_tables(double cm, int32_t M, double *etL, double *etH, int
 {
     const int n = nH > 1024 ? nH : 1024;
     exp_table_kernel<<<(n + 255) / 256, 256, 0, s>>>(cm, M, etL, etH, nH);
+    return cudaGetLastError();
+}
+
+cudaError_t setup_background_by_count(int32_t L, int32_t Z, const DevConst *K, double2 *out, cudaStream_t s)
+{
+    background_by_count_kernel<<<(unsigned)((L + 256) / 256), 256, 0, s>>>(L, Z, K, out);
     return cudaGetLastError();
 }
 

@@ -371,49 +371,6 @@ __device__ __forceinline__ double trial_weight(int A, int n, double r1, double q
 {
     return __fma_rn(-(double)n, q, __dmul_rn((double)A, r1));
 }
-// Tests on a double's bit pattern, on the integer pipe (FP64 compares take
-// the FP64 pipe, the gradient pass's bottleneck): x != 0 (NaN counts as
-// nonzero, as the FP64 test does), equality of two values that are never NaN
-// (+0 and -0 differ: a stale mark at worst), and lo < x < hi for lo, hi
-// positive and finite (positive doubles order as their bit patterns; negative
-// values and NaN fall outside).
-__device__ __forceinline__ bool nonzero_bits(double x)
-{
-    return ((unsigned long long)__double_as_longlong(x) << 1) != 0ull;
-}
-__device__ __forceinline__ bool same_bits(double x, double y)
-{
-    return __double_as_longlong(x) == __double_as_longlong(y);
-}
-__device__ __forceinline__ bool inside_bits(double x, double lo, double hi)
-{
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-    const unsigned long long l = (unsigned long long)__double_as_longlong(lo);
-    const unsigned long long h = (unsigned long long)__double_as_longlong(hi);
-    return u - (l + 1ull) < h - (l + 1ull);
-}
-
-// 1 / d for d > 0 (normal, finite) by Newton-Raphson on f(r) = 1/r - d from the
-// hardware approximation (rcp.approx.ftz.f64, about 2^-22 relative): each
-// step r <- r + r (1 - d r) squares the relative error, so two give full FP64
-// accuracy up to a few ulp, enough for score weights.
-__device__ __forceinline__ double recip_newton(double d)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = __fma_rn(-d, r, 1.0);
-    r = __fma_rn(r, e, r);
-    e = __fma_rn(-d, r, 1.0);
-    return __fma_rn(r, e, r);
-}
-
-// Score weight of one electrode trial of probability p, outcome hit, with
-// r1 = 1 / (1 - p) (0 when p >= 1)
-__device__ __forceinline__ double et_weight(int hit, double p, double r1)
-{
-    if (p >= 1.0) return (double)hit;
-    return __fma_rn(-1.0, __dmul_rn(p, r1), __dmul_rn((double)hit, r1));
-}
 // r1 and q of a trial of probability p (cached for inner trials)
 __device__ __forceinline__ double2 trial_factors(double p, double r1_if_uncertain)
 {
@@ -1662,13 +1619,18 @@ cudaError_t with_shape(int k, F &&f)
     }
 }
 
-cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, int warps, cudaStream_t s)
+cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, cudaStream_t s)
 {
-    for (int k = 0; k < kWordKinds; ++k) {
+    for (int k = 0; k < kShapeKinds; ++k) {
         if (plan.grid[k] <= 0) continue;
+        if (k >= kWordKinds) {
+            const cudaError_t e = ion_batch_grad_launch(b, k, plan.grid[k], plan.warps[k], plan.smem[k], s);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
         const cudaError_t e = with_shape(k, [&](auto lpr, auto wpl) {
             constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
-            sweep_batch_grad_kernel<P, Q><<<plan.grid[k], warps * 32, plan.smem[k], s>>>(b);
+            sweep_batch_grad_kernel<P, Q><<<plan.grid[k], plan.warps[k] * 32, plan.smem[k], s>>>(b);
             return cudaGetLastError();
         });
         if (e != cudaSuccess) return e;
@@ -1678,7 +1640,7 @@ cudaError_t batch_grad_launch(const BatchArgs &b, const BatchPlan &plan, int war
 
 int batch_ctas_per_sm(int kind, int mode, int warps, size_t smem)
 {
-    if (kind >= kWordKinds) return ion_batch_ctas_per_sm(kind, mode == 1, warps, smem);
+    if (kind >= kWordKinds) return ion_batch_ctas_per_sm(kind, mode, warps, smem);
     int n = 0;
     const cudaError_t e = with_shape(kind, [&](auto lpr, auto wpl) {
         constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
