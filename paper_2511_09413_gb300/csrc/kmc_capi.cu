@@ -54,6 +54,20 @@ void kmc::kmc_internal_set_error(const char *msg) { g_err = msg ? msg : ""; }
 
 namespace {
 
+// Makes the pages of an output buffer present before the device writes them.  A
+// freshly allocated buffer has none, and on a host whose memory the GPU reaches
+// through the host's page tables the copy then takes a fault per page on the
+// GPU's side: 65,536 x 1,024 occupancy bytes took 59 ms into fresh pages and
+// 0.5 ms into present ones, with 2.4 ms for touching them here, while the sweep
+// that was queued before is still running.  The buffer is written in full later.
+void touch_pages(void *p, size_t bytes)
+{
+    constexpr size_t kPage = 4096;      // the smallest page
+    volatile char *c = (volatile char *)p;
+    for (size_t i = 0; i < bytes; i += kPage) c[i] = 0;
+    if (bytes > 0) c[bytes - 1] = 0;
+}
+
 bool finite_pos(double x) { return isfinite(x) && x > 0.0; }
 
 int validate(const kmc_params *p, const double *V, int64_t n_total, const uint8_t *occ0)
@@ -618,18 +632,24 @@ int kmc_observables(kmc_handle *h, int64_t first_step, int64_t count, int64_t *J
         return fail(KMC_E_RANGE, "steps [%lld, %lld) not simulated yet (current step %lld)",
                     (long long)first_step, (long long)(first_step + count), (long long)h->t);
     cudaStream_t s = h->stream;
+    const int64_t Z = h->p.n_zones, L = h->p.n_sites, R = h->p.n_rails;
+    if (J_out) touch_pages(J_out, sizeof(int64_t) * (size_t)count);
+    if (zone_counts_out) touch_pages(zone_counts_out, sizeof(int64_t) * (size_t)(count * Z));
+    if (occ_out_or_null) touch_pages(occ_out_or_null, (size_t)(R * L));
     if (count > 0 && J_out)
         CK(cudaMemcpyAsync(J_out, h->J + first_step, sizeof(int64_t) * (size_t)count,
                            cudaMemcpyDeviceToHost, s),
            "copy J");
     if (count > 0 && zone_counts_out)
-        CK(cudaMemcpyAsync(zone_counts_out, h->Zc + first_step * h->p.n_zones,
-                           sizeof(int64_t) * (size_t)count * (size_t)h->p.n_zones,
+        CK(cudaMemcpyAsync(zone_counts_out, h->Zc + first_step * Z, sizeof(int64_t) * (size_t)(count * Z),
                            cudaMemcpyDeviceToHost, s),
            "copy zone counts");
-    if (occ_out_or_null)
-        CK(cudaMemcpy2DAsync(occ_out_or_null, (size_t)h->p.n_sites, h->occ, (size_t)h->stride,
-                             (size_t)h->p.n_sites, (size_t)h->p.n_rails, cudaMemcpyDeviceToHost, s),
+    if (occ_out_or_null && h->stride == L)      // rows without padding: one block
+        CK(cudaMemcpyAsync(occ_out_or_null, h->occ, (size_t)(R * L), cudaMemcpyDeviceToHost, s),
+           "copy occupancy");
+    else if (occ_out_or_null)
+        CK(cudaMemcpy2DAsync(occ_out_or_null, (size_t)L, h->occ, (size_t)h->stride, (size_t)L, (size_t)R,
+                             cudaMemcpyDeviceToHost, s),
            "copy occupancy");
     CK(cudaStreamSynchronize(s), "observables");
     return KMC_OK;
@@ -638,6 +658,7 @@ int kmc_observables(kmc_handle *h, int64_t first_step, int64_t count, int64_t *J
 int kmc_rail_current(kmc_handle *h, int64_t *J_rail_out)
 {
     if (!h || !J_rail_out) return fail(KMC_E_ARG, "handle or J_rail_out is NULL");
+    touch_pages(J_rail_out, sizeof(int64_t) * (size_t)h->p.n_rails);
     CK(cudaMemcpyAsync(J_rail_out, h->Jr, sizeof(int64_t) * (size_t)h->p.n_rails,
                        cudaMemcpyDeviceToHost, h->stream),
        "copy per-rail current");
