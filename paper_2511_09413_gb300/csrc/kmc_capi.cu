@@ -151,6 +151,7 @@ int pick_launch(kmc_handle *h)
     max_smem = std::min(max_smem, 200 * 1024);
     auto smem_for = [&](int w) { return tile_args(h->args, t, p, h->P0site != nullptr, w, l.acc != 0); };
     while (warps > 1 && smem_for(warps) > (size_t)max_smem) warps >>= 1;
+    if (t.ions && h->warps_req <= 0) warps = ion_cta_warps(h->args, (p.n_rails * (int64_t)t.lpr + 31) / 32, warps);
     l.warps = warps;
     l.smem = smem_for(warps);
     const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * warps;
@@ -184,6 +185,7 @@ void fill_args(kmc_handle *h)
     a.P0site = h->P0site;
     a.P0f = h->P0f;
     a.P0bnd = h->P0bnd;
+    a.P0cls = h->P0bnd ? (const uint32_t *)(h->P0bnd + (int64_t)p.n_rails * p.n_zones) : nullptr;
     a.bgd = h->bgd;
     a.K = h->K;
     a.self = h->args_dev;
@@ -302,7 +304,8 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
     if (Ea) {
         h->P0site = (double *)h->alloc(sizeof(double) * (size_t)(R * L));
         h->P0f = (float *)h->alloc(sizeof(float) * (size_t)(R * L));
-        h->P0bnd = (float2 *)h->alloc(sizeof(float2) * (size_t)(R * Z));
+        // the classes of the sites follow the bounds of the zones
+        h->P0bnd = (float2 *)h->alloc(sizeof(float2) * (size_t)(R * Z) + sizeof(uint32_t) * (size_t)(R * ((L + 15) / 16)));
         if (!h->P0site || !h->P0f || !h->P0bnd)
             return fail(KMC_E_NOMEM, "device allocation failed (P0 table)");
     }
@@ -344,6 +347,8 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         CK(setup_p0_bounds(h->P0site, (int32_t)R, (int32_t)L, (int32_t)Z, h->K, h->P0bnd, s),
            "P0 bounds");
         CK(setup_p0_float(h->P0site, R * L, h->P0f, s), "P0 float table");
+        CK(setup_p0_classes(h->P0f, h->P0bnd, R, (int32_t)L, (int32_t)Z, h->K, (uint32_t *)(h->P0bnd + R * Z), s),
+           "P0 classes");
     }
     // check derived values
     DevConst kc;

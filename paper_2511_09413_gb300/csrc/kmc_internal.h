@@ -37,10 +37,10 @@ struct DevConst {
 struct IonLayout {
     uint32_t tab;     // the site table, uint4 [L + 2]
     uint32_t row;     // one rail's decision bounds (after the block's fixed part)
-    uint32_t zf;      // float4 [G][Z]: B/(1+B), 1/(1+B), band factors (per-site barriers)
     uint32_t p0b;     // float2 [G][Z]: per-site P0 bounds of the zone (per-site barriers)
     uint32_t pb;      // int [G][Z + 1]: ions below each zone boundary
     uint32_t st;      // uint32 [slots][32]: each lane's state words
+    uint32_t hit;     // uint32 [4 or 8][32]: outcome bits of the steps drawn ahead (no accept path)
     uint32_t g;       // gradient pass: its sums, counts and factors (IonView)
     uint32_t col;     // uint32 [rcap][32]: each lane's entries
     uint32_t bytes;   // one warp's block
@@ -62,6 +62,8 @@ struct SweepArgs {
     const double *P0site;      // [R][L] or null
     const float *P0f;          // [R][L] P0site rounded to FP32, or null
     const float2 *P0bnd;       // [R][Z] (min, max) of P0site over the zone, or null
+    const uint32_t *P0cls;     // [R][(L + 15) / 16] classes of P0f against the zone's max, 2 bits a site
+    int32_t cls_shift;         // ion lists: 2 with classes, else 0
     const double2 *bgd;        // [R][Z] (N0 w_z / L, D'_z) in FP64 for the FP64 paths, or null
     const DevConst *K;
     const SweepArgs *self;     // copy of these arguments in device memory (rare paths)
@@ -84,6 +86,10 @@ struct SweepArgs {
     int32_t rule;                 // 0 synchronous update, 1 brick-wall (even/odd bonds)
     int32_t rcap;                 // ion lists: rows of a lane's column
     uint32_t rcpZ;                // ion lists: i / Z = (i rcpZ) >> 16 for i < 1024
+    // ion lists without the accept path: room in the exponent of the bounds, the
+    // boundary crossings that fit in it, and what an exchange with an electrode counts
+    float ion_slack;
+    int32_t ion_budget, ion_exchange;
     IonLayout iy;                 // ion lists: shared memory
 
     // likelihood-ratio gradient pass only (unused by the forward sweep)
@@ -206,6 +212,7 @@ TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_
 // filling of the sites up to which the ion lists are the better tile
 float tile_max_fill(bool acc);
 // sets a.rcap and a.iy for the tile; shared memory of a CTA of `warps` warps
+int ion_cta_warps(const SweepArgs &a, int64_t warps, int most);
 size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool persite, int warps, bool acc);
 // the batch's kernels of ion-list kinds
 cudaError_t ion_batch_launch(const BatchArgs &b, int kind, int grid, int warps, size_t smem, bool acc,
@@ -256,6 +263,8 @@ cudaError_t setup_p0_table(const kmc_params &p, const double *Ea, double *P0, in
                            cudaStream_t s);
 cudaError_t setup_p0_bounds(const double *P0, int32_t R, int32_t L, int32_t Z, const DevConst *K,
                             float2 *out, cudaStream_t s);
+cudaError_t setup_p0_classes(const float *P0f, const float2 *bnd, int64_t R, int32_t L, int32_t Z, const DevConst *K,
+                             uint32_t *out, cudaStream_t s);
 cudaError_t setup_p0_float(const double *P0, int64_t n, float *out, cudaStream_t s);
 // ions of each rail; with stats, also their total (stats[0]) and the largest (stats[1])
 cudaError_t setup_row_counts(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,

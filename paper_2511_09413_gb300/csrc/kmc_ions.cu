@@ -40,20 +40,20 @@ int ion_rows(int P, int L, bool open, int64_t n_max)
 
 }  // namespace
 
-IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, bool grad)
+IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, bool grad, bool ahead)
 {
-    const uint32_t G = 32u / (uint32_t)P, rows = (uint32_t)Z + (open ? 5u : 1u);
+    const uint32_t G = 32u / (uint32_t)P, rows = ((uint32_t)Z << (persite && ahead ? 2 : 0)) + (open ? 5u : 1u);
     const uint32_t words = G * (uint32_t)((L + 31) >> 5) * 4u;   // occupancy words, staged in the bounds
     const uint32_t gz = G * (uint32_t)Z;
     const uint32_t pz = (uint32_t)align16(4u * G * (uint32_t)(Z + 1));
     IonLayout y;
     y.tab = 16u * (uint32_t)(L + 2);
     y.row = rows * 16u;
-    y.zf = ion_fixed(P) + (uint32_t)align16(std::max(G * y.row, words));
-    y.p0b = y.zf + (persite ? 16u * gz : 0u);
+    y.p0b = ion_fixed(P) + (uint32_t)align16(std::max(G * y.row, words));
     y.pb = y.p0b + (persite ? (uint32_t)align16(8u * gz) : 0u);
     y.st = y.pb + pz;
-    y.g = y.st + 128u * kIonSlots;
+    y.hit = y.st + 128u * kIonSlots;
+    y.g = y.hit + (ahead ? 128u * kIonAhead * (rcap > 34 ? 2u : 1u) : 0u);
     y.col = y.g + (grad ? 2688u + 64u * G + (uint32_t)align16(8u * G * (uint32_t)(Z + 1)) + 48u * gz : 0u);
     y.bytes = y.col + (uint32_t)rcap * 128u;
     return y;
@@ -103,13 +103,61 @@ TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_
     return t;
 }
 
+// One ion crossing boundary b changes P_b by one, so Q_b-1 and Q_b by a half and
+// their mean by at most that much: no zone's Q_z - Qbar moves by more than a half,
+// its exponent by |kappa alpha| / (2 L kT).  Exchanges with an electrode alternate
+// in and out as long as the list keeps its entries, so they shift a rail by one at
+// each end and are not counted; where that leaves no room they are.  Room for ten
+// crossings, at most 0.25 (a fifth more draws to look at), at least 0.05.
+static void ion_slack(SweepArgs &a, bool open)
+{
+    const double per = 0.505 * fabs((double)a.ka_f) * (double)a.inv_LkT;
+    const double slack = std::min(0.25, std::max(0.05, 10.0 * per));
+    a.ion_slack = (float)slack;
+    const int fits = per * 1000.0 < 0.99 * slack ? 1000 : (int)floor(0.99 * slack / per);
+    a.ion_exchange = open && fits < 4 ? 1 : 0;
+    a.ion_budget = open && fits >= 4 ? fits - 2 : fits;
+}
+
 size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool persite, int warps, bool acc)
 {
     if (!t.ions) return sweep_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps, 0, acc);
     a.rcap = t.rcap;
     a.rcpZ = 65536u / (uint32_t)p.n_zones + 1u;
-    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, persite, t.rcap, false);
+    ion_slack(a, p.electrodes == 1);
+    a.cls_shift = persite && !acc ? 2 : 0;
+    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, persite, t.rcap, false, !acc);
     return a.iy.tab + (size_t)warps * a.iy.bytes;
+}
+
+// Warps per CTA (at most `most`) of a launch over `warps` warps.  When all are
+// resident at once the launch takes as long as the fullest SM sub-partition: the
+// CTA size that leaves it the fewest warps, of equals the largest (4,000 warps of
+// 16,000 x 200 rails: 8 to a sub-partition and 2.94 ms in CTAs of 8, 7 and 2.60 ms
+// in CTAs of 7; 64 warps: 2 and 0.41 ms in CTAs of 8, 1 and 0.36 ms in CTAs of 4).
+// In more than one wave `most` (16,384 x 1,024: 6.8 ms in CTAs of 8, 6.8 of 4, 7.6
+// of 2, which repeat the site table more often).
+int ion_cta_warps(const SweepArgs &a, int64_t warps, int most)
+{
+    int dev = 0, sms = 0, sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    sms = std::max(sms, 1);
+    int best = most;
+    int64_t least = INT64_MAX;
+    for (int w = most; w >= 1; --w) {
+        const size_t smem = a.iy.tab + (size_t)w * a.iy.bytes + 1024;     // the system's 1 KB a CTA
+        const int64_t resident = std::min<int64_t>(32 / w, (int64_t)((size_t)std::max(sm, 1) / smem));
+        const int64_t per_sm = ((warps + w - 1) / w + sms - 1) / sms;
+        if (per_sm > resident) continue;
+        const int64_t fullest = (per_sm * w + 3) / 4;
+        if (fullest < least) {
+            least = fullest;
+            best = w;
+        }
+    }
+    return best;
 }
 
 // The gradient pass's tile.  An FP64 warp instruction takes the SM's FP64 pipe for
@@ -177,7 +225,7 @@ size_t grad_tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, int
     if (!t.ions) return grad_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps);
     a.rcap = t.rcap;
     a.rcpZ = 65536u / (uint32_t)p.n_zones + 1u;
-    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, false, t.rcap, true);
+    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, false, t.rcap, true, false);
     return a.iy.tab + (size_t)warps * a.iy.bytes;
 }
 

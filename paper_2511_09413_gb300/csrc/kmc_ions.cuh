@@ -96,19 +96,18 @@ __device__ __forceinline__ void site_draw(const StepDraw &d, uint32_t w0, uint32
 // The site table (per CTA, one uint4 per position -1 .. L): the three words of
 // site_words, and the position's entry, as the lists hold it: 16 times
 // (position + 1), its own byte offset in the table, in the low 16 bits, above
-// them the byte offset of its row of decision bounds.  Rows: one per zone, of
-// an open rail four more for positions -1, 0, L - 1, L, and a dead row (nothing
-// accepted) for the unused slots of a column.  Looking the words up takes two of
+// them the byte offset of its row of decision bounds.  Rows: one per zone, or four
+// with per-site barriers (2^cls_shift), of an open rail four more for positions
+// -1, 0, L - 1, L, and a dead row (nothing accepted) for the unused slots of a
+// column.  With per-site barriers the table holds a zone's first row and an ion's
+// entry adds the class of its site: P0 within a half, a quarter, an eighth of the
+// zone's largest one or below.  At a spread of 20 meV the largest of a zone's 100
+// sites is five times the mean, so bounds of whole zones let through six draws to
+// look at for each that is accepted, those of classes 1.5.  Looking the words up takes two of
 // the draw's 16 widening multiplies off the pipe that bounds the loop.
 constexpr int kStep = 16;          // an entry's difference between neighbouring positions
 __device__ __forceinline__ int pos_of(uint32_t e) { return (int)((e & 0xFFFFu) / kStep) - 1; }
 __device__ __forceinline__ uint4 site_at(const uint8_t *tab, uint32_t e) { return *(const uint4 *)(tab + (e & 0xFFFFu)); }
-// zone code of a row: z + 1, and 0 / Z + 1 for the virtual sites -1 / L
-__device__ __forceinline__ int code_of_row(int row, int Z)
-{
-    return row < Z ? row + 1 : (row < Z + 2 ? row - Z : (row == Z + 2 ? Z : Z + 1));
-}
-
 // A warp's block: header of 64 bytes (band factor and mid voltage of the voltage
 // window float [2], the largest column, the step up to which draws are counted;
 // in the gradient pass the doubles of IonScore from byte 24 on),
@@ -121,6 +120,7 @@ __host__ __device__ constexpr uint32_t ion_fixed(int P) { return kIonHead + (uin
 // (high half), on the neighbouring lanes or the rail's ends; moves since the
 // last flush
 enum { kSlotN = 0, kSlotGaps = 1, kSlotMoves = 2, kIonSlots = 3 };
+constexpr int kIonAhead = 4;       // steps drawn for at once without the accept path
 
 // The thread index, read anew.  Each phase of a step forms its addresses from
 // it and takes its state from shared memory, so that no phase's registers are
@@ -132,8 +132,10 @@ __device__ __forceinline__ uint32_t tid_here()
     asm volatile("mov.u32 %0, %%tid.x;" : "=r"(v));
     return v;
 }
-// A lane's view of its warp's shared memory.
-template <int P>
+// A lane's view of its warp's shared memory.  CLS: with per-site barriers the rows
+// of bounds distinguish classes of sites (without the accept path: with it the look
+// for a moved ion's class cost the replicated 512-site device 8 %).
+template <int P, bool CLS>
 struct IonView {
     static constexpr int G = 32 / P;
     const SweepArgs &a;
@@ -148,6 +150,26 @@ struct IonView {
     __device__ __forceinline__ int seg() const { return (int)(tid & 31u) / P; }
     __device__ __forceinline__ int sl() const { return (int)(tid & (P - 1)); }
     __device__ __forceinline__ int64_t rail(int64_t tile_rail0) const { return tile_rail0 + (int64_t)(tid >> 5) * G + seg(); }
+    __device__ __forceinline__ int cls() const { return CLS ? a.cls_shift : 0; }
+    // zone code of an entry: z + 1, and 0 / Z + 1 for the virtual sites -1 / L
+    __device__ __forceinline__ int code(uint32_t e) const
+    {
+        const int row = (int)(e >> 20), q = row - (a.Z << cls());
+        return q < 0 ? (row >> cls()) + 1 : (q < 2 ? q : a.Z + q - 2);
+    }
+    __device__ __forceinline__ int zone(uint32_t e) const { return min(max(code(e) - 1, 0), a.Z - 1); }
+    // rows of the ends of an open rail
+    __device__ __forceinline__ uint8_t *end_rows(int sg) const { return bounds(sg) + (a.Z << cls()) * 16; }
+    // the entry at 16 (x + 1) of the site table for an ion of `rail`
+    __device__ __forceinline__ uint32_t entry(const uint8_t *tab, uint32_t at, int64_t rail) const
+    {
+        uint32_t e = site_at(tab, at).w;
+        if (cls() != 0 && (int)(e >> 20) < a.Z << cls()) {
+            const int x = pos_of(at);
+            e += ((__ldg(a.P0cls + rail * ((a.L + 15) >> 4) + (x >> 4)) >> (2 * (x & 15))) & 3u) << 20;
+        }
+        return e;
+    }
     __device__ __forceinline__ float4 &band() const { return *(float4 *)sb; }
     __device__ __forceinline__ int &kmax() const { return *(int *)(sb + 16); }
     __device__ __forceinline__ int &mark() const { return *(int *)(sb + 20); }
@@ -157,10 +179,12 @@ struct IonView {
     __device__ __forceinline__ uint8_t *bounds(int sg) const { return sb + ion_fixed(P) + sg * (int)a.iy.row; }
     __device__ __forceinline__ uint8_t *bounds() const { return bounds(seg()); }
     __device__ __forceinline__ uint32_t *words() const { return (uint32_t *)(sb + ion_fixed(P)); }
-    __device__ __forceinline__ float4 *zf(int sg) const { return (float4 *)(sb + a.iy.zf) + sg * a.Z; }
     __device__ __forceinline__ float2 *p0b(int sg) const { return (float2 *)(sb + a.iy.p0b) + sg * a.Z; }
     __device__ __forceinline__ int32_t *Pb(int sg) const { return (int32_t *)(sb + a.iy.pb) + sg * (a.Z + 1); }
     __device__ __forceinline__ uint32_t &slot(int k) const { return ((uint32_t *)(sb + a.iy.st))[k * 32 + lane()]; }
+    // without the accept path: rows that may be accepted, per step drawn ahead
+    // (kIonAhead words, as many again for the rows from 32 on)
+    __device__ __forceinline__ uint32_t &hits(int k) const { return ((uint32_t *)(sb + a.iy.hit))[k * 32 + lane()]; }
     __device__ __forceinline__ uint32_t *col() const { return (uint32_t *)(sb + a.iy.col); }
     __device__ __forceinline__ uint32_t *colp() const { return col() + lane(); }
     // gradient pass: [0] V of the cached probabilities, [1] exp(xV V), [2] xV:
@@ -227,8 +251,8 @@ __device__ __forceinline__ IonEntry ion_entry(const uint32_t *colp, int j, int n
 
 // A draw within the FP32 band of its probability: the FP64 band, then the exact
 // path.  d* in: 2 for a trial to decide, else 0 or 1; out: 0 or 1.
-template <int P>
-__device__ __forceinline__ void ion_exact(const IonView<P> &c, int sg, int64_t r2, int pos, int zone,
+template <int P, bool CLS>
+__device__ __forceinline__ void ion_exact(const IonView<P, CLS> &c, int sg, int64_t r2, int pos, int zone,
                                           uint32_t t, int &dR, int &dL)
 {
     constexpr int G = 32 / P;
@@ -296,8 +320,8 @@ __device__ __forceinline__ void ion_exact(const IonView<P> &c, int sg, int64_t r
 
 // Distances across the lanes of a rail, for the columns as they stand (n entries
 // on this lane).  wallL, wallR: the positions beyond a rail's ends.
-template <int P>
-__device__ __forceinline__ void ion_refresh(const IonView<P> &c, int n, int wallL, int wallR)
+template <int P, bool CLS>
+__device__ __forceinline__ void ion_refresh(const IonView<P, CLS> &c, int n, int wallL, int wallR)
 {
     const uint32_t *colp = c.colp();
     const int xF = n > 0 ? pos_of(colp[0]) : wallR;
@@ -311,8 +335,8 @@ __device__ __forceinline__ void ion_refresh(const IonView<P> &c, int n, int wall
 // Deals a warp's entries out evenly from the occupancy words (staged where the
 // bounds are): M / P to a lane and one more to the first M % P lanes; the other
 // slots are dead.  Sets the lane's state words and the largest column.
-template <int P, bool OPEN>
-__device__ __forceinline__ void ion_build(const IonView<P> &c, const uint8_t *tab, bool active)
+template <int P, bool OPEN, bool CLS>
+__device__ __forceinline__ void ion_build(const IonView<P, CLS> &c, const uint8_t *tab, int64_t rail)
 {
     const SweepArgs &a = c.a;
     const int L = a.L, W = (L + 31) >> 5, C = (W + P - 1) / P, sl = c.sl();
@@ -331,7 +355,7 @@ __device__ __forceinline__ void ion_build(const IonView<P> &c, const uint8_t *ta
     }
     const int total = __shfl_sync(FULL, incl, P - 1, P);
     int vl = 0, vr = 0;
-    if (OPEN && active) {
+    if (OPEN && rail < a.R) {
         vl = (words[0] & 1u) ? 0 : 1;
         vr = ((words[(L - 1) >> 5] >> ((L - 1) & 31)) & 1u) ? 0 : 1;
     }
@@ -349,7 +373,7 @@ __device__ __forceinline__ void ion_build(const IonView<P> &c, const uint8_t *ta
             r = i2 - l * base;
             l += rem;
         }
-        col[r * 32 + c.seg() * P + l] = site_at(tab, (uint32_t)xb * kStep).w;
+        col[r * 32 + c.seg() * P + l] = c.entry(tab, (uint32_t)xb * kStep, rail);
     };
     int i = incl - cnt + vl;
     for (int w = w0; w < w1; ++w) {
@@ -372,8 +396,8 @@ __device__ __forceinline__ void ion_build(const IonView<P> &c, const uint8_t *ta
 }
 
 // The sum of the positions of a rail's entries (on all of its lanes).
-template <int P>
-__device__ __forceinline__ int ion_sum(const IonView<P> &c)
+template <int P, bool CLS>
+__device__ __forceinline__ int ion_sum(const IonView<P, CLS> &c)
 {
     const uint32_t *colp = c.colp();
     const int n = (int)c.slot(kSlotN);
@@ -385,8 +409,8 @@ __device__ __forceinline__ int ion_sum(const IonView<P> &c)
 }
 
 // The occupancy words of the lists (staged where the bounds are).
-template <int P>
-__device__ __forceinline__ void ion_to_words(const IonView<P> &c)
+template <int P, bool CLS>
+__device__ __forceinline__ void ion_to_words(const IonView<P, CLS> &c)
 {
     const int L = c.a.L, W = (L + 31) >> 5;
     uint32_t *words = c.words();
@@ -405,17 +429,18 @@ __device__ __forceinline__ void ion_to_words(const IonView<P> &c)
 // Entry e at *at moves by m: its new entry, and when it crosses a zone boundary
 // b the counts P_b and F, which lose (rightward) or gain one ion, and the zone
 // counts of the next step, zc[b - 1] and zc[b] (null after the launch's last
-// step).  Returns whether it crossed one.
-template <int P>
-__device__ __forceinline__ bool ion_commit(const IonView<P> &c, const uint8_t *tab, uint32_t *at, uint32_t e,
-                                           int m, unsigned long long *zc)
+// step).  Returns 0 when it crossed none, 1 for a boundary inside the rail, 2 for
+// an end of the rail (an exchange with an electrode).
+template <int P, bool CLS>
+__device__ __forceinline__ int ion_commit(const IonView<P, CLS> &c, const uint8_t *tab, int64_t rail, uint32_t *at,
+                                          uint32_t e, int m, unsigned long long *zc)
 {
     const SweepArgs &a = c.a;
-    const uint32_t en = site_at(tab, (e & 0xFFFFu) + (uint32_t)(kStep * m)).w;
+    const uint32_t en = c.entry(tab, (e & 0xFFFFu) + (uint32_t)(kStep * m), rail);
     *at = en;
-    if (((e ^ en) >> 16) == 0u) return false;
-    const int k0 = code_of_row((int)(e >> 20), a.Z), k1 = code_of_row((int)(en >> 20), a.Z);
-    if (k0 == k1) return false;
+    if (((e ^ en) >> 16) == 0u) return 0;
+    const int k0 = c.code(e), k1 = c.code(en);
+    if (k0 == k1) return 0;
     const int b = max(k0, k1) - 1;
     atomicAdd(&c.Pb(c.seg())[b], -m);
     atomicAdd(c.Fs(), -m * a.wsum[b]);
@@ -423,130 +448,317 @@ __device__ __forceinline__ bool ion_commit(const IonView<P> &c, const uint8_t *t
         if (b > 0) atomicAdd(zc + (b - 1), (unsigned long long)(long long)(-m));
         if (b < a.Z) atomicAdd(zc + b, (unsigned long long)(long long)m);
     }
-    return true;
+    return b == 0 || b == a.Z ? 2 : 1;
 }
 
-// The field of S2.1.8, Eqs. 3-6 and the decision bounds of the zones of the rail
-// slots in `dirty` (bits), for step s.  Bounds: p lies within a factor 1 +- eps
-// of its FP32 value, times [1 / eh, eh] over a voltage window.  With u = 2^-24,
-// every one of the twelve roundings that lead to the exponent x is relative to
-// at most S = (|V| + |kappa alpha| (P_z + P_z+1 + F / L + N0)) / (L kT), so x is
-// off by less than 16 u S, and Eqs. 5-6 move by that relatively (their
-// logarithmic derivatives with respect to x are at most 1); __expf adds
-// (2 + 1.2 |x|) ulp, the division two, the other operations three.
-template <int P, bool OPEN>
-__device__ __forceinline__ void ion_zones(const IonView<P> &c, int64_t t0, int s, int n_steps, bool window,
-                                          uint32_t dirty, int &wend)
+// Zone z of rail slot sg as it stands (the field of S2.1.8, Eqs. 3-4) at the mid
+// voltage of the window: B/(1+B) and 1/(1+B) in FP32 and the factors [lo, hi]
+// that enclose the exact probabilities.  p lies within a factor 1 +- eps of its
+// FP32 value, times [1 / eh, eh] over a voltage window.  With u = 2^-24, every one
+// of the twelve roundings that lead to the exponent x is relative to at most
+// S = (|V| + |kappa alpha| (P_z + P_z+1 + F / L + N0)) / (L kT), so x is off by
+// less than 16 u S, and Eqs. 5-6 move by that relatively (their logarithmic
+// derivatives with respect to x are at most 1); __expf adds (2 + 1.2 |x|) ulp, the
+// division two, the other operations three.
+struct IonZone {
+    float sR, inv, lo, hi;
+    bool ok;        // false: no bounds, every draw goes to the FP64 paths
+};
+template <int P, bool OPEN, bool CLS>
+__device__ __forceinline__ IonZone ion_zone(const IonView<P, CLS> &c, int sg, int z)
 {
-    constexpr int VWIN = 32;              // steps per voltage window of the bounds
+    constexpr int G = 32 / P;
+    const SweepArgs &a = c.a;
+    const float eh = c.band().x, Vf = c.band().y;
+    const int32_t *Pb = c.Pb(sg), *Fs = c.Fs(sg);
+    // an open rail's counts are relative to its first boundary
+    const int p0 = OPEN ? Pb[0] : 0;
+    const int Pz = Pb[z] - p0, Pz1 = Pb[z + 1] - p0;
+    const int F = OPEN ? (int)((uint32_t)Fs[0] - (uint32_t)p0 * (uint32_t)(2 * a.L)) : Fs[0];
+    const float Ff = (float)F * a.inv_L, Nf = (float)Fs[G], Pf = (float)(Pz + Pz1);
+    const float qd = 0.5f * (Pf - Ff) - Nf * a.cz[z];
+    const float x = -(Vf - a.ka_f * qd) * a.inv_LkT;
+    const float S = (fabsf(Vf) + fabsf(a.ka_f) * (Pf + Ff + Nf)) * a.inv_LkT;
+    const float eps = 4e-6f + 5e-7f * fabsf(x) + 1.2e-6f * S;
+    IonZone r{0.0f, 0.0f, 0.0f, 0.0f, fabsf(x) <= 40.0f && eps < 0.25f};
+    if (r.ok) {
+        const float B = __expf(x);
+        r.inv = __fdividef(1.0f, 1.0f + B);
+        r.sR = r.inv * B;
+        r.lo = __fdividef(1.0f - eps, eh);
+        r.hi = (1.0f + eps) * eh;
+    }
+    return r;
+}
+
+// A voltage window: steps from s on, at most 32, whose voltage stays near the
+// first one's.  Evaluating at the window's mid voltage changes B/(1+B) and
+// 1/(1+B) by a factor within [e^-h, e^h] (logarithmic derivatives at most 1); a
+// jump (a pulse's edge) would widen the bounds by several per cent for all of the
+// window's steps, so it starts the next one.  Returns the first step after it.
+template <int P, bool CLS>
+__device__ __forceinline__ int ion_window(const IonView<P, CLS> &c, int64_t t0, int s, int n_steps)
+{
+    const SweepArgs &a = c.a;
+    const int left = min(32, n_steps - s);
+    const double v = a.V[t0 + s + min(c.lane(), left - 1)];
+    const float v0 = __shfl_sync(FULL, (float)v, 0);
+    const uint32_t far = __ballot_sync(FULL, fabsf((float)v - v0) * a.inv_LkT > 2e-3f);
+    const int len = min(left, far ? __ffs(far) - 1 : 32);
+    float vlo = __double2float_rd(v), vhi = __double2float_ru(v);
+    if (c.lane() >= len) vlo = vhi = v0;
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+        vlo = fminf(vlo, __shfl_xor_sync(FULL, vlo, off));
+        vhi = fmaxf(vhi, __shfl_xor_sync(FULL, vhi, off));
+    }
+    const float h = 0.5f * (vhi - vlo) * a.inv_LkT;
+    if (c.lane() == 0) {
+        float4 &b = c.band();
+        b.x = __expf(h) * (1.0f + 4e-6f + 2e-6f * h);
+        b.y = 0.5f * (vlo + vhi);
+    }
+    return s + len;
+}
+
+// Decision bounds of the zones of the rail slots in `dirty` (bits).  Without ACC
+// they only tell which draws may be accepted, for any state of an end entry and
+// with room for a.ion_slack in the exponent, so that they hold while ions cross a
+// few boundaries (a.ion_budget); the draws below them are decided with ion_zone.
+__device__ __forceinline__ float ion_class(int k) { return __int_as_float((127 - k) << 23); }     // 2^-k
+template <int P, bool ACC, bool OPEN, bool CLS>
+__device__ __forceinline__ void ion_zones(const IonView<P, CLS> &c, uint32_t dirty)
+{
     constexpr int G = 32 / P;
     const SweepArgs &a = c.a;
     const int Z = a.Z;
-    if (window) {
-        // A window: steps from s on, at most VWIN, whose voltage stays near the
-        // first one's.  Evaluating at the window's mid voltage changes B/(1+B)
-        // and 1/(1+B) by a factor within [e^-h, e^h] (logarithmic derivatives at
-        // most 1); a jump (a pulse's edge) would widen the bounds by several per
-        // cent for all of the window's steps, so it starts the next one.
-        const int left = min(VWIN, n_steps - s);
-        const double v = a.V[t0 + s + min(c.lane(), left - 1)];
-        const float v0 = __shfl_sync(FULL, (float)v, 0);
-        const uint32_t far = __ballot_sync(FULL, fabsf((float)v - v0) * a.inv_LkT > 2e-3f);
-        const int len = min(left, far ? __ffs(far) - 1 : VWIN);
-        float vlo = __double2float_rd(v), vhi = __double2float_ru(v);
-        if (c.lane() >= len) vlo = vhi = v0;
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            vlo = fminf(vlo, __shfl_xor_sync(FULL, vlo, off));
-            vhi = fmaxf(vhi, __shfl_xor_sync(FULL, vhi, off));
-        }
-        const float h = 0.5f * (vhi - vlo) * a.inv_LkT;
-        if (c.lane() == 0) {
-            float4 &b = c.band();
-            b.x = __expf(h) * (1.0f + 4e-6f + 2e-6f * h);
-            b.y = 0.5f * (vlo + vhi);
-        }
-        wend = s + len;
-    }
     __syncwarp();
-    const float eh = c.band().x, Vf = c.band().y;
     const int items = __popc(dirty) * Z;
     for (int i = c.lane(); i < items; i += 32) {
         const int k = (int)(((uint32_t)i * a.rcpZ) >> 16), z = i - k * Z;    // i / Z for i < 1024
         uint32_t m = dirty;
         for (int q = 0; q < k; ++q) m &= m - 1;
         const int sg = G == 1 ? 0 : __ffs(m) - 1;
-        const int32_t *Pb = c.Pb(sg), *Fs = c.Fs(sg);
-        uint8_t *rm = c.bounds(sg);
-        // an open rail's counts are relative to its first boundary
-        const int p0 = OPEN ? Pb[0] : 0;
-        const int Pz = Pb[z] - p0, Pz1 = Pb[z + 1] - p0;
-        const int F = OPEN ? (int)((uint32_t)Fs[0] - (uint32_t)p0 * (uint32_t)(2 * a.L)) : Fs[0];
-        const float Ff = (float)F * a.inv_L, Nf = (float)Fs[G], Pf = (float)(Pz + Pz1);
-        const float qd = 0.5f * (Pf - Ff) - Nf * a.cz[z];
-        const float x = -(Vf - a.ka_f * qd) * a.inv_LkT;
-        const float S = (fabsf(Vf) + fabsf(a.ka_f) * (Pf + Ff + Nf)) * a.inv_LkT;
-        const float eps = 4e-6f + 5e-7f * fabsf(x) + 1.2e-6f * S;
-        const bool ok = fabsf(x) <= 40.0f && eps < 0.25f;
-        // no bounds: every draw of the zone goes to the FP64 paths
-        uint4 b = make_uint4(FULL, FULL, 0u, 0u);
-        float inv = 0.0f, sR = 0.0f, flo = 0.0f, fhi = 0.0f;
-        if (ok) {
-            const float B = __expf(x);
-            inv = __fdividef(1.0f, 1.0f + B);
-            sR = inv * B;
-            flo = __fdividef(1.0f - eps, eh);
-            fhi = (1.0f + eps) * eh;
-            float blo = a.P0f_scalar, bhi = a.P0f_scalar;
-            if (a.P0bnd != nullptr) {
-                const float2 pp = c.p0b(sg)[z];
-                blo = pp.x;
-                bhi = pp.y;
-            }
-            b.x = rej_thr(bhi * sR * fhi);
-            b.y = rej_thr(bhi * inv * fhi);
-            b.z = acc_thr(blo * sR * flo);
-            b.w = acc_thr(blo * inv * flo);
+        const IonZone r = ion_zone<P, OPEN>(c, sg, z);
+        uint8_t *rm = c.bounds(sg) + (z << c.cls()) * 16, *ends = c.end_rows(sg);
+        float blo = a.P0f_scalar, bhi = a.P0f_scalar;
+        if (a.P0bnd != nullptr) {
+            const float2 pp = c.p0b(sg)[z];
+            blo = pp.x;
+            bhi = pp.y;
         }
-        *(uint4 *)(rm + z * 16) = b;
-        if (a.P0bnd != nullptr) c.zf(sg)[z] = make_float4(sR, inv, flo, fhi);
+        if constexpr (!ACC) {
+            const float top = r.hi * (1.0f + a.ion_slack + a.ion_slack * a.ion_slack);    // above e^slack
+            const float bot = a.ion_exchange ? 0.0f : r.lo * (1.0f - a.ion_slack);
+            uint2 b = make_uint2(FULL, FULL);
+            if (r.ok) b = make_uint2(rej_thr(bhi * r.sR * top), rej_thr(bhi * r.inv * top));
+            *(uint2 *)rm = b;
+            for (int k = 1; k < 1 << c.cls(); ++k) {
+                const float bk = bhi * ion_class(k) * (1.0f + 2.4e-7f);     // P0 rounded to FP32 chose the class
+                if (r.ok) *(uint2 *)(rm + 16 * k) = make_uint2(rej_thr(bk * r.sR * top), rej_thr(bk * r.inv * top));
+                else *(uint2 *)(rm + 16 * k) = b;
+            }
+            if (OPEN && (z == 0 || z == Z - 1)) {
+                // end rows: the hop inward, then the bounds of the exchange with
+                // the electrode, from the virtual site in, from the site out
+                const float Ein = a.E_inf, Eout = a.E_outf;
+                if (z == 0) {
+                    uint4 in = make_uint4(FULL, FULL, FULL, 0u), out = in;
+                    if (r.ok) {
+                        in = make_uint4(b.x, 0u, rej_thr(Ein * r.sR * top), acc_thr(Ein * r.sR * bot));
+                        out = make_uint4(b.x, 0u, rej_thr(Eout * r.inv * top), acc_thr(Eout * r.inv * bot));
+                    }
+                    *(uint4 *)ends = in;
+                    *(uint4 *)(ends + 16) = out;
+                }
+                if (z == Z - 1) {
+                    uint4 in = make_uint4(FULL, FULL, FULL, 0u), out = in;
+                    if (r.ok) {
+                        in = make_uint4(0u, b.y, rej_thr(Ein * r.inv * top), acc_thr(Ein * r.inv * bot));
+                        out = make_uint4(0u, b.y, rej_thr(Eout * r.sR * top), acc_thr(Eout * r.sR * bot));
+                    }
+                    *(uint4 *)(ends + 32) = out;
+                    *(uint4 *)(ends + 48) = in;
+                }
+            }
+            continue;
+        }
+        uint4 b = make_uint4(FULL, FULL, 0u, 0u);
+        if (r.ok) {
+            b.x = rej_thr(bhi * r.sR * r.hi);
+            b.y = rej_thr(bhi * r.inv * r.hi);
+            b.z = acc_thr(blo * r.sR * r.lo);
+            b.w = acc_thr(blo * r.inv * r.lo);
+        }
+        *(uint4 *)rm = b;
         if (OPEN && (z == 0 || z == Z - 1)) {
             // electrode positions: outward trials are extractions, the virtual
             // sites' inward trials injections
             const float Ein = a.E_inf, Eout = a.E_outf;
             if (z == 0) {
                 uint4 e = b, q = b;
-                if (ok) {
-                    e.x = rej_thr(Ein * sR * fhi);
-                    e.z = acc_thr(Ein * sR * flo);
-                    q.y = rej_thr(Eout * inv * fhi);
-                    q.w = acc_thr(Eout * inv * flo);
+                if (r.ok) {
+                    e.x = rej_thr(Ein * r.sR * r.hi);
+                    e.z = acc_thr(Ein * r.sR * r.lo);
+                    q.y = rej_thr(Eout * r.inv * r.hi);
+                    q.w = acc_thr(Eout * r.inv * r.lo);
                 }
-                *(uint4 *)(rm + Z * 16) = e;
-                *(uint4 *)(rm + Z * 16 + 16) = q;
+                *(uint4 *)ends = e;
+                *(uint4 *)(ends + 16) = q;
             }
             if (z == Z - 1) {
                 uint4 e = b, q = b;
-                if (ok) {
-                    e.y = rej_thr(Ein * inv * fhi);
-                    e.w = acc_thr(Ein * inv * flo);
-                    q.x = rej_thr(Eout * sR * fhi);
-                    q.z = acc_thr(Eout * sR * flo);
+                if (r.ok) {
+                    e.y = rej_thr(Ein * r.inv * r.hi);
+                    e.w = acc_thr(Ein * r.inv * r.lo);
+                    q.x = rej_thr(Eout * r.sR * r.hi);
+                    q.z = acc_thr(Eout * r.sR * r.lo);
                 }
-                *(uint4 *)(rm + Z * 16 + 32) = q;
-                *(uint4 *)(rm + Z * 16 + 48) = e;
+                *(uint4 *)(ends + 32) = q;
+                *(uint4 *)(ends + 48) = e;
             }
         }
     }
     __syncwarp();
 }
 
+// A draw that may be accepted, decided in the FP32 band of its own probability:
+// the site's P0, or the electrode's.  d* out: 0, 1, or 2 when it lies in the band.
+template <int P, bool OPEN, bool CLS>
+__device__ __forceinline__ void ion_decide(const IonView<P, CLS> &c, const IonEntry &q, int64_t rail, uint32_t xy,
+                                           uint32_t xw, int &dR, int &dL)
+{
+    const SweepArgs &a = c.a;
+    const int L = a.L;
+    const IonZone r = ion_zone<P, OPEN>(c, c.seg(), c.zone(q.e));
+    float P0 = a.P0f_scalar;
+    if (a.P0bnd != nullptr && (!OPEN || (q.x >= 0 && q.x < L))) P0 = __ldg(a.P0f + rail * L + q.x);
+    float bR = P0, bL = P0;
+    if (OPEN) {
+        if (q.x < 0) bR = a.E_inf;
+        if (q.x == 0) bL = a.E_outf;
+        if (q.x == L - 1) bR = a.E_outf;
+        if (q.x >= L) bL = a.E_inf;
+    }
+    dR = q.fR ? (r.ok ? bounded(xy, bR * r.sR, r.lo, r.hi) : 2) : 0;
+    dL = q.fL ? (r.ok ? bounded(xw, bL * r.inv, r.lo, r.hi) : 2) : 0;
+}
+
+// Exchanges with the electrodes without the accept path.  They are the most
+// frequent events of an open rail, and as long as no ion inside it moves they
+// concern its end entries only, which then step in and out in turn.  ion_end_draws
+// draws for both ends over the next kIonAhead steps, one lane to an end and step;
+// its result, on the lane that holds the end entry: bits q of a step where an
+// injection may (0..3) or surely will (4..7) be accepted, and an extraction (8..15).
+template <int P, bool CLS>
+__device__ __forceinline__ bool ion_end(const IonView<P, CLS> &c, bool &left, uint32_t *&at)
+{
+    const int n = (int)c.slot(kSlotN), sl = c.sl();
+    left = sl == 0;
+    at = c.colp();
+    if (n <= 0) return false;
+    if (left) return true;
+    at += (n - 1) * 32;
+    return sl == P - 1 || pos_of(*at) + gap_last(c.slot(kSlotGaps)) == c.a.L + 1;
+}
+template <int P, bool CLS>
+__device__ __forceinline__ uint32_t ion_end_draws(const IonView<P, CLS> &c, const uint8_t *tab, uint32_t t, uint32_t prail,
+                                                  const uint32_t *rk0, const uint32_t *rk1)
+{
+    const SweepArgs &a = c.a;
+    uint32_t *at;
+    bool left;
+    const bool own = ion_end<P>(c, left, at);
+    uint32_t r = 0u;
+#pragma unroll
+    for (int pass = 0; pass < (P >= 8 ? 1 : 2); ++pass) {
+        const bool right = P >= 8 ? (c.sl() & 4) != 0 : pass != 0;
+        const uint32_t tk = t + (uint32_t)(c.sl() & 3);
+        const uint4 w = site_at(tab, (uint32_t)(right ? a.L : 1) * kStep);
+        uint32_t xy, xw;
+        site_draw(step_draw(tk, prail, rk0, rk1), w.x, w.y, w.z, rk0, rk1, xy, xw);
+        const uint8_t *rm = c.end_rows(c.seg()) + 8;
+        const uint2 in = *(const uint2 *)(rm + (right ? 48 : 0)), out = *(const uint2 *)(rm + (right ? 32 : 16));
+        const uint32_t xi = right ? xw : xy, xo = right ? xy : xw;
+        // the even/odd rule: the bond right of x is active when x = t (mod 2)
+        const bool act = a.rule == 0 || (((uint32_t)(right ? a.L - 1 : -1) ^ tk) & 1u) == 0u;
+        const uint32_t b0 = __ballot_sync(FULL, act && xi <= in.x), b1 = __ballot_sync(FULL, act && xi < in.y);
+        const uint32_t b2 = __ballot_sync(FULL, act && xo <= out.x), b3 = __ballot_sync(FULL, act && xo < out.y);
+        const int sh = c.lane() - c.sl() + (P >= 8 && !left ? 4 : 0);
+        if (own && (P >= 8 || left == (pass == 0)))
+            r = ((b0 >> sh) & 15u) | ((b1 >> sh) & 15u) << 4 | ((b2 >> sh) & 15u) << 8 | ((b3 >> sh) & 15u) << 12;
+    }
+    return r;
+}
+// Steps q .. stop - 1 (after step s of the launch), in which nothing but exchanges
+// can happen: carries them out, up to the first one that is not sure, and returns
+// the step that has to be looked at, stop when there was none.  und: the end entry's
+// bit if its exchange may be accepted in that step.
+template <int P, class M, bool CLS>
+__device__ __forceinline__ int ion_exchanges(const IonView<P, CLS> &c, const uint8_t *tab, int64_t t0, int s, int n_steps,
+                                             int q, int stop, uint32_t bits, M &und)
+{
+    const SweepArgs &a = c.a;
+    uint32_t *at;
+    bool left;
+    const bool own = ion_end<P>(c, left, at);
+    const int x = own ? pos_of(*at) : 0;
+    const bool full = left ? x >= 0 : x < a.L;
+    uint32_t moved = 0u;
+    int mine = stop;
+    if (bits != 0u) {
+        bool o = full;
+        for (int k = q; k < stop; ++k) {
+            const uint32_t b = bits >> (k + (o ? 8 : 0));
+            if ((b & 0x11u) == 0x1u) {
+                mine = k;
+                break;
+            }
+            if (b & 1u) {
+                moved |= 1u << k;
+                o = !o;
+            }
+        }
+    }
+    stop = __reduce_min_sync(FULL, mine);
+    moved &= (1u << stop) - 1u;
+    if (__any_sync(FULL, moved != 0u)) {
+        if (moved) {
+            int m = full == left ? -1 : 1;
+            const int cnt = __popc(moved);
+            if (cnt & 1) {
+                const int b = left ? 0 : a.Z;
+                atomicAdd(&c.Pb(c.seg())[b], -m);
+                atomicAdd(c.Fs(), -m * a.wsum[b]);
+                *at = site_at(tab, (uint32_t)(x + 1 + m) * kStep).w;
+            }
+            c.slot(kSlotMoves) += (uint32_t)cnt;
+            unsigned long long *const J = a.J + t0 + s, *const zc = a.Zc + (t0 + s + 1) * a.Z + (left ? 0 : a.Z - 1);
+            for (uint32_t k = moved; k; k &= k - 1) {
+                const int w = __ffs(k) - 1;
+                atomicAdd(J + w, (unsigned long long)(long long)(-m));
+                if (s + w + 1 < n_steps)
+                    atomicAdd(zc + (int64_t)w * a.Z, (unsigned long long)(long long)(left ? m : -m));
+                m = -m;
+            }
+        }
+        __syncwarp();
+        ion_refresh<P>(c, (int)c.slot(kSlotN), -2, a.L + 1);
+        __syncwarp();
+    }
+    if (own) {
+        const bool o = full != ((__popc(moved) & 1) != 0);
+        if ((bits >> (stop + (o ? 8 : 0))) & 1u) und = left ? M(1) : M(1) << ((int)c.slot(kSlotN) - 1);
+    }
+    return stop;
+}
+
 // The list ends of open rails after a step's moves: the first entry stays at
-// site -1 or 0, the last at L - 1 or L.  Returns (warp-uniform) whether the
-// bounds were overwritten.
-template <int P>
-__device__ __forceinline__ bool ion_ends(const IonView<P> &c, const uint8_t *tab, int s, bool active,
-                                         uint32_t &draws)
+// site -1 or 0, the last at L - 1 or L.  Returns (warp-uniform) 0 when no entry
+// came or went, 1 when one did, 2 when the bounds were overwritten on the way.
+template <int P, bool CLS>
+__device__ __forceinline__ int ion_ends(const IonView<P, CLS> &c, const uint8_t *tab, int s, int64_t rail,
+                                        uint32_t &draws)
 {
     const SweepArgs &a = c.a;
     const int L = a.L, sl = c.sl();
@@ -587,7 +799,7 @@ __device__ __forceinline__ bool ion_ends(const IonView<P> &c, const uint8_t *tab
             }
         }
     }
-    if (!__any_sync(FULL, n != n0)) return false;
+    if (!__any_sync(FULL, n != n0)) return 0;
     // draws so far were of the old columns
     draws = __reduce_add_sync(FULL, (uint32_t)n0) * (uint32_t)(s + 1 - c.mark());
     __syncwarp();
@@ -600,14 +812,14 @@ __device__ __forceinline__ bool ion_ends(const IonView<P> &c, const uint8_t *tab
     for (int off = P / 2; off >= 1; off >>= 1) M += __shfl_xor_sync(FULL, M, off, P);
     if (__any_sync(FULL, (n0 > 0 && n == 0) || n > min((M + P - 1) / P + 1, a.rcap - 2))) {
         ion_to_words<P>(c);
-        ion_build<P, true>(c, tab, active);
-        return true;
+        ion_build<P, true>(c, tab, rail);
+        return 2;
     }
     const int km = __reduce_max_sync(FULL, n);
     if (c.lane() == 0) c.kmax() = km;
     ion_refresh<P>(c, n, -2, L + 1);
     __syncwarp();
-    return false;
+    return 1;
 }
 
 // ------------------------------------------------- gradient pass
@@ -620,8 +832,8 @@ __device__ __forceinline__ double count_to_double(int n)
 }
 
 // Constants and empty sums of the warp's rails.
-template <int P>
-__device__ __forceinline__ void ion_score_begin(const IonView<P> &c)
+template <int P, bool CLS>
+__device__ __forceinline__ void ion_score_begin(const IonView<P, CLS> &c)
 {
     const SweepArgs &a = c.a;
     const int L = a.L;
@@ -644,8 +856,8 @@ __device__ __forceinline__ void ion_score_begin(const IonView<P> &c)
 // exp(xV V), exp(xV kappa alpha D'_z) and the tabulated exponential of the
 // integer zone sum m_z = L (P_z + P_z+1) - F; one reciprocal of x1 y2 y3 with
 // x1 = 1 + B, y2 = x1 (1 - p_R), y3 = x1 (1 - p_L) serves all three quotients.
-template <int P, bool OPEN>
-__device__ __forceinline__ void ion_score_zones(const IonView<P> &c, uint32_t t, uint32_t stale)
+template <int P, bool OPEN, bool CLS>
+__device__ __forceinline__ void ion_score_zones(const IonView<P, CLS> &c, uint32_t t, uint32_t stale)
 {
     constexpr int G = 32 / P;
     const SweepArgs &a = c.a;
@@ -730,8 +942,8 @@ __device__ __forceinline__ void ion_score_zones(const IonView<P> &c, uint32_t t,
 // take its zones in turn and keep their own shares of W, K and the estimator
 // sums; only the step's coefficient (the zone counts' share less the current's
 // innovation, a control variate of zero mean) is summed over them.
-template <int P, bool OPEN, class M>
-__device__ __forceinline__ void ion_score(const IonView<P> &c, uint32_t t, M fR, M fL, M aR, M aL)
+template <int P, bool OPEN, class M, bool CLS>
+__device__ __forceinline__ void ion_score(const IonView<P, CLS> &c, uint32_t t, M fR, M fL, M aR, M aL)
 {
     const SweepArgs &a = c.a;
     const int Z = a.Z, L = a.L, sl = c.sl();
@@ -863,8 +1075,8 @@ __device__ __forceinline__ void ion_score(const IonView<P> &c, uint32_t t, M fR,
 
 // The current of step t pairs with the score of steps <= t.  Jl: this lane's net
 // leftward crossings.
-template <int P>
-__device__ __forceinline__ void ion_score_current(const IonView<P> &c, uint32_t t, int Jl)
+template <int P, bool CLS>
+__device__ __forceinline__ void ion_score_current(const IonView<P, CLS> &c, uint32_t t, int Jl)
 {
     const SweepArgs &a = c.a;
     if (!a.wJ) return;
@@ -879,8 +1091,8 @@ __device__ __forceinline__ void ion_score_current(const IonView<P> &c, uint32_t 
 }
 
 // The rails' W, K, G_W, G_K: sums of their lanes' shares.
-template <int P>
-__device__ __forceinline__ void ion_score_end(const IonView<P> &c, int64_t rail)
+template <int P, bool CLS>
+__device__ __forceinline__ void ion_score_end(const IonView<P, CLS> &c, int64_t rail)
 {
     const SweepArgs &a = c.a;
     for (int k = 0; k < 5; ++k) {
@@ -899,7 +1111,14 @@ __device__ __forceinline__ void ion_score_end(const IonView<P> &c, int64_t rail)
 // accepted draws per warp and step) it also compares with the lower bounds and
 // keeps which neighbours are one and two sites away, so that exclusion and
 // conflicts are a few operations on bits; without, the entries with a word
-// below its upper bound are looked at one by one.  GRAD: the gradient pass, which
+// below its upper bound are looked at one by one, and as moves are rare the loop
+// draws for kIonAhead steps at once: an entry is loaded once for four draws, and the
+// four chains hide each other's latency.  An ion that moves is drawn for again for
+// the steps left.  Steps with nothing but exchanges are left to ion_exchanges (the
+// virtual site -1 draws for site 0, so they change no draw).  Against one step at a
+// time, 1,000 steps at P0 = 3.8e-4: 64 rails of 100 sites 0.35 -> 0.18 ms, 16,000 of
+// 200 3.2 -> 2.6 ms, 3,001 open ones of 777 3.0 -> 2.2 ms; 65,536 of 1,024 with
+// per-site barriers 60 -> 50 ms.  GRAD: the gradient pass, which
 // replays the sweep from its first occupancy with the score accumulated instead
 // of the traces.
 template <int P, bool ACC, bool OPEN, class M, bool GRAD = false>
@@ -908,7 +1127,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                                          uint8_t *smem)
 {
     constexpr int G = 32 / P;
-    using View = IonView<P>;
+    using View = IonView<P, !ACC>;
     uint8_t *tab = smem;    // site table of the CTA
 
     {
@@ -921,8 +1140,9 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             const int k = min(max(i - 1, 0), L - 1);
             int row = 0;
             while (a.bnd[row + 1] <= k) ++row;
-            if (OPEN && i <= 1) row = Z + i;
-            if (OPEN && i >= L) row = Z + 2 + (i - L);
+            row <<= c.cls();
+            if (OPEN && i <= 1) row = (Z << c.cls()) + i;
+            if (OPEN && i >= L) row = (Z << c.cls()) + 2 + (i - L);
             const uint3 w = site_words((uint32_t)k, a.instance ^ rk1[0]);
             ((uint4 *)tab)[i] = make_uint4(w.x, w.y, w.z, (uint32_t)(i * kStep) | (uint32_t)(row * 16) << 16);
         }
@@ -968,7 +1188,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             const int nz = c.Pb(c.seg())[z + 1] - c.Pb(c.seg())[z];
             if (nz != 0) atomicAdd(&a.Zc[t0 * Z + z], (unsigned long long)(long long)nz);
         }
-        ion_build<P, OPEN>(c, tab, active);
+        ion_build<P, OPEN>(c, tab, rail);
         const int sum = ion_sum<P>(c);
         if (sl == 0) c.Fs()[2 * G] = sum;
         __syncwarp();
@@ -976,16 +1196,19 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
     }
 
     int wend = 0;          // first step after the voltage window of the bounds
+    int spent = 0;         // boundary crossings since the bounds were evaluated
     uint32_t dirty = 0u;   // rail slots whose zone sums changed since their bounds were evaluated
     for (int c0 = 0; c0 < n_steps; c0 += flush) {
         const int c1 = min(n_steps, c0 + flush);
-        for (int s = c0; s < c1; ++s) {
+        for (int s = c0; s < c1;) {
             const uint32_t t = (uint32_t)(t0 + s);
 
-            if (dirty != 0u || s == wend) {
+            const bool window = s == wend;
+            if (dirty != 0u || window) {
                 const View c(a, smem);
-                ion_zones<P, OPEN>(c, t0, s, n_steps, s == wend,
-                                   s == wend ? (uint32_t)((1ull << G) - 1u) : dirty, wend);
+                if (window) wend = ion_window<P>(c, t0, s, n_steps);
+                ion_zones<P, ACC, OPEN>(c, window ? (uint32_t)((1ull << G) - 1u) : dirty);
+                spent = 0;
             }
             const uint32_t stale = GRAD ? dirty : 0u;   // rail slots to score anew
             dirty = 0u;
@@ -995,13 +1218,15 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             //      sites away
             M aR = 0, aL = 0, und = 0, two = 0;
             M fR = 0, fL = 0;       // rows with open trials (gradient pass)
+            uint32_t look = 0u, ends_at = 0u;   // without ACC: steps with a draw that may be accepted, exchanges
             {
                 const View c(a, smem);
-                const StepDraw sd = step_draw(t, a.rail_base + (uint32_t)c.rail(tile_rail0), rk0, rk1);
+                const uint32_t prail = a.rail_base + (uint32_t)c.rail(tile_rail0);
                 const uint8_t *rm = c.bounds();
                 const uint32_t *cp = c.colp();
                 const uint32_t *const end = cp + c.kmax() * 32;
                 if constexpr (ACC) {
+                    const StepDraw sd = step_draw(t, prail, rk0, rk1);
                     M sR = 0, sL = 0, one = 0;
                     uint32_t e = *cp;
                     for (int half = 0; half < (int)sizeof(M) / 4 && cp != end; ++half) {
@@ -1052,25 +1277,55 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                     }
                     und = (aR & ~sR) | (aL & ~sL);
                 } else {
-                    for (int half = 0; half < (int)sizeof(M) / 4 && cp != end; ++half) {
+                    StepDraw sd[kIonAhead];
+#pragma unroll
+                    for (int q = 0; q < kIonAhead; ++q) sd[q] = step_draw(t + q, prail, rk0, rk1);
+                    for (int half = 0; half < (int)sizeof(M) / 4; ++half) {
                         const uint32_t *const to = end - cp > 32 * 32 ? cp + 32 * 32 : end;
-                        uint32_t h = 0u, bit = 1u;
-#pragma unroll 4
+                        uint32_t h[kIonAhead] = {}, bit = 1u;
+#pragma unroll 1
                         while (cp != to) {
                             const uint32_t e = *cp;
                             cp += 32;
                             const uint4 w = site_at(tab, e);
-                            uint32_t xy, xw;
-                            site_draw(sd, w.x, w.y, w.z, rk0, rk1, xy, xw);
                             const uint2 th = *(const uint2 *)(rm + (e >> 16));
-                            if (xy <= th.x || xw <= th.y) h |= bit;
+#pragma unroll
+                            for (int q = 0; q < kIonAhead; ++q) {
+                                uint32_t xy, xw;
+                                site_draw(sd[q], w.x, w.y, w.z, rk0, rk1, xy, xw);
+                                if (xy <= th.x || xw <= th.y) h[q] |= bit;
+                            }
                             bit <<= 1;
                         }
-                        und |= (M)h << (32 * half);
+#pragma unroll
+                        for (int q = 0; q < kIonAhead; ++q) {
+                            c.hits(q + kIonAhead * half) = h[q];
+                            if (h[q]) look |= 1u << q;
+                        }
                     }
+                    look = __reduce_or_sync(FULL, look);
+                    if constexpr (OPEN) ends_at = ion_end_draws<P>(c, tab, t, prail, rk0, rk1);
                 }
             }
-            if (!GRAD && !__any_sync(FULL, (aR | aL | und) != 0)) continue;
+            // ---- the steps drawn for, up to one that changes what the next draw
+            int ahead = ACC ? 1 : min(kIonAhead, min(c1, wend) - s);
+#pragma unroll 1
+            for (int q = 0; q < ahead; ++q) {
+            if constexpr (!ACC) {
+                const uint32_t next = look >> q;
+                int stop = next ? min(ahead, q + __ffs(next) - 1) : ahead;
+                und = 0;
+                const View c(a, smem);
+                if (OPEN) stop = ion_exchanges<P, M>(c, tab, t0, s, n_steps, q, stop, ends_at, und);
+                if (stop >= ahead) break;
+                q = stop;
+                und |= c.hits(q);
+                if (sizeof(M) > 4) und |= (M)c.hits(q + kIonAhead) << (8 * sizeof(M) - 32);
+                aR = aL = two = 0;
+            }
+            const int sq = s + q;
+            const uint32_t tq = t + (uint32_t)q;
+            if (ACC && !GRAD && !__any_sync(FULL, (aR | aL | und) != 0)) continue;
 
             // ---- draws between their bounds (without ACC every draw that may be
             //      accepted): the site's own base probability in the FP32 band
@@ -1079,32 +1334,20 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 {
                     const View c(a, smem);
                     const int64_t rail = c.rail(tile_rail0);
-                    const StepDraw sd = step_draw(t, a.rail_base + (uint32_t)rail, rk0, rk1);
+                    const StepDraw sd = step_draw(tq, a.rail_base + (uint32_t)rail, rk0, rk1);
                     const int n = (int)c.slot(kSlotN);
                     const uint32_t gaps = c.slot(kSlotGaps);
                     for (; und; und &= und - 1) {
                         const M bit = und & (M(0) - und);
-                        const IonEntry q = ion_entry(c.colp(), first_bit(und), n, gaps, a.rule, t);
-                        const uint32_t site = (uint32_t)min(max(q.x, 0), a.L - 1);
-                        const uint4 w = site_at(tab, q.e);
+                        const IonEntry en = ion_entry(c.colp(), first_bit(und), n, gaps, a.rule, tq);
+                        const uint4 w = site_at(tab, en.e);
                         uint32_t xy, xw;
                         site_draw(sd, w.x, w.y, w.z, rk0, rk1, xy, xw);
-                        const uint4 th = *(const uint4 *)(c.bounds() + (q.e >> 16));
-                        int dR = q.fR && xy <= th.x ? (xy < th.z ? 1 : 2) : 0;
-                        int dL = q.fL && xw <= th.y ? (xw < th.w ? 1 : 2) : 0;
-                        if (a.P0bnd != nullptr && (dR == 2 || dL == 2)) {
-                            // inner trials (electrode trials have one base probability)
-                            const int row = (int)(q.e >> 20);
-                            const float4 z = c.zf(c.seg())[min(max(code_of_row(row, a.Z) - 1, 0), a.Z - 1)];
-                            if (z.y > 0.0f) {
-                                const float P0 = __ldg(a.P0f + rail * a.L + site);
-                                if (dR == 2 && row != a.Z && row != a.Z + 2) dR = bounded(xy, P0 * z.x, z.z, z.w);
-                                if (dL == 2 && row != a.Z + 1 && row != a.Z + 3) dL = bounded(xw, P0 * z.y, z.z, z.w);
-                            }
-                        }
+                        int dR, dL;
+                        ion_decide<P, OPEN>(c, en, rail, xy, xw, dR, dL);
                         aR = dR == 1 ? aR | bit : aR & ~bit;
                         aL = dL == 1 ? aL | bit : aL & ~bit;
-                        if (q.gR == 2) two |= bit;
+                        if (en.gR == 2) two |= bit;
                         if (dR == 2 || dL == 2) left |= bit;
                     }
                 }
@@ -1113,11 +1356,10 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                     const View c(a, smem);
                     for (; left; left &= left - 1) {
                         const M bit = left & (M(0) - left);
-                        const IonEntry q = ion_entry(c.colp(), first_bit(left), (int)c.slot(kSlotN),
-                                                     c.slot(kSlotGaps), a.rule, t);
-                        int dR = q.fR ? 2 : 0, dL = q.fL ? 2 : 0;
-                        ion_exact<P>(c, c.seg(), c.rail(tile_rail0), q.x,
-                                     min(max(code_of_row((int)(q.e >> 20), a.Z) - 1, 0), a.Z - 1), t, dR, dL);
+                        const IonEntry en = ion_entry(c.colp(), first_bit(left), (int)c.slot(kSlotN),
+                                                     c.slot(kSlotGaps), a.rule, tq);
+                        int dR = en.fR ? 2 : 0, dL = en.fL ? 2 : 0;
+                        ion_exact<P>(c, c.seg(), c.rail(tile_rail0), en.x, c.zone(en.e), tq, dR, dL);
                         aR = dR == 1 ? aR | bit : aR & ~bit;
                         aL = dL == 1 ? aL | bit : aL & ~bit;
                     }
@@ -1132,7 +1374,9 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
 
             // ---- moves and the current: both trials accepted, the ion stays; two
             //      ions entering the site between them are both cancelled
-            bool crossed = false;
+            bool inner = false;      // a move inside the rail
+            uint32_t more = 0u;      // steps in which it may move again
+            int crossings = 0;       // zone boundaries crossed
             {
                 const View c(a, smem);
                 const M both = aR & aL;
@@ -1156,31 +1400,66 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 uint32_t *colp = c.colp();
                 for (M todo = aR | aL; todo; todo &= todo - 1) {
                     const int j = first_bit(todo);
-                    crossed |= ion_commit<P>(c, tab, colp + j * 32, colp[j * 32], (aR >> j) & 1 ? 1 : -1,
-                                             !GRAD && s + 1 < n_steps ? a.Zc + (t0 + s + 1) * a.Z : nullptr);
+                    const int r = ion_commit<P>(c, tab, c.rail(tile_rail0), colp + j * 32, colp[j * 32], (aR >> j) & 1 ? 1 : -1,
+                                                !GRAD && sq + 1 < n_steps ? a.Zc + (t0 + sq + 1) * a.Z : nullptr);
+                    if constexpr (ACC) {
+                        crossings += r != 0 ? 1 : 0;
+                    } else {
+                        crossings += r == 2 ? a.ion_exchange : r;
+                        if (r == 2) continue;
+                        inner = true;
+                        const uint32_t e = colp[j * 32], prail = a.rail_base + (uint32_t)c.rail(tile_rail0);
+                        const uint4 w = site_at(tab, e);
+                        const uint2 th = *(const uint2 *)(c.bounds() + (e >> 16));
+#pragma unroll 1
+                        for (int k = q + 1; k < ahead; ++k) {
+                            uint32_t xy, xw;
+                            site_draw(step_draw(t + (uint32_t)k, prail, rk0, rk1), w.x, w.y, w.z, rk0, rk1, xy, xw);
+                            if (xy <= th.x || xw <= th.y) {
+                                c.hits(k + kIonAhead * (j >> 5)) |= 1u << (j & 31);
+                                more |= 1u << k;
+                            }
+                        }
+                    }
                 }
                 if constexpr (GRAD) {
                     ion_score_current<P>(c, t, nL - nR);
                 } else {
                     c.slot(kSlotMoves) += (uint32_t)(nR + nL);
                     const int Jw = __reduce_add_sync(FULL, nL - nR);
-                    if (c.lane() == 0 && Jw != 0) atomicAdd(&a.J[t0 + s], (unsigned long long)(long long)Jw);
+                    if (c.lane() == 0 && Jw != 0) atomicAdd(&a.J[t0 + sq], (unsigned long long)(long long)Jw);
                 }
                 ion_refresh<P>(c, n, OPEN ? -2 : -1, OPEN ? a.L + 1 : a.L);
+                __syncwarp();
             }
-            if (OPEN) {
+            // an entry can come or go at an end only when one inside has moved
+            int ends = 0;
+            if (!ACC && __any_sync(FULL, inner)) {
+                look |= __reduce_or_sync(FULL, more);
+                inner = true;
+            }
+            if (OPEN && (ACC || inner)) {
                 const View c(a, smem);
                 uint32_t draws = 0u;
-                crossed |= ion_ends<P>(c, tab, s, c.rail(tile_rail0) < a.R, draws);
+                ends = ion_ends<P>(c, tab, sq, c.rail(tile_rail0), draws);
                 if (!GRAD && draws != 0u && c.lane() == 0) atomicAdd(&a.counters[0], (unsigned long long)draws);
             }
-            // lanes to rail slots
-            const uint32_t cm = __ballot_sync(FULL, crossed);
-            if (G == 1) dirty = cm != 0u ? 1u : 0u;
-            else
+            if constexpr (ACC) {
+                // lanes to rail slots
+                const uint32_t cm = ends == 2 ? FULL : __ballot_sync(FULL, crossings != 0);
+                if (G == 1) dirty = cm != 0u ? 1u : 0u;
+                else
 #pragma unroll
-                for (int q = 0; q < G; ++q)
-                    if ((cm >> (q * P)) & ((1u << (P & 31)) - 1u)) dirty |= 1u << q;
+                    for (int k = 0; k < G; ++k)
+                        if ((cm >> (k * P)) & ((1u << (P & 31)) - 1u)) dirty |= 1u << k;
+            } else {
+                if (__any_sync(FULL, crossings != 0)) spent += __reduce_add_sync(FULL, crossings);
+                if (ends != 0) spent += 2;
+                if (spent > a.ion_budget || ends == 2) dirty = (uint32_t)((1ull << G) - 1u);
+                if (ends != 0 || dirty != 0u) ahead = q + 1;
+            }
+            }
+            s += ahead;
         }
         // ---- flush this warp's counters and per-rail current
         if constexpr (!GRAD) {

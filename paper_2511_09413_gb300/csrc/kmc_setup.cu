@@ -121,6 +121,26 @@ __global__ void p0_float_kernel(const double *P0, int64_t n, float *out)
         out[i] = (float)P0[i];
 }
 
+// 16 sites to a thread.
+__global__ void p0_classes_kernel(const float *P0f, const float2 *bnd, int64_t R, int32_t L, int32_t Z,
+                                  const DevConst *K, uint32_t *out)
+{
+    const int W = (L + 15) >> 4;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < R * W; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = i / W;
+        const int k0 = (int)(i - r * W) * 16;
+        uint32_t bits = 0;
+        int z = 0;
+        for (int k = k0; k < min(k0 + 16, L); ++k) {
+            while (K->bnd[z + 1] <= k) ++z;
+            const float v = P0f[r * L + k], hi = bnd[r * Z + z].y;
+            const uint32_t c = v > 0.5f * hi ? 0u : v > 0.25f * hi ? 1u : v > 0.125f * hi ? 2u : 3u;
+            bits |= c << (2 * (k - k0));
+        }
+        out[i] = bits;
+    }
+}
+
 // One warp per rail: ion count, and a count of bytes that are not 0 or 1.
 __global__ void row_counts_kernel(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
                                   int32_t *N0, unsigned long long *bad, unsigned long long *stats)
@@ -276,6 +296,13 @@ cudaError_t setup_p0_bounds(const double *P0, int32_t R, int32_t L, int32_t Z, c
 cudaError_t setup_p0_float(const double *P0, int64_t n, float *out, cudaStream_t s)
 {
     p0_float_kernel<<<grid_for(n, 256), 256, 0, s>>>(P0, n, out);
+    return cudaGetLastError();
+}
+
+cudaError_t setup_p0_classes(const float *P0f, const float2 *bnd, int64_t R, int32_t L, int32_t Z, const DevConst *K,
+                             uint32_t *out, cudaStream_t s)
+{
+    p0_classes_kernel<<<grid_for(R * ((L + 15) / 16), 256), 256, 0, s>>>(P0f, bnd, R, L, Z, K, out);
     return cudaGetLastError();
 }
 

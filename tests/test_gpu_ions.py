@@ -29,10 +29,10 @@ def _dev(**kw):
     return d
 
 
-def _check(K, dev, V, fill, chunks):
+def _check(K, dev, V, fill, chunks, Ea=None):
     occ0 = oracle.init_occupancy(dev, 1, fill=fill)
-    sim = K.Sim(dev, V, 2, occ0=occ0)
-    orc = oracle.OracleSim(dev, V, occ0, None)
+    sim = K.Sim(dev, V, 2, occ0=occ0, Ea_site=Ea)
+    orc = oracle.OracleSim(dev, V, occ0, Ea)
     for c in chunks:
         sim.step_n(c)
     n = sum(chunks)
@@ -69,6 +69,22 @@ def test_open_rails_grow_and_shrink(kmc, L, fill, rho, rule):
     dev = _dev(R=70, L=L, Z=min(L, 7), electrodes=1, k_e=4e6, rho_e=rho, dt=2e-6, rule=rule)
     V = 2.0 * np.sin(np.arange(500) / 40.0)
     _check(kmc, dev, V, fill, [500])
+
+
+# rare moves: four steps drawn at once, ions that move and exchanges in between,
+# launches and voltage jumps that end inside the four.  kappa sets how many moves
+# the decision bounds hold for (3: exchanges count as well; 300: none is left);
+# barriers of a wide spread fill every class of sites
+@pytest.mark.parametrize("L,Z", [(8, 8), (33, 1), (100, 10), (777, 32)])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("kappa", [1.0, 3.0, 300.0])
+@pytest.mark.parametrize("spread,rule", [(None, 0), (0.06, 0), (0.06, 1), (None, 1)])
+def test_rare_moves(kmc, L, Z, electrodes, kappa, spread, rule):
+    dev = _dev(R=45, L=L, Z=Z, electrodes=electrodes, k_e=2e7 if electrodes else 0.0, rho_e=0.4, dt=1e-8,
+               kappa=kappa, rule=rule)
+    Ea = None if spread is None else np.maximum(np.random.default_rng(L).normal(0.40, spread, (45, L)), 0.30)
+    V = np.where(np.arange(603) % 150 < 71, 1.0, -0.5) + 1e-3 * np.sin(np.arange(603))
+    _check(kmc, dev, V, 0.3, [1, 2, 3, 261, 336], Ea)
 
 
 # a batch chooses its tiles from all rails together: the same devices alone
