@@ -151,7 +151,8 @@ int pick_launch(kmc_handle *h)
     max_smem = std::min(max_smem, 200 * 1024);
     auto smem_for = [&](int w) { return tile_args(h->args, t, p, h->P0site != nullptr, w, l.acc != 0); };
     while (warps > 1 && smem_for(warps) > (size_t)max_smem) warps >>= 1;
-    if (t.ions && h->warps_req <= 0) warps = ion_cta_warps(h->args, (p.n_rails * (int64_t)t.lpr + 31) / 32, warps);
+    if (t.ions && h->warps_req <= 0)
+        warps = ion_cta_warps(h->args, t.kind, (p.n_rails * (int64_t)t.lpr + 31) / 32);
     l.warps = warps;
     l.smem = smem_for(warps);
     const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * warps;

@@ -40,7 +40,7 @@ struct IonLayout {
     uint32_t p0b;     // float2 [G][Z]: per-site P0 bounds of the zone (per-site barriers)
     uint32_t pb;      // int [G][Z + 1]: ions below each zone boundary
     uint32_t st;      // uint32 [slots][32]: each lane's state words
-    uint32_t hit;     // uint32 [4 or 8][32]: outcome bits of the steps drawn ahead (no accept path)
+    uint32_t hit;     // uint32 [0 .. 8][32]: outcome bits of the steps drawn ahead (no accept path), or rows at odd positions
     uint32_t g;       // gradient pass: its sums, counts and factors (IonView)
     uint32_t col;     // uint32 [rcap][32]: each lane's entries
     uint32_t bytes;   // one warp's block
@@ -212,7 +212,7 @@ TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_
 // filling of the sites up to which the ion lists are the better tile
 float tile_max_fill(bool acc);
 // sets a.rcap and a.iy for the tile; shared memory of a CTA of `warps` warps
-int ion_cta_warps(const SweepArgs &a, int64_t warps, int most);
+int ion_cta_warps(const SweepArgs &a, int kind, int64_t warps);
 size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool persite, int warps, bool acc);
 // the batch's kernels of ion-list kinds
 cudaError_t ion_batch_launch(const BatchArgs &b, int kind, int grid, int warps, size_t smem, bool acc,

@@ -13,9 +13,18 @@ namespace kmc {
 namespace {
 
 // 4 CTAs of 256 threads per SM (64 registers).  With 5 (48 registers) the
-// replicated 512-site device ran 4-11 % slower, with 3 (80) 4 % slower.
+// replicated 512-site device ran 4-11 % slower, with 3 (80) 4 % slower.  Rails of
+// more than 32 entries a lane are of 1,025 sites and more, whose site table and
+// columns leave room for 20 warps on an SM at most: they run in CTAs of up to as
+// many (96 registers), so that the table is held once.  2,500 rails of 2,048 sites
+// (16.4 warps an SM, half of them in a second wave in CTAs of 8): 5.1 -> 3.5 ms for
+// 300 steps in one wave of CTAs of 17.
+bool ion_wide(int kind) { return kind >= kWordKinds + 8; }
+int ion_most_smem(int kind) { return ion_wide(kind) ? kGradSmem : 200 * 1024; }
+template <class M>
+constexpr int kIonWarps = sizeof(M) > 4 ? 20 : 8;
 template <int P, bool ACC, bool OPEN, class M>
-__global__ void __launch_bounds__(256, 4) ion_kernel(const __grid_constant__ SweepArgs a, const int *gate)
+__global__ void __launch_bounds__(32 * kIonWarps<M>, sizeof(M) > 4 ? 1 : 4) ion_kernel(const __grid_constant__ SweepArgs a, const int *gate)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     if (gate && *gate != 0) return;     // the occupancy words advance this device
@@ -40,9 +49,9 @@ int ion_rows(int P, int L, bool open, int64_t n_max)
 
 }  // namespace
 
-IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, bool grad, bool ahead)
+IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, bool grad, bool acc, bool rule)
 {
-    const uint32_t G = 32u / (uint32_t)P, rows = ((uint32_t)Z << (persite && ahead ? 2 : 0)) + (open ? 5u : 1u);
+    const uint32_t G = 32u / (uint32_t)P, rows = ((uint32_t)Z << (persite && !acc ? 2 : 0)) + (open ? 5u : 1u);
     const uint32_t words = G * (uint32_t)((L + 31) >> 5) * 4u;   // occupancy words, staged in the bounds
     const uint32_t gz = G * (uint32_t)Z;
     const uint32_t pz = (uint32_t)align16(4u * G * (uint32_t)(Z + 1));
@@ -53,7 +62,7 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
     y.pb = y.p0b + (persite ? (uint32_t)align16(8u * gz) : 0u);
     y.st = y.pb + pz;
     y.hit = y.st + 128u * kIonSlots;
-    y.g = y.hit + (ahead ? 128u * kIonAhead * (rcap > 34 ? 2u : 1u) : 0u);
+    y.g = y.hit + 128u * (acc ? (rule ? 1u : 0u) : (uint32_t)kIonAhead) * (grad || rcap > 34 ? 2u : 1u);
     y.col = y.g + (grad ? 2688u + 64u * G + (uint32_t)align16(8u * G * (uint32_t)(Z + 1)) + 48u * gz : 0u);
     y.bytes = y.col + (uint32_t)rcap * 128u;
     return y;
@@ -76,7 +85,7 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
 // the last wave; below about six ions to a lane the fixed work costs more than
 // half-empty SMs (32,768 x 128, 26 ions: 3.0e11 on 32 lanes, 4.1e11 on 16,
 // 5.6e11 on 8, 6.0e11 on 4).
-float tile_max_fill(bool acc) { return acc ? 0.7f : 0.42f; }
+float tile_max_fill(bool acc) { return acc ? 0.7f : 0.5f; }
 
 TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max, bool acc)
 {
@@ -86,7 +95,7 @@ TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_
         int P = 32;
         while (P > 4) {
             const int64_t warps = rails * (P / 2) / 32;
-            const bool enough = warps >= 6000 || (mean / P < 6.0 && warps >= 2400);
+            const bool enough = warps >= (acc ? 3600 : 6000) || (mean / P < 6.0 && warps >= 2400);
             if (!enough || ion_rows(P / 2, L, open, n_max) == 0) break;
             P >>= 1;
         }
@@ -126,31 +135,44 @@ size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool per
     a.rcpZ = 65536u / (uint32_t)p.n_zones + 1u;
     ion_slack(a, p.electrodes == 1);
     a.cls_shift = persite && !acc ? 2 : 0;
-    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, persite, t.rcap, false, !acc);
+    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, persite, t.rcap, false, acc,
+                      p.update_rule != 0);
     return a.iy.tab + (size_t)warps * a.iy.bytes;
 }
 
-// Warps per CTA (at most `most`) of a launch over `warps` warps.  When all are
+// Warps per CTA of a launch over `warps` warps.  When all are
 // resident at once the launch takes as long as the fullest SM sub-partition: the
 // CTA size that leaves it the fewest warps, of equals the largest (4,000 warps of
 // 16,000 x 200 rails: 8 to a sub-partition and 2.94 ms in CTAs of 8, 7 and 2.60 ms
 // in CTAs of 7; 64 warps: 2 and 0.41 ms in CTAs of 8, 1 and 0.36 ms in CTAs of 4).
-// In more than one wave `most` (16,384 x 1,024: 6.8 ms in CTAs of 8, 6.8 of 4, 7.6
-// of 2, which repeat the site table more often).
-int ion_cta_warps(const SweepArgs &a, int64_t warps, int most)
+// In more than one wave 8 (16,384 x 1,024: 6.8 ms in CTAs of 8, 6.8 of 4, 7.6
+// of 2, which repeat the site table more often), or of the wide CTAs those that
+// hold the most warps on an SM.
+int ion_cta_warps(const SweepArgs &a, int kind, int64_t warps)
 {
-    int dev = 0, sms = 0, sm = 0;
+    int dev = 0, sms = 0, sm = 0, cta = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&cta, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (cta <= 0) cta = 48 * 1024;
     sms = std::max(sms, 1);
-    int best = most;
-    int64_t least = INT64_MAX;
-    for (int w = most; w >= 1; --w) {
-        const size_t smem = a.iy.tab + (size_t)w * a.iy.bytes + 1024;     // the system's 1 KB a CTA
-        const int64_t resident = std::min<int64_t>(32 / w, (int64_t)((size_t)std::max(sm, 1) / smem));
+    const bool wide = ion_wide(kind);
+    int best = 1;
+    int64_t least = INT64_MAX, most = 0;
+    for (int w = wide ? kIonWarps<uint64_t> : kIonWarps<uint32_t>; w >= 1; --w) {
+        const size_t smem = a.iy.tab + (size_t)w * a.iy.bytes;
+        if (smem > (size_t)std::min(cta, ion_most_smem(kind))) continue;
+        // the system takes 1 KB a CTA
+        const int64_t resident = std::min<int64_t>((wide ? 20 : 32) / w, std::max(sm, cta) / (int64_t)(smem + 1024));
         const int64_t per_sm = ((warps + w - 1) / w + sms - 1) / sms;
-        if (per_sm > resident) continue;
+        if (per_sm > resident) {
+            if (least == INT64_MAX && (wide ? resident * w : w) > most) {
+                most = wide ? resident * w : w;
+                best = w;
+            }
+            continue;
+        }
         const int64_t fullest = (per_sm * w + 3) / 4;
         if (fullest < least) {
             least = fullest;
@@ -225,7 +247,7 @@ size_t grad_tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, int
     if (!t.ions) return grad_smem_bytes(t.lpr, t.wpl, p.n_zones, p.n_sites, warps);
     a.rcap = t.rcap;
     a.rcpZ = 65536u / (uint32_t)p.n_zones + 1u;
-    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, false, t.rcap, true, false);
+    a.iy = ion_layout(t.lpr, p.n_zones, p.n_sites, p.electrodes == 1, false, t.rcap, true, true, p.update_rule != 0);
     return a.iy.tab + (size_t)warps * a.iy.bytes;
 }
 
@@ -234,10 +256,10 @@ cudaError_t ion_set_smem_limits()
     cudaError_t e = cudaSuccess;
     for (int k = kWordKinds; k < kShapeKinds; ++k)
         for (int acc = 0; acc < 2; ++acc) {
-            const cudaError_t r = with_ions(k, acc != 0, [](auto p, auto ac, auto open, auto m) {
+            const cudaError_t r = with_ions(k, acc != 0, [k](auto p, auto ac, auto open, auto m) {
                 return cudaFuncSetAttribute(
                     ion_kernel<decltype(p)::value, decltype(ac)::value, decltype(open)::value, decltype(m)>,
-                    cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+                    cudaFuncAttributeMaxDynamicSharedMemorySize, ion_most_smem(k));
             });
             if (r != cudaSuccess) e = r;
         }

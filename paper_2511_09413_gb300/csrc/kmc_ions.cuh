@@ -182,7 +182,8 @@ struct IonView {
     __device__ __forceinline__ float2 *p0b(int sg) const { return (float2 *)(sb + a.iy.p0b) + sg * a.Z; }
     __device__ __forceinline__ int32_t *Pb(int sg) const { return (int32_t *)(sb + a.iy.pb) + sg * (a.Z + 1); }
     __device__ __forceinline__ uint32_t &slot(int k) const { return ((uint32_t *)(sb + a.iy.st))[k * 32 + lane()]; }
-    // without the accept path: rows that may be accepted, per step drawn ahead
+    // without the accept path: rows that may be accepted, per step drawn ahead;
+    // with it and the even/odd rule: rows at odd positions
     // (kIonAhead words, as many again for the rows from 32 on)
     __device__ __forceinline__ uint32_t &hits(int k) const { return ((uint32_t *)(sb + a.iy.hit))[k * 32 + lane()]; }
     __device__ __forceinline__ uint32_t *col() const { return (uint32_t *)(sb + a.iy.col); }
@@ -449,6 +450,31 @@ __device__ __forceinline__ int ion_commit(const IonView<P, CLS> &c, const uint8_
         if (b < a.Z) atomicAdd(zc + b, (unsigned long long)(long long)m);
     }
     return b == 0 || b == a.Z ? 2 : 1;
+}
+
+// Under the even/odd rule with the accept path: the rows at odd positions.  A move
+// flips its row's bit, so they are formed anew only when rows come or go.
+template <int P, class M, bool CLS>
+__device__ __forceinline__ M ion_odd(const IonView<P, CLS> &c)
+{
+    M m = c.hits(0);
+    if (sizeof(M) > 4) m |= (M)c.hits(1) << (8 * sizeof(M) - 32);
+    return m;
+}
+template <int P, class M, bool CLS>
+__device__ __forceinline__ void ion_set_odd(const IonView<P, CLS> &c, M m)
+{
+    c.hits(0) = (uint32_t)m;
+    if (sizeof(M) > 4) c.hits(1) = (uint32_t)(m >> (8 * sizeof(M) - 32));
+}
+template <int P, class M, bool CLS>
+__device__ __forceinline__ void ion_parity(const IonView<P, CLS> &c)
+{
+    const int n = (int)c.slot(kSlotN);
+    M m = 0;
+    for (int r = 0; r < n; ++r)
+        if (pos_of(c.colp()[r * 32]) & 1) m |= M(1) << r;
+    ion_set_odd<P, M>(c, m);
 }
 
 // Zone z of rail slot sg as it stands (the field of S2.1.8, Eqs. 3-4) at the mid
@@ -1192,6 +1218,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
         const int sum = ion_sum<P>(c);
         if (sl == 0) c.Fs()[2 * G] = sum;
         __syncwarp();
+        if (ACC && a.rule != 0) ion_parity<P, M>(c);
         if constexpr (GRAD) ion_score_begin<P>(c);
     }
 
@@ -1269,9 +1296,8 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                     aR &= fR;
                     aL &= fL;
                     if (a.rule != 0) {
-                        M odd = 0;
-                        for (int r = 0; r < n; ++r)
-                            if ((pos_of(c.colp()[r * 32]) ^ (int)t) & 1) odd |= M(1) << r;
+                        M odd = ion_odd<P, M>(c);
+                        if (t & 1u) odd = ~odd;
                         aR &= ~odd;
                         aL &= odd;
                     }
@@ -1422,6 +1448,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                         }
                     }
                 }
+                if (ACC && a.rule != 0) ion_set_odd<P, M>(c, ion_odd<P, M>(c) ^ (aR | aL));
                 if constexpr (GRAD) {
                     ion_score_current<P>(c, t, nL - nR);
                 } else {
@@ -1443,6 +1470,10 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 uint32_t draws = 0u;
                 ends = ion_ends<P>(c, tab, sq, c.rail(tile_rail0), draws);
                 if (!GRAD && draws != 0u && c.lane() == 0) atomicAdd(&a.counters[0], (unsigned long long)draws);
+            }
+            if (ACC && OPEN && ends != 0 && a.rule != 0) {
+                const View c(a, smem);
+                ion_parity<P, M>(c);
             }
             if constexpr (ACC) {
                 // lanes to rail slots

@@ -254,7 +254,7 @@ extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t 
         while (l.warps > 1 && tile_args(a, t, *p, false, l.warps, acc) > (size_t)max_smem) l.warps >>= 1;
         if (t.ions) {
             tile_args(a, t, *p, false, l.warps, acc);
-            l.warps = ion_cta_warps(a, (R * (int64_t)t.lpr + 31) / 32, l.warps);
+            l.warps = ion_cta_warps(a, t.kind, (R * (int64_t)t.lpr + 31) / 32);
         }
         l.smem = tile_args(a, t, *p, false, l.warps, acc);
         const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * l.warps;

@@ -60,6 +60,15 @@ def test_shapes_of_the_lists(kmc, R, L, electrodes, dt):
     _check(kmc, dev, V, 0.25, [n // 3, n - n // 3])
 
 
+# more than 32 entries a lane: CTAs of up to 20 warps, in one wave and in several,
+# each with a last CTA that is not full
+@pytest.mark.parametrize("R,L,fill", [(2500, 2048, 0.5), (5001, 1100, 0.25)])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_wide_ctas(kmc, R, L, fill, dt):
+    dev = _dev(R=R, L=L, Z=32, electrodes=1, k_e=1.0 / dt, rho_e=0.3, dt=dt)
+    _check(kmc, dev, np.where(np.arange(9) % 6 < 3, 1.0, -0.5), fill, [4, 5])
+
+
 # open rails that fill up from empty, drain from half full, and swap their ions
 # at a high rate: entries come and go at both ends
 @pytest.mark.parametrize("L", [8, 33, 64, 200])
