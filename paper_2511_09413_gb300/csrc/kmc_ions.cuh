@@ -171,6 +171,8 @@ struct IonView {
         return e;
     }
     __device__ __forceinline__ float4 &band() const { return *(float4 *)sb; }
+    // with the accept path: the widest band of the bounds, in units of a draw's high word
+    __device__ __forceinline__ uint32_t &width() const { return *(uint32_t *)(sb + 12); }
     __device__ __forceinline__ int &kmax() const { return *(int *)(sb + 16); }
     __device__ __forceinline__ int &mark() const { return *(int *)(sb + 20); }
     // [0] F, [G] N0, [2 G] sum of positions
@@ -547,19 +549,23 @@ __device__ __forceinline__ int ion_window(const IonView<P, CLS> &c, int64_t t0, 
     return s + len;
 }
 
-// Decision bounds of the zones of the rail slots in `dirty` (bits).  Without ACC
+// Decision bounds of the zones of the rail slots in `dirty` (bits; `all`: of every
+// one).  With ACC they are upper bounds too, and the widest band between a bound and
+// the draws that are surely accepted is kept beside them: a draw nearer to its bound
+// than that is decided with its own zone and site.  Without ACC
 // they only tell which draws may be accepted, for any state of an end entry and
 // with room for a.ion_slack in the exponent, so that they hold while ions cross a
 // few boundaries (a.ion_budget); the draws below them are decided with ion_zone.
 __device__ __forceinline__ float ion_class(int k) { return __int_as_float((127 - k) << 23); }     // 2^-k
 template <int P, bool ACC, bool OPEN, bool CLS>
-__device__ __forceinline__ void ion_zones(const IonView<P, CLS> &c, uint32_t dirty)
+__device__ __forceinline__ void ion_zones(const IonView<P, CLS> &c, uint32_t dirty, bool all)
 {
     constexpr int G = 32 / P;
     const SweepArgs &a = c.a;
     const int Z = a.Z;
     __syncwarp();
     const int items = __popc(dirty) * Z;
+    uint32_t wide = 0u;
     for (int i = c.lane(); i < items; i += 32) {
         const int k = (int)(((uint32_t)i * a.rcpZ) >> 16), z = i - k * Z;    // i / Z for i < 1024
         uint32_t m = dirty;
@@ -609,41 +615,43 @@ __device__ __forceinline__ void ion_zones(const IonView<P, CLS> &c, uint32_t dir
             }
             continue;
         }
-        uint4 b = make_uint4(FULL, FULL, 0u, 0u);
+        const float sm = fmaxf(r.sR, r.inv);
+        uint2 b = make_uint2(FULL, FULL);
+        uint32_t w = FULL;
         if (r.ok) {
-            b.x = rej_thr(bhi * r.sR * r.hi);
-            b.y = rej_thr(bhi * r.inv * r.hi);
-            b.z = acc_thr(blo * r.sR * r.lo);
-            b.w = acc_thr(blo * r.inv * r.lo);
+            b = make_uint2(rej_thr(bhi * r.sR * r.hi), rej_thr(bhi * r.inv * r.hi));
+            w = rej_thr(bhi * sm * r.hi) - acc_thr(blo * sm * r.lo) + 2u;
         }
-        *(uint4 *)rm = b;
+        *(uint2 *)rm = b;
         if (OPEN && (z == 0 || z == Z - 1)) {
             // electrode positions: outward trials are extractions, the virtual
             // sites' inward trials injections
-            const float Ein = a.E_inf, Eout = a.E_outf;
+            const float Ein = a.E_inf, Eout = a.E_outf, Em = fmaxf(Ein, Eout) * sm;
+            if (r.ok) w = max(w, rej_thr(Em * r.hi) - acc_thr(Em * r.lo) + 2u);
             if (z == 0) {
-                uint4 e = b, q = b;
+                uint2 in = b, out = b;
                 if (r.ok) {
-                    e.x = rej_thr(Ein * r.sR * r.hi);
-                    e.z = acc_thr(Ein * r.sR * r.lo);
-                    q.y = rej_thr(Eout * r.inv * r.hi);
-                    q.w = acc_thr(Eout * r.inv * r.lo);
+                    in.x = rej_thr(Ein * r.sR * r.hi);
+                    out.y = rej_thr(Eout * r.inv * r.hi);
                 }
-                *(uint4 *)ends = e;
-                *(uint4 *)(ends + 16) = q;
+                *(uint2 *)ends = in;
+                *(uint2 *)(ends + 16) = out;
             }
             if (z == Z - 1) {
-                uint4 e = b, q = b;
+                uint2 in = b, out = b;
                 if (r.ok) {
-                    e.y = rej_thr(Ein * r.inv * r.hi);
-                    e.w = acc_thr(Ein * r.inv * r.lo);
-                    q.x = rej_thr(Eout * r.sR * r.hi);
-                    q.z = acc_thr(Eout * r.sR * r.lo);
+                    in.y = rej_thr(Ein * r.inv * r.hi);
+                    out.x = rej_thr(Eout * r.sR * r.hi);
                 }
-                *(uint4 *)(ends + 32) = q;
-                *(uint4 *)(ends + 48) = e;
+                *(uint2 *)(ends + 32) = out;
+                *(uint2 *)(ends + 48) = in;
             }
         }
+        wide = max(wide, w);
+    }
+    if constexpr (ACC) {
+        wide = __reduce_max_sync(FULL, wide);
+        if (c.lane() == 0) c.width() = all ? wide : max(wide, c.width());
     }
     __syncwarp();
 }
@@ -1134,9 +1142,13 @@ __device__ __forceinline__ void ion_score_end(const IonView<P, CLS> &c, int64_t 
 // [tile_rail0, tile_rail0 + G * warps).  The draw loop only compares each
 // entry's two words with its bounds and keeps the outcomes as bits of M, one
 // per row.  With ACC (hop probabilities of order 1e-2 and above, several
-// accepted draws per warp and step) it also compares with the lower bounds and
-// keeps which neighbours are one and two sites away, so that exclusion and
-// conflicts are a few operations on bits; without, the entries with a word
+// accepted draws per warp and step) it also keeps the least distance of a draw
+// below its bound and which neighbours are one and two sites away, so that exclusion
+// and conflicts are a few operations on bits.  That loop takes 100 cycles a row on a
+// sub-partition, 69 of the multiplier and 73 of the ALU pipe; so an entry's halves
+// are two loads instead of a mask and a shift, and the distance stands for the
+// comparisons with two lower bounds (65,536 rails of 512 sites, 20 % full: 8.8 ->
+// 8.4 ms for 300 steps).  Without ACC, the entries with a word
 // below its upper bound are looked at one by one, and as moves are rare the loop
 // draws for kIonAhead steps at once: an entry is loaded once for four draws, and the
 // four chains hide each other's latency.  An ion that moves is drawn for again for
@@ -1234,7 +1246,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             if (dirty != 0u || window) {
                 const View c(a, smem);
                 if (window) wend = ion_window<P>(c, t0, s, n_steps);
-                ion_zones<P, ACC, OPEN>(c, window ? (uint32_t)((1ull << G) - 1u) : dirty);
+                ion_zones<P, ACC, OPEN>(c, window ? (uint32_t)((1ull << G) - 1u) : dirty, window);
                 spent = 0;
             }
             const uint32_t stale = GRAD ? dirty : 0u;   // rail slots to score anew
@@ -1254,25 +1266,24 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 const uint32_t *const end = cp + c.kmax() * 32;
                 if constexpr (ACC) {
                     const StepDraw sd = step_draw(t, prail, rk0, rk1);
-                    M sR = 0, sL = 0, one = 0;
-                    uint32_t e = *cp;
+                    M one = 0;
+                    uint32_t e = *(const uint16_t *)cp, least = FULL;    // distance of a draw below its bound
                     for (int half = 0; half < (int)sizeof(M) / 4 && cp != end; ++half) {
                         // 32 rows at a time, their bits in one register each
                         const uint32_t *const to = end - cp > 32 * 32 ? cp + 32 * 32 : end;
-                        uint32_t hR = 0u, hL = 0u, kR = 0u, kL = 0u, g1 = 0u, g2 = 0u, bit = 1u;
+                        uint32_t hR = 0u, hL = 0u, g1 = 0u, g2 = 0u, bit = 1u;
 #pragma unroll 4
                         while (cp != to) {
+                            const uint2 th = *(const uint2 *)(rm + ((const uint16_t *)cp)[1]);
                             cp += 32;
-                            const uint32_t en = *cp;    // the column has one slot more than rows in use
-                            const uint32_t gap = (en & 0xFFFFu) - (e & 0xFFFFu);
-                            const uint4 w = site_at(tab, e);
+                            const uint32_t en = *(const uint16_t *)cp;  // the column has one slot more than rows in use
+                            const uint32_t gap = en - e;
+                            const uint4 w = *(const uint4 *)(tab + e);
                             uint32_t xy, xw;
                             site_draw(sd, w.x, w.y, w.z, rk0, rk1, xy, xw);
-                            const uint4 th = *(const uint4 *)(rm + (e >> 16));
                             if (xy <= th.x) hR |= bit;
                             if (xw <= th.y) hL |= bit;
-                            if (xy < th.z) kR |= bit;
-                            if (xw < th.w) kL |= bit;
+                            least = min(least, min(th.x - xy, th.y - xw));
                             if (gap == 1u * kStep) g1 |= bit;
                             if (gap == 2u * kStep) g2 |= bit;
                             bit <<= 1;
@@ -1280,8 +1291,6 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                         }
                         aR |= (M)hR << (32 * half);
                         aL |= (M)hL << (32 * half);
-                        sR |= (M)kR << (32 * half);
-                        sL |= (M)kL << (32 * half);
                         one |= (M)g1 << (32 * half);
                         two |= (M)g2 << (32 * half);
                     }
@@ -1301,7 +1310,8 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                         aR &= ~odd;
                         aL &= odd;
                     }
-                    und = (aR & ~sR) | (aL & ~sL);
+                    // some draw is within a bound's band: all that may be accepted are looked at
+                    und = least <= c.width() ? aR | aL : 0;
                 } else {
                     StepDraw sd[kIonAhead];
 #pragma unroll
