@@ -186,6 +186,7 @@ void fill_args(kmc_handle *h)
     a.P0site = h->P0site;
     a.P0f = h->P0f;
     a.P0bnd = h->P0bnd;
+    a.order = h->order;
     a.P0cls = h->P0bnd ? (const uint32_t *)(h->P0bnd + (int64_t)p.n_rails * p.n_zones) : nullptr;
     a.bgd = h->bgd;
     a.K = h->K;
@@ -289,13 +290,17 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
     const size_t occ_bytes = (size_t)(R * h->stride);
     h->occ = (uint8_t *)h->alloc(occ_bytes);
     h->V = (double *)h->alloc(sizeof(double) * (size_t)std::max<int64_t>(n_total, 1));
-    h->N0 = (int32_t *)h->alloc(sizeof(int32_t) * (size_t)R);
+    // the ion counts, and for the devices that fill the GPU the rails' order by them,
+    // formed with two words per count behind misc
+    const bool ordered = R >= 1024;
+    h->N0 = (int32_t *)h->alloc(sizeof(int32_t) * (size_t)(ordered ? 2 * R : R));
     h->K = (DevConst *)h->alloc(sizeof(DevConst));
     h->J = (unsigned long long *)h->alloc(sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1));
     h->Zc = (unsigned long long *)h->alloc(sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1) *
                                            (size_t)Z);
     h->log = (kmc_log_entry *)h->alloc(sizeof(kmc_log_entry) * (size_t)h->log_cap);
-    h->misc = (unsigned long long *)h->alloc(sizeof(unsigned long long) * 16);
+    const size_t misc_bytes = sizeof(unsigned long long) * 16, bin_bytes = ordered ? sizeof(int32_t) * 2 * (size_t)(L + 1) : 0;
+    h->misc = (unsigned long long *)h->alloc(misc_bytes + bin_bytes);
     h->args_dev = (SweepArgs *)h->alloc(sizeof(SweepArgs));
     h->occ_init = (uint8_t *)h->alloc(occ_bytes);
     h->Jr = (int64_t *)h->alloc(sizeof(int64_t) * (size_t)R);
@@ -311,7 +316,7 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
             return fail(KMC_E_NOMEM, "device allocation failed (P0 table)");
     }
     cudaStream_t s = h->stream;
-    CK(cudaMemsetAsync(h->misc, 0, sizeof(unsigned long long) * 16, s), "memset");
+    CK(cudaMemsetAsync(h->misc, 0, misc_bytes + bin_bytes, s), "memset");
     CK(cudaMemsetAsync(h->J, 0, sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1), s), "memset");
     CK(cudaMemsetAsync(h->Zc, 0, sizeof(int64_t) * (size_t)std::max<int64_t>(n_total, 1) * (size_t)Z, s),
        "memset");
@@ -334,9 +339,14 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         if (rc) return rc;
     }
     unsigned long long *bad = h->misc + 5;
+    int32_t *const bins = ordered ? (int32_t *)(h->misc + 16) : nullptr;
     CK(setup_row_counts(h->occ, h->stride, (int32_t)R, (int32_t)L, h->N0, bad, h->misc + 8,
-                        s),
+                        bins, s),
        "row counts");
+    if (ordered) {
+        h->order = h->N0 + R;
+        CK(setup_order(h->N0, (int32_t)R, (int32_t)L, bins, bins + L + 1, h->order, s), "rail order");
+    }
     CK(setup_background(h->N0, (int32_t)R, (int32_t)L, (int32_t)Z, h->K, h->bgd, s), "background");
     CK(cudaMemcpyAsync(h->occ_init, h->occ, occ_bytes, cudaMemcpyDeviceToDevice, s), "checkpoint");
 

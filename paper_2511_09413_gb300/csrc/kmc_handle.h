@@ -33,6 +33,7 @@ struct kmc_handle {
     uint8_t *occ = nullptr;
     double *V = nullptr;
     int32_t *N0 = nullptr;
+    int32_t *order = nullptr;                 // rails by falling ion count, or null
     double *P0site = nullptr;
     float *P0f = nullptr;
     float2 *P0bnd = nullptr;

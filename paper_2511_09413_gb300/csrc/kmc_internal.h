@@ -63,6 +63,7 @@ struct SweepArgs {
     const float *P0f;          // [R][L] P0site rounded to FP32, or null
     const float2 *P0bnd;       // [R][Z] (min, max) of P0site over the zone, or null
     const uint32_t *P0cls;     // [R][(L + 15) / 16] classes of P0f against the zone's max, 2 bits a site
+    const int32_t *order;      // [R] the rails by falling ion count (ion lists), or null
     int32_t cls_shift;         // ion lists: 2 with classes, else 0
     const double2 *bgd;        // [R][Z] (N0 w_z / L, D'_z) in FP64 for the FP64 paths, or null
     const DevConst *K;
@@ -269,11 +270,13 @@ cudaError_t setup_p0_float(const double *P0, int64_t n, float *out, cudaStream_t
 // ions of each rail; with stats, also their total (stats[0]) and the largest (stats[1])
 cudaError_t setup_row_counts(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
                              int32_t *N0, unsigned long long *bad, unsigned long long *stats,
-                             cudaStream_t s);
+                             int32_t *bins, cudaStream_t s);
 // bgd[r][z] = (N0[r] w_z / L in the oracle's FP64 order, D'_z): the background
 // of zone z of rail r and its part of Q_z - Qbar (S2.1.8 reading)
 cudaError_t setup_background(const int32_t *N0, int32_t R, int32_t L, int32_t Z, const DevConst *K,
                              double2 *bgd, cudaStream_t s);
+cudaError_t setup_order(const int32_t *N0, int32_t R, int32_t L, const int32_t *bins, int32_t *next, int32_t *order,
+                        cudaStream_t s);
 cudaError_t setup_init_bernoulli(const kmc_params &p, uint8_t *occ, int64_t stride,
                                  cudaStream_t s);
 // mode 0: count init keys <= key_bound; mode 1: keys == key_bound with linear index <= idx_bound

@@ -111,10 +111,10 @@ __device__ __forceinline__ uint4 site_at(const uint8_t *tab, uint32_t e) { retur
 // A warp's block: header of 64 bytes (band factor and mid voltage of the voltage
 // window float [2], the largest column, the step up to which draws are counted;
 // in the gradient pass the doubles of IonScore from byte 24 on),
-// int [G] each of F, N0 and the sum of positions that the per-rail current
-// counts from, then the bounds.
+// int [G] each of F, N0, the sum of positions that the per-rail current counts
+// from, and the rail, then the bounds.
 constexpr uint32_t kIonHead = 64u;
-__host__ __device__ constexpr uint32_t ion_fixed(int P) { return kIonHead + (uint32_t)align16(12u * (32u / (uint32_t)P)); }
+__host__ __device__ constexpr uint32_t ion_fixed(int P) { return kIonHead + 16u * (32u / (uint32_t)P); }
 // per-lane words ([kIonSlots][32]): entries of the column; distances from its
 // first entry to the one before (low half) and from its last to the one after
 // (high half), on the neighbouring lanes or the rail's ends; moves since the
@@ -149,7 +149,9 @@ struct IonView {
     __device__ __forceinline__ int lane() const { return (int)(tid & 31u); }
     __device__ __forceinline__ int seg() const { return (int)(tid & 31u) / P; }
     __device__ __forceinline__ int sl() const { return (int)(tid & (P - 1)); }
-    __device__ __forceinline__ int64_t rail(int64_t tile_rail0) const { return tile_rail0 + (int64_t)(tid >> 5) * G + seg(); }
+    // the lane's place in the tiles' order of rails, and its rail
+    __device__ __forceinline__ int64_t place(int64_t tile_rail0) const { return tile_rail0 + (int64_t)(tid >> 5) * G + seg(); }
+    __device__ __forceinline__ int64_t rail() const { return (int64_t)Fs()[3 * G]; }
     __device__ __forceinline__ int cls() const { return CLS ? a.cls_shift : 0; }
     // zone code of an entry: z + 1, and 0 / Z + 1 for the virtual sites -1 / L
     __device__ __forceinline__ int code(uint32_t e) const
@@ -175,7 +177,7 @@ struct IonView {
     __device__ __forceinline__ uint32_t &width() const { return *(uint32_t *)(sb + 12); }
     __device__ __forceinline__ int &kmax() const { return *(int *)(sb + 16); }
     __device__ __forceinline__ int &mark() const { return *(int *)(sb + 20); }
-    // [0] F, [G] N0, [2 G] sum of positions
+    // [0] F, [G] N0, [2 G] sum of positions, [3 G] rail (a.R: none)
     __device__ __forceinline__ int32_t *Fs(int sg) const { return (int32_t *)(sb + kIonHead) + sg; }
     __device__ __forceinline__ int32_t *Fs() const { return Fs(seg()); }
     __device__ __forceinline__ uint8_t *bounds(int sg) const { return sb + ion_fixed(P) + sg * (int)a.iy.row; }
@@ -1159,6 +1161,11 @@ __device__ __forceinline__ void ion_score_end(const IonView<P, CLS> &c, int64_t 
 // per-site barriers 60 -> 50 ms.  GRAD: the gradient pass, which
 // replays the sweep from its first occupancy with the score accumulated instead
 // of the traces.
+//
+// The lanes of a warp go through as many rows as its fullest lane, so the rails that
+// share a warp should hold equally many ions: a.order lists them by their first
+// occupancy's counts, the fullest first (65,536 rails of 512 sites, 102 +- 9 ions, 8
+// to a warp: 29 rows on average in the order of their indices, 26 in this one).
 template <int P, bool ACC, bool OPEN, class M, bool GRAD = false>
 __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0, const uint32_t *rk1,
                                          int64_t t0, int n_steps, int flush, int64_t tile_rail0,
@@ -1171,8 +1178,9 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
     {
         const View c(a, smem);
         const int L = a.L, Z = a.Z, sl = c.sl();
-        const int64_t rail = c.rail(tile_rail0);
-        const bool active = rail < a.R;
+        const int64_t place = c.place(tile_rail0);
+        const bool active = place < a.R;
+        const int64_t rail = !active ? a.R : a.order != nullptr ? a.order[place] : place;
         // ---- site table of the CTA
         for (int i = (int)c.tid; i < L + 2; i += blockDim.x) {
             const int k = min(max(i - 1, 0), L - 1);
@@ -1199,14 +1207,17 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             }
             words[w] = bits;
         }
-        if (sl == 0) c.Fs()[G] = active ? a.N0[rail] : 0;
+        if (sl == 0) {
+            c.Fs()[G] = active ? a.N0[rail] : 0;
+            c.Fs()[3 * G] = (int32_t)rail;
+        }
         if (a.P0bnd != nullptr)
             for (int z = sl; z < Z; z += P)
                 c.p0b(c.seg())[z] = active ? a.P0bnd[rail * Z + z] : make_float2(0.0f, 0.0f);
         c.slot(kSlotMoves) = 0u;
         if (c.lane() == 0) c.mark() = 0;
         __syncthreads();
-        if (rail - c.seg() >= a.R) return;
+        if (place - c.seg() >= a.R) return;
         // ---- ions below each zone boundary and F
         for (int b = sl; b <= Z; b += P) {
             const int e = a.bnd[b];
@@ -1260,7 +1271,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             uint32_t look = 0u, ends_at = 0u;   // without ACC: steps with a draw that may be accepted, exchanges
             {
                 const View c(a, smem);
-                const uint32_t prail = a.rail_base + (uint32_t)c.rail(tile_rail0);
+                const uint32_t prail = a.rail_base + (uint32_t)c.rail();
                 const uint8_t *rm = c.bounds();
                 const uint32_t *cp = c.colp();
                 const uint32_t *const end = cp + c.kmax() * 32;
@@ -1369,7 +1380,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 M left = 0;
                 {
                     const View c(a, smem);
-                    const int64_t rail = c.rail(tile_rail0);
+                    const int64_t rail = c.rail();
                     const StepDraw sd = step_draw(tq, a.rail_base + (uint32_t)rail, rk0, rk1);
                     const int n = (int)c.slot(kSlotN);
                     const uint32_t gaps = c.slot(kSlotGaps);
@@ -1395,7 +1406,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                         const IonEntry en = ion_entry(c.colp(), first_bit(left), (int)c.slot(kSlotN),
                                                      c.slot(kSlotGaps), a.rule, tq);
                         int dR = en.fR ? 2 : 0, dL = en.fL ? 2 : 0;
-                        ion_exact<P>(c, c.seg(), c.rail(tile_rail0), en.x, c.zone(en.e), tq, dR, dL);
+                        ion_exact<P>(c, c.seg(), c.rail(), en.x, c.zone(en.e), tq, dR, dL);
                         aR = dR == 1 ? aR | bit : aR & ~bit;
                         aL = dL == 1 ? aL | bit : aL & ~bit;
                     }
@@ -1436,7 +1447,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 uint32_t *colp = c.colp();
                 for (M todo = aR | aL; todo; todo &= todo - 1) {
                     const int j = first_bit(todo);
-                    const int r = ion_commit<P>(c, tab, c.rail(tile_rail0), colp + j * 32, colp[j * 32], (aR >> j) & 1 ? 1 : -1,
+                    const int r = ion_commit<P>(c, tab, c.rail(), colp + j * 32, colp[j * 32], (aR >> j) & 1 ? 1 : -1,
                                                 !GRAD && sq + 1 < n_steps ? a.Zc + (t0 + sq + 1) * a.Z : nullptr);
                     if constexpr (ACC) {
                         crossings += r != 0 ? 1 : 0;
@@ -1444,7 +1455,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                         crossings += r == 2 ? a.ion_exchange : r;
                         if (r == 2) continue;
                         inner = true;
-                        const uint32_t e = colp[j * 32], prail = a.rail_base + (uint32_t)c.rail(tile_rail0);
+                        const uint32_t e = colp[j * 32], prail = a.rail_base + (uint32_t)c.rail();
                         const uint4 w = site_at(tab, e);
                         const uint2 th = *(const uint2 *)(c.bounds() + (e >> 16));
 #pragma unroll 1
@@ -1478,7 +1489,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
             if (OPEN && (ACC || inner)) {
                 const View c(a, smem);
                 uint32_t draws = 0u;
-                ends = ion_ends<P>(c, tab, sq, c.rail(tile_rail0), draws);
+                ends = ion_ends<P>(c, tab, sq, c.rail(), draws);
                 if (!GRAD && draws != 0u && c.lane() == 0) atomicAdd(&a.counters[0], (unsigned long long)draws);
             }
             if (ACC && OPEN && ends != 0 && a.rule != 0) {
@@ -1517,7 +1528,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 c.mark() = c1;
             }
             c.slot(kSlotMoves) = 0u;
-            const int64_t rail = c.rail(tile_rail0);
+            const int64_t rail = c.rail();
             if (c.sl() == 0) {
                 const int v = c.Fs()[2 * G] - sum;
                 c.Fs()[2 * G] = sum;
@@ -1529,7 +1540,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
 
     if constexpr (GRAD) {
         const View c(a, smem);
-        ion_score_end<P>(c, c.rail(tile_rail0));
+        ion_score_end<P>(c, c.rail());
         return;
     }
     // ---- write the rails back
@@ -1539,7 +1550,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
         const int W = (a.L + 31) >> 5, C = (W + P - 1) / P;
         const int w0 = min(c.sl() * C, W), w1 = min(w0 + C, W);
         const uint32_t *words = c.words() + c.seg() * W;
-        const int64_t rail = c.rail(tile_rail0);
+        const int64_t rail = c.rail();
         if (rail < a.R)
             for (int w = w0; w < w1; ++w) {
                 const uint32_t o = words[w];

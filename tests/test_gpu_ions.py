@@ -96,6 +96,30 @@ def test_rare_moves(kmc, L, Z, electrodes, kappa, spread, rule):
     _check(kmc, dev, V, 0.3, [1, 2, 3, 261, 336], Ea)
 
 
+# rails that share a warp are taken in the order of their ion counts: empty, full
+# and uneven ones, with places beyond the last rail, and a count per rail that must
+# come back at the rail's own index
+@pytest.mark.parametrize("R", [1023, 1024, 1025, 4099])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_uneven_rails(kmc, R, electrodes, dt):
+    L = 75
+    dev = _dev(R=R, L=L, electrodes=electrodes, k_e=1.0 / dt if electrodes else 0.0, rho_e=0.3, dt=dt)
+    rng = np.random.default_rng(R)
+    share = rng.choice([0.0, 0.02, 0.2, 0.5, 1.0], size=R, p=[0.1, 0.3, 0.4, 0.15, 0.05])
+    occ0 = (rng.random((R, L)) < share[:, None]).astype(np.uint8)
+    V = np.where(np.arange(40) % 6 < 3, 1.0, -0.5)
+    sim = kmc.Sim(dev, V, 2, occ0=occ0)
+    orc = oracle.OracleSim(dev, V, occ0, None)
+    sim.step_n(40)
+    Jo, Zo = orc.step_n(40)
+    Jg, Zg = sim.traces()
+    assert np.array_equal(Zg, Zo) and np.array_equal(Jg, Jo)
+    assert np.array_equal(sim.occupancy(), orc.occ)
+    assert np.array_equal(sim.rail_current(), orc.J_rail)
+    sim.close()
+
+
 # a batch chooses its tiles from all rails together: the same devices alone
 # and together give the same results, lists and words side by side
 def test_batch_of_lists_and_words(kmc):
