@@ -40,7 +40,7 @@ struct IonLayout {
     uint32_t p0b;     // float2 [G][Z]: per-site P0 bounds of the zone (per-site barriers)
     uint32_t pb;      // int [G][Z + 1]: ions below each zone boundary
     uint32_t st;      // uint32 [slots][32]: each lane's state words
-    uint32_t hit;     // uint32 [0 .. 8][32]: outcome bits of the steps drawn ahead (no accept path), or rows at odd positions
+    uint32_t hit;     // uint32 [0 .. 16][32]: outcome bits of the steps drawn ahead (no accept path), or rows at odd positions
     uint32_t g;       // gradient pass: its sums, counts and factors (IonView)
     uint32_t col;     // uint32 [rcap][32]: each lane's entries
     uint32_t bytes;   // one warp's block

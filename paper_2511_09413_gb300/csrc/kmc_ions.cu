@@ -23,13 +23,13 @@ bool ion_wide(int kind) { return kind >= kWordKinds + 8; }
 int ion_most_smem(int kind) { return ion_wide(kind) ? kGradSmem : 200 * 1024; }
 template <class M>
 constexpr int kIonWarps = sizeof(M) > 4 ? 20 : 8;
-template <int P, bool ACC, bool OPEN, class M>
+template <int P, bool ACC, bool OPEN, class M, int AHEAD = OPEN ? kIonAhead : 4>
 __global__ void __launch_bounds__(32 * kIonWarps<M>, sizeof(M) > 4 ? 1 : 4) ion_kernel(const __grid_constant__ SweepArgs a, const int *gate)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     if (gate && *gate != 0) return;     // the occupancy words advance this device
     const int64_t tile_rail0 = (int64_t)blockIdx.x * (blockDim.x >> 5) * (32 / P);
-    ion_tile<P, ACC, OPEN, M>(a, a.rk0, a.rk1, a.t0, a.n_steps, a.flush, tile_rail0, smem);
+    ion_tile<P, ACC, OPEN, M, false, AHEAD>(a, a.rk0, a.rk1, a.t0, a.n_steps, a.flush, tile_rail0, smem);
 }
 
 // Slots of a lane's column, two more than the rows its bits can count (one that
@@ -49,6 +49,9 @@ int ion_rows(int P, int L, bool open, int64_t n_max)
 
 }  // namespace
 
+// Blocking rails on 32 lanes with at most four ions to a lane (two slots more)
+static bool ion_few(int P, bool open, int rcap) { return P == 32 && !open && rcap <= 6; }
+
 IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, bool grad, bool acc, bool rule)
 {
     const uint32_t G = 32u / (uint32_t)P, rows = ((uint32_t)Z << (persite && !acc ? 2 : 0)) + (open ? 5u : 1u);
@@ -62,7 +65,7 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
     y.pb = y.p0b + (persite ? (uint32_t)align16(8u * gz) : 0u);
     y.st = y.pb + pz;
     y.hit = y.st + 128u * kIonSlots;
-    y.g = y.hit + 128u * (acc ? (rule ? 1u : 0u) : (uint32_t)kIonAhead) * (grad || rcap > 34 ? 2u : 1u);
+    y.g = y.hit + 128u * (acc ? (rule ? 1u : 0u) : open || ion_few(P, open, rcap) ? (uint32_t)kIonAhead : 4u) * (grad || rcap > 34 ? 2u : 1u);
     y.col = y.g + (grad ? 2688u + 64u * G + (uint32_t)align16(8u * G * (uint32_t)(Z + 1)) + 48u * gz : 0u);
     y.bytes = y.col + (uint32_t)rcap * 128u;
     return y;
@@ -253,7 +256,8 @@ size_t grad_tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, int
 
 cudaError_t ion_set_smem_limits()
 {
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(ion_kernel<32, false, false, uint32_t, kIonAhead>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, ion_most_smem(kWordKinds));
     for (int k = kWordKinds; k < kShapeKinds; ++k)
         for (int acc = 0; acc < 2; ++acc) {
             const cudaError_t r = with_ions(k, acc != 0, [k](auto p, auto ac, auto open, auto m) {
@@ -269,6 +273,10 @@ cudaError_t ion_set_smem_limits()
 
 cudaError_t ion_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s)
 {
+    if (!l.acc && ion_few(l.lpr, a.electrodes == 1, a.rcap)) {
+        ion_kernel<32, false, false, uint32_t, kIonAhead><<<l.grid, l.warps * 32, l.smem, s>>>(a, gate);
+        return cudaGetLastError();
+    }
     return with_ions(l.kind, l.acc != 0, [&](auto p, auto acc, auto open, auto m) {
         ion_kernel<decltype(p)::value, decltype(acc)::value, decltype(open)::value, decltype(m)>
             <<<l.grid, l.warps * 32, l.smem, s>>>(a, gate);

@@ -120,7 +120,7 @@ __host__ __device__ constexpr uint32_t ion_fixed(int P) { return kIonHead + 16u 
 // (high half), on the neighbouring lanes or the rail's ends; moves since the
 // last flush
 enum { kSlotN = 0, kSlotGaps = 1, kSlotMoves = 2, kIonSlots = 3 };
-constexpr int kIonAhead = 4;       // steps drawn for at once without the accept path
+constexpr int kIonAhead = 8;       // steps drawn ahead without the accept path at most, four at a time
 
 // The thread index, read anew.  Each phase of a step forms its addresses from
 // it and takes its state from shared memory, so that no phase's registers are
@@ -685,7 +685,7 @@ __device__ __forceinline__ void ion_decide(const IonView<P, CLS> &c, const IonEn
 // concern its end entries only, which then step in and out in turn.  ion_end_draws
 // draws for both ends over the next kIonAhead steps, one lane to an end and step;
 // its result, on the lane that holds the end entry: bits q of a step where an
-// injection may (0..3) or surely will (4..7) be accepted, and an extraction (8..15).
+// injection may (0..7) or surely will (8..15) be accepted, and an extraction (16..31).
 template <int P, bool CLS>
 __device__ __forceinline__ bool ion_end(const IonView<P, CLS> &c, bool &left, uint32_t *&at)
 {
@@ -705,11 +705,12 @@ __device__ __forceinline__ uint32_t ion_end_draws(const IonView<P, CLS> &c, cons
     uint32_t *at;
     bool left;
     const bool own = ion_end<P>(c, left, at);
-    uint32_t r = 0u;
+    uint32_t f[4] = {};     // 16 bits each: the left end's steps, the right end's
 #pragma unroll
-    for (int pass = 0; pass < (P >= 8 ? 1 : 2); ++pass) {
-        const bool right = P >= 8 ? (c.sl() & 4) != 0 : pass != 0;
-        const uint32_t tk = t + (uint32_t)(c.sl() & 3);
+    for (int pass = 0; pass < (P >= 16 ? 1 : 16 / P); ++pass) {
+        const int ci = pass * P + (c.sl() & 15);
+        const bool right = (ci & 8) != 0;
+        const uint32_t tk = t + (uint32_t)(ci & 7);
         const uint4 w = site_at(tab, (uint32_t)(right ? a.L : 1) * kStep);
         uint32_t xy, xw;
         site_draw(step_draw(tk, prail, rk0, rk1), w.x, w.y, w.z, rk0, rk1, xy, xw);
@@ -718,13 +719,16 @@ __device__ __forceinline__ uint32_t ion_end_draws(const IonView<P, CLS> &c, cons
         const uint32_t xi = right ? xw : xy, xo = right ? xy : xw;
         // the even/odd rule: the bond right of x is active when x = t (mod 2)
         const bool act = a.rule == 0 || (((uint32_t)(right ? a.L - 1 : -1) ^ tk) & 1u) == 0u;
-        const uint32_t b0 = __ballot_sync(FULL, act && xi <= in.x), b1 = __ballot_sync(FULL, act && xi < in.y);
-        const uint32_t b2 = __ballot_sync(FULL, act && xo <= out.x), b3 = __ballot_sync(FULL, act && xo < out.y);
-        const int sh = c.lane() - c.sl() + (P >= 8 && !left ? 4 : 0);
-        if (own && (P >= 8 || left == (pass == 0)))
-            r = ((b0 >> sh) & 15u) | ((b1 >> sh) & 15u) << 4 | ((b2 >> sh) & 15u) << 8 | ((b3 >> sh) & 15u) << 12;
+        const int sh = c.lane() - c.sl();
+        constexpr uint32_t mine = P >= 16 ? 0xFFFFu : (1u << P) - 1u;
+        f[0] |= ((__ballot_sync(FULL, act && xi <= in.x) >> sh) & mine) << (pass * P);
+        f[1] |= ((__ballot_sync(FULL, act && xi < in.y) >> sh) & mine) << (pass * P);
+        f[2] |= ((__ballot_sync(FULL, act && xo <= out.x) >> sh) & mine) << (pass * P);
+        f[3] |= ((__ballot_sync(FULL, act && xo < out.y) >> sh) & mine) << (pass * P);
     }
-    return r;
+    const int sh = left ? 0 : 8;
+    const uint32_t r = ((f[0] >> sh) & 255u) | ((f[1] >> sh) & 255u) << 8 | ((f[2] >> sh) & 255u) << 16 | ((f[3] >> sh) & 255u) << 24;
+    return own ? r : 0u;
 }
 // Steps q .. stop - 1 (after step s of the launch), in which nothing but exchanges
 // can happen: carries them out, up to the first one that is not sure, and returns
@@ -745,8 +749,8 @@ __device__ __forceinline__ int ion_exchanges(const IonView<P, CLS> &c, const uin
     if (bits != 0u) {
         bool o = full;
         for (int k = q; k < stop; ++k) {
-            const uint32_t b = bits >> (k + (o ? 8 : 0));
-            if ((b & 0x11u) == 0x1u) {
+            const uint32_t b = bits >> (k + (o ? 16 : 0));
+            if ((b & 0x101u) == 0x1u) {
                 mine = k;
                 break;
             }
@@ -784,7 +788,7 @@ __device__ __forceinline__ int ion_exchanges(const IonView<P, CLS> &c, const uin
     }
     if (own) {
         const bool o = full != ((__popc(moved) & 1) != 0);
-        if ((bits >> (stop + (o ? 8 : 0))) & 1u) und = left ? M(1) : M(1) << ((int)c.slot(kSlotN) - 1);
+        if (stop < kIonAhead && ((bits >> (stop + (o ? 16 : 0))) & 1u) != 0u) und = left ? M(1) : M(1) << ((int)c.slot(kSlotN) - 1);
     }
     return stop;
 }
@@ -1152,11 +1156,14 @@ __device__ __forceinline__ void ion_score_end(const IonView<P, CLS> &c, int64_t 
 // comparisons with two lower bounds (65,536 rails of 512 sites, 20 % full: 8.8 ->
 // 8.4 ms for 300 steps).  Without ACC, the entries with a word
 // below its upper bound are looked at one by one, and as moves are rare the loop
-// draws for kIonAhead steps at once: an entry is loaded once for four draws, and the
-// four chains hide each other's latency.  An ion that moves is drawn for again for
+// draws for four steps at once: an entry is loaded once for four draws, and the four
+// chains hide each other's latency.  AHEAD: twice four on open rails (16,384 x 1,024:
+// 6.7 -> 6.5 ms) and where a lane holds four ions at most (64 x 100: 0.36 -> 0.32 ms),
+// once on others, where every ion that moves is drawn for again for the steps left
+// (8,192 x 1,000 30 % full: 1.21 -> 1.23 ms for twice).  An ion that moves is drawn for again for
 // the steps left.  Steps with nothing but exchanges are left to ion_exchanges (the
 // virtual site -1 draws for site 0, so they change no draw).  Against one step at a
-// time, 1,000 steps at P0 = 3.8e-4: 64 rails of 100 sites 0.35 -> 0.18 ms, 16,000 of
+// time, 1,000 steps at P0 = 3.8e-4: 64 rails of 100 sites 0.35 -> 0.16 ms, 16,000 of
 // 200 3.2 -> 2.6 ms, 3,001 open ones of 777 3.0 -> 2.2 ms; 65,536 of 1,024 with
 // per-site barriers 60 -> 50 ms.  GRAD: the gradient pass, which
 // replays the sweep from its first occupancy with the score accumulated instead
@@ -1166,7 +1173,7 @@ __device__ __forceinline__ void ion_score_end(const IonView<P, CLS> &c, int64_t 
 // share a warp should hold equally many ions: a.order lists them by their first
 // occupancy's counts, the fullest first (65,536 rails of 512 sites, 102 +- 9 ions, 8
 // to a warp: 29 rows on average in the order of their indices, 26 in this one).
-template <int P, bool ACC, bool OPEN, class M, bool GRAD = false>
+template <int P, bool ACC, bool OPEN, class M, bool GRAD = false, int AHEAD = OPEN ? kIonAhead : 4>
 __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0, const uint32_t *rk1,
                                          int64_t t0, int n_steps, int flush, int64_t tile_rail0,
                                          uint8_t *smem)
@@ -1324,38 +1331,42 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                     // some draw is within a bound's band: all that may be accepted are looked at
                     und = least <= c.width() ? aR | aL : 0;
                 } else {
-                    StepDraw sd[kIonAhead];
-#pragma unroll
-                    for (int q = 0; q < kIonAhead; ++q) sd[q] = step_draw(t + q, prail, rk0, rk1);
-                    for (int half = 0; half < (int)sizeof(M) / 4; ++half) {
-                        const uint32_t *const to = end - cp > 32 * 32 ? cp + 32 * 32 : end;
-                        uint32_t h[kIonAhead] = {}, bit = 1u;
 #pragma unroll 1
-                        while (cp != to) {
-                            const uint32_t e = *cp;
-                            cp += 32;
-                            const uint4 w = site_at(tab, e);
-                            const uint2 th = *(const uint2 *)(rm + (e >> 16));
+                    for (int q0 = 0; q0 < (AHEAD > 4 ? min(AHEAD, min(c1, wend) - s) : 1); q0 += 4) {
+                        StepDraw sd[4];
 #pragma unroll
-                            for (int q = 0; q < kIonAhead; ++q) {
-                                uint32_t xy, xw;
-                                site_draw(sd[q], w.x, w.y, w.z, rk0, rk1, xy, xw);
-                                if (xy <= th.x || xw <= th.y) h[q] |= bit;
+                        for (int q = 0; q < 4; ++q) sd[q] = step_draw(t + (uint32_t)(q0 + q), prail, rk0, rk1);
+                        cp = c.colp();
+                        for (int half = 0; half < (int)sizeof(M) / 4; ++half) {
+                            const uint32_t *const to = end - cp > 32 * 32 ? cp + 32 * 32 : end;
+                            uint32_t h[4] = {}, bit = 1u;
+#pragma unroll 1
+                            while (cp != to) {
+                                const uint32_t e = *cp;
+                                cp += 32;
+                                const uint4 w = site_at(tab, e);
+                                const uint2 th = *(const uint2 *)(rm + (e >> 16));
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    uint32_t xy, xw;
+                                    site_draw(sd[q], w.x, w.y, w.z, rk0, rk1, xy, xw);
+                                    if (xy <= th.x || xw <= th.y) h[q] |= bit;
+                                }
+                                bit <<= 1;
                             }
-                            bit <<= 1;
-                        }
 #pragma unroll
-                        for (int q = 0; q < kIonAhead; ++q) {
-                            c.hits(q + kIonAhead * half) = h[q];
-                            if (h[q]) look |= 1u << q;
+                            for (int q = 0; q < 4; ++q) {
+                                c.hits(q0 + q + AHEAD * half) = h[q];
+                                if (h[q]) look |= 1u << (q0 + q);
+                            }
                         }
                     }
                     look = __reduce_or_sync(FULL, look);
                     if constexpr (OPEN) ends_at = ion_end_draws<P>(c, tab, t, prail, rk0, rk1);
                 }
             }
-            // ---- the steps drawn for, up to one that changes what the next draw
-            int ahead = ACC ? 1 : min(kIonAhead, min(c1, wend) - s);
+            // ---- the steps drawn for, up to one whose draws are to be made again
+            int ahead = ACC ? 1 : min(AHEAD, min(c1, wend) - s);
 #pragma unroll 1
             for (int q = 0; q < ahead; ++q) {
             if constexpr (!ACC) {
@@ -1367,7 +1378,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                 if (stop >= ahead) break;
                 q = stop;
                 und |= c.hits(q);
-                if (sizeof(M) > 4) und |= (M)c.hits(q + kIonAhead) << (8 * sizeof(M) - 32);
+                if (sizeof(M) > 4) und |= (M)c.hits(q + AHEAD) << (8 * sizeof(M) - 32);
                 aR = aL = two = 0;
             }
             const int sq = s + q;
@@ -1463,7 +1474,7 @@ __device__ __forceinline__ void ion_tile(const SweepArgs &a, const uint32_t *rk0
                             uint32_t xy, xw;
                             site_draw(step_draw(t + (uint32_t)k, prail, rk0, rk1), w.x, w.y, w.z, rk0, rk1, xy, xw);
                             if (xy <= th.x || xw <= th.y) {
-                                c.hits(k + kIonAhead * (j >> 5)) |= 1u << (j & 31);
+                                c.hits(k + AHEAD * (j >> 5)) |= 1u << (j & 31);
                                 more |= 1u << k;
                             }
                         }
