@@ -377,7 +377,7 @@ def run_kmc(args):
             "e2e": {"value": e2e_value, "unit": UNIT, "steps": args.steps,
                     "h2d_bytes_per_step": int(Vpin.nbytes),
                     "d2h_bytes_per_step": int(Jpin.nbytes + Zpin.nbytes)},
-            # per timed step: one sweep_kernel launch and one zone_scan_kernel launch
+            # per timed step: one launch of the sweep and one of zone_scan_kernel
             "gpu_launches": 2 * args.steps,
             "counters": {"philox_blocks_per_site_update": draws / su_per_step,
                          "fp64_decisions": int(cnt1[1] - cnt0[1]),

@@ -74,20 +74,21 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
 // The tile and its lanes per rail.
 //
 // Ion lists against occupancy words (one GB300, site-updates/s, words first):
-// with the accept path 6.6e11 -> 1.15e12 at 65,536 x 512 rails 20 % full, 3.9e11
-// -> 5.3e11 at 8,192 x 1,000 half full, 3.9e11 -> 4.7e11 at 60 %, 4.0e11 ->
-// 4.2e11 at 70 %; without it 1.10e12 -> 1.22e12 at 30 %, 9.3e11 -> 9.7e11 at
-// 40 %, 8.5e11 -> 8.1e11 half full (blocked ions draw in vain, and there is
-// little rebuilding to save).  Rails of a few sites have next to no ions, and
-// the words put 32 of them on a warp (4 sites: 2.7e11 -> 1.2e11; 8: 1.1e11 ->
-// 1.6e11).
+// with the accept path 6.6e11 -> 1.29e12 at 65,536 x 512 rails 20 % full, 3.9e11
+// -> 5.7e11 at 8,192 x 1,000 half full, 4.0e11 -> 4.2e11 at 70 %; without it
+// 8.5e11 -> 8.6e11 at 8,192 x 1,000 and 7.6e11 -> 8.4e11 at 16,384 x 512 half
+// full, 8.4e11 -> 7.3e11 at 60 % (blocked ions draw in vain, and there is little
+// rebuilding to save).  Rails of a few sites have next to no ions, and the words
+// put 32 of them on a warp (4 sites: 2.7e11 -> 1.2e11; 8: 1.1e11 -> 1.6e11).
 //
 // Few lanes per rail spread a step's fixed work (bounds, refresh, votes) over
 // more ions of a lane and waste less of the last row; they also make fewer
 // warps.  6,000 warps fill the GPU (152 SMs x 32) with something to spare for
-// the last wave; below about six ions to a lane the fixed work costs more than
-// half-empty SMs (32,768 x 128, 26 ions: 3.0e11 on 32 lanes, 4.1e11 on 16,
-// 5.6e11 on 8, 6.0e11 on 4).
+// the last wave; with the accept path 3,600 in one wave of even CTAs do (8,192 x
+// 1,000 on 16 lanes: 300 steps 3.16 -> 2.91 ms; without it 1.23 -> 1.25 ms for
+// 200).  Below about six ions to a lane the fixed work costs more than half-empty
+// SMs (32,768 x 128, 26 ions: 3.0e11 on 32 lanes, 4.1e11 on 16, 5.6e11 on 8,
+// 6.0e11 on 4).
 float tile_max_fill(bool acc) { return acc ? 0.7f : 0.5f; }
 
 TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max, bool acc)
