@@ -109,7 +109,7 @@ constexpr int kStep = 16;          // an entry's difference between neighbouring
 __device__ __forceinline__ int pos_of(uint32_t e) { return (int)((e & 0xFFFFu) / kStep) - 1; }
 __device__ __forceinline__ uint4 site_at(const uint8_t *tab, uint32_t e) { return *(const uint4 *)(tab + (e & 0xFFFFu)); }
 // A warp's block: header of 64 bytes (band factor and mid voltage of the voltage
-// window float [2], the largest column, the step up to which draws are counted;
+// window float [2], the bounds' widest band in its last word, the largest column, the step up to which draws are counted;
 // in the gradient pass the doubles of IonScore from byte 24 on),
 // int [G] each of F, N0, the sum of positions that the per-rail current counts
 // from, and the rail, then the bounds.
