@@ -133,14 +133,12 @@ int build_items(kmc_batch *b, int warps)
         const kmc_params &p = h->p;
         const TileShape t = pick_tile(rails, p.n_rails, p.n_sites, p.electrodes == 1, h->n_tot, h->n_max, acc != 0);
         host[i] = h->args;
-        const size_t need = tile_args(host[i], t, p, h->P0site != nullptr, warps, acc != 0);
-        plan.smem[t.kind] = std::max(plan.smem[t.kind], need);
         devs.push_back(&p);
         shapes.push_back(t);
         inst.push_back((int)i);
     }
-    // the occupancy words of every device have to fit as well: the limit of a CTA
-    // size does not depend on the filling
+    // the limit of a CTA size is that of the occupancy words of every device, whatever
+    // its filling
     for (size_t i = 0; i < b->dev.size(); ++i) {
         const kmc_params &p = *devs[i];
         int wpl = 1;
@@ -148,12 +146,25 @@ int build_items(kmc_batch *b, int warps)
         if (sweep_smem_bytes(lpr, wpl, p.n_zones, p.n_sites, warps, b->flush, acc != 0) + 1024 > (size_t)max_smem)
             return fail(KMC_E_ARG, "batch: shared memory for this CTA size exceeds the device limit");
     }
-    for (int k = 0; k < kShapeKinds; ++k)
-        if (plan.smem[k] + 1024 > (size_t)max_smem)
+    // ion lists can need more (four lanes to a rail, 32 zones, per-site barriers: 25 KB a
+    // warp): a shape whose devices do not fit runs in smaller CTAs.  One warp always
+    // fits (33 KB of site table and the warp's block).
+    for (int k = 0; k < kShapeKinds; ++k) plan.warps[k] = warps;
+    for (size_t i = 0; i < devs.size(); ++i) {
+        const TileShape &t = shapes[i];
+        int &w = plan.warps[t.kind];
+        auto need = [&] { return tile_args(host[i], t, *devs[i], b->dev[i]->P0site != nullptr, w, acc != 0); };
+        while (w > 1 && need() + 1024 > (size_t)max_smem) w >>= 1;
+        if (need() + 1024 > (size_t)max_smem)
             return fail(KMC_E_ARG, "batch: shared memory for this CTA size exceeds the device limit");
+    }
+    for (size_t i = 0; i < devs.size(); ++i) {
+        const int k = shapes[i].kind;
+        plan.smem[k] = std::max(plan.smem[k], tile_args(host[i], shapes[i], *devs[i], b->dev[i]->P0site != nullptr,
+                                                        plan.warps[k], acc != 0));
+    }
     std::vector<BatchItem> sorted;
     int cls_off[kShapeKinds + 1];
-    for (int k = 0; k < kShapeKinds; ++k) plan.warps[k] = warps;
     make_items(devs, shapes, inst, plan.warps, sorted, cls_off);
     BCK(cudaMemcpyAsync(b->inst, host.data(), sizeof(SweepArgs) * host.size(), cudaMemcpyHostToDevice, b->user),
         "copy device arguments");
@@ -174,7 +185,7 @@ int build_items(kmc_batch *b, int warps)
     for (int k = 0; k < kShapeKinds; ++k) {
         const int n = cls_off[k + 1] - cls_off[k];
         b->cls_off[k] = cls_off[k];
-        plan.grid[k] = n > 0 ? std::min(n, sms * batch_ctas_per_sm(k, acc, warps, plan.smem[k])) : 0;
+        plan.grid[k] = n > 0 ? std::min(n, sms * batch_ctas_per_sm(k, acc, plan.warps[k], plan.smem[k])) : 0;
     }
     b->cls_off[kShapeKinds] = cls_off[kShapeKinds];
     b->plan = plan;
@@ -215,8 +226,7 @@ int run_chunk(kmc_batch *b, int n_steps)
             drop_graph(b);
             cudaGraph_t g = nullptr;
             BCK(cudaStreamBeginCapture(b->work, cudaStreamCaptureModeThreadLocal), "begin capture");
-            cudaError_t le = batch_launch(batch_args(b, n_steps), b->plan, b->warps, b->acc != 0,
-                                          b->work);
+            cudaError_t le = batch_launch(batch_args(b, n_steps), b->plan, b->acc != 0, b->work);
             cudaError_t ce = cudaStreamEndCapture(b->work, &g);
             if (le != cudaSuccess) {
                 if (g) cudaGraphDestroy(g);
@@ -233,7 +243,7 @@ int run_chunk(kmc_batch *b, int n_steps)
         BCK(cudaGraphLaunch(b->graph, b->work), "cudaGraphLaunch");
         return KMC_OK;
     }
-    BCK(batch_launch(batch_args(b, n_steps), b->plan, b->warps, b->acc != 0, b->work),
+    BCK(batch_launch(batch_args(b, n_steps), b->plan, b->acc != 0, b->work),
         "batched launch");
     return KMC_OK;
 }

@@ -252,8 +252,7 @@ int sweep_kind(int lpr, int wpl);
 cudaError_t batch_set_smem_limit();
 // launches the batched sweep (one launch per shape), the zone-count scans, and
 // then advances *t0 by n_steps and re-arms the work counters
-cudaError_t batch_launch(const BatchArgs &b, const BatchPlan &plan, int warps, bool acc,
-                         cudaStream_t s);
+cudaError_t batch_launch(const BatchArgs &b, const BatchPlan &plan, bool acc, cudaStream_t s);
 
 // Sets the message returned by kmc_last_error() on this thread (kmc_capi.cu).
 void kmc_internal_set_error(const char *msg);

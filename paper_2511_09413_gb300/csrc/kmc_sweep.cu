@@ -1719,18 +1719,17 @@ cudaError_t batch_set_smem_limit()
     return cudaSuccess;
 }
 
-cudaError_t batch_launch(const BatchArgs &b, const BatchPlan &plan, int warps, bool acc,
-                         cudaStream_t s)
+cudaError_t batch_launch(const BatchArgs &b, const BatchPlan &plan, bool acc, cudaStream_t s)
 {
     cudaError_t e;
     for (int k = 0; k < kShapeKinds; ++k) {
         if (plan.grid[k] <= 0) continue;
-        if (k >= kWordKinds) e = ion_batch_launch(b, k, plan.grid[k], warps, plan.smem[k], acc, s);
+        if (k >= kWordKinds) e = ion_batch_launch(b, k, plan.grid[k], plan.warps[k], plan.smem[k], acc, s);
         else
             e = with_shape(k, [&](auto lpr, auto wpl) {
             constexpr int P = decltype(lpr)::value, Q = decltype(wpl)::value;
-            if (acc) sweep_batch_kernel<true, P, Q><<<plan.grid[k], warps * 32, plan.smem[k], s>>>(b);
-            else sweep_batch_kernel<false, P, Q><<<plan.grid[k], warps * 32, plan.smem[k], s>>>(b);
+            if (acc) sweep_batch_kernel<true, P, Q><<<plan.grid[k], plan.warps[k] * 32, plan.smem[k], s>>>(b);
+            else sweep_batch_kernel<false, P, Q><<<plan.grid[k], plan.warps[k] * 32, plan.smem[k], s>>>(b);
             return cudaGetLastError();
         });
         if (e != cudaSuccess) return e;

@@ -144,3 +144,27 @@ def test_batch_with_per_site_barriers_bit_exact(kmc, mode):
     with pytest.raises(kmc.KmcError):
         b.grad(0, np.ones(n_steps), None)
     b.close()
+
+
+# 32 zones, per-site barriers and four lanes to a rail: CTAs of 8 warps do not fit in
+# shared memory, those of the occupancy words do; the batch takes smaller ones
+@pytest.mark.parametrize("n,R,L,electrodes,fill", [(16, 3073, 480, 0, 0.175), (1, 20001, 128, 1, 0.2)])
+@pytest.mark.parametrize("dt", [2e-8, 5e-7])
+def test_batch_of_lists_beyond_the_shared_memory_of_eight_warps(kmc, n, R, L, electrodes, fill, dt):
+    devs = [dict(R=R, L=L, Z=32, electrodes=electrodes, d=1.0, dt=dt, T=300.0, Ea=0.40, nu=1e12, alpha=0.2,
+                 kappa=1.0, k_e=0.5 / dt if electrodes else 0.0, rho_e=0.3 if electrodes else 0.0, seed=5,
+                 instance=i) for i in range(n)]
+    V = np.where(np.arange(24) % 6 < 3, 1.0, -0.5)
+    Ea = W.normal_barriers(R, L, 0.40, 0.01, seed=6)
+    b = kmc.Batch(devs, [V] * n, [1] * n, fills=[fill] * n, Ea_sites=[Ea] * n)
+    b.step_n(10)
+    b.set_accept_path(0)
+    b.step_n(14)
+    for i in {0, n - 1}:
+        s = kmc.Sim(devs[i], V, 1, fill=fill, Ea_site=Ea)
+        s.step_n(24)
+        for x, y in zip((*b.traces(i), b.occupancy(i), b.rail_current(i)),
+                        (*s.traces(), s.occupancy(), s.rail_current())):
+            assert np.array_equal(x, y)
+        s.close()
+    b.close()
