@@ -26,8 +26,6 @@ thread_local std::string g_err;
 
 Allocator g_alloc;
 std::mutex g_alloc_mu;
-std::once_flag g_attr_once;
-cudaError_t g_attr_err = cudaSuccess;
 
 int fail(int code, const char *fmt, ...) __attribute__((format(printf, 2, 3)));
 int fail(int code, const char *fmt, ...)
@@ -50,6 +48,23 @@ int cuda_fail(cudaError_t e, const char *what)
 }  // namespace
 
 void kmc::kmc_internal_set_error(const char *msg) { g_err = msg ? msg : ""; }
+
+// A function's attributes belong to a device, so they are set once on each.
+cudaError_t kmc::raise_smem_limits()
+{
+    constexpr int kKnown = 64;
+    static std::mutex mu;
+    static bool done[kKnown] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev >= 0 && dev < kKnown && done[dev]) return cudaSuccess;
+    e = sweep_set_smem_limits();
+    if (e == cudaSuccess) e = ion_set_smem_limits();
+    if (e == cudaSuccess && dev >= 0 && dev < kKnown) done[dev] = true;
+    return e;
+}
 
 
 namespace {
@@ -278,11 +293,7 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         std::lock_guard<std::mutex> lk(g_alloc_mu);
         h->al = g_alloc;
     }
-    std::call_once(g_attr_once, [] { 
-        g_attr_err = sweep_set_smem_limits();
-        if (g_attr_err == cudaSuccess) g_attr_err = ion_set_smem_limits();
-    });
-    if (g_attr_err != cudaSuccess) return cuda_fail(g_attr_err, "cudaFuncSetAttribute");
+    CK(raise_smem_limits(), "cudaFuncSetAttribute");
 
     const kmc_params &p = h->p;
     const int64_t R = p.n_rails, L = p.n_sites, Z = p.n_zones;

@@ -254,6 +254,10 @@ cudaError_t batch_set_smem_limit();
 // then advances *t0 by n_steps and re-arms the work counters
 cudaError_t batch_launch(const BatchArgs &b, const BatchPlan &plan, bool acc, cudaStream_t s);
 
+// Raises the kernels' dynamic shared-memory limits on the current device, at the
+// first call on it (kmc_capi.cu).
+cudaError_t raise_smem_limits();
+
 // Sets the message returned by kmc_last_error() on this thread (kmc_capi.cu).
 void kmc_internal_set_error(const char *msg);
 

@@ -69,8 +69,7 @@ int scratch_for_current_device(unsigned char **out)
         void *ptr = nullptr;
         e = cudaGetSymbolAddress(&ptr, g_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(scratch)");
-        e = sweep_set_smem_limits();
-        if (e == cudaSuccess) e = ion_set_smem_limits();
+        e = raise_smem_limits();
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         g_scratch_addr[dev] = ptr;
     }
