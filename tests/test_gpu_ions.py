@@ -96,6 +96,21 @@ def test_rare_moves(kmc, L, Z, electrodes, kappa, spread, rule):
     _check(kmc, dev, V, 0.3, [1, 2, 3, 261, 336], Ea)
 
 
+# a voltage that moves within a window, by 0.01 to 1 of the exponent in a step, with
+# jumps beside it: wide bounds without the accept path, windows that end inside the
+# steps drawn ahead
+@pytest.mark.parametrize("L,Z", [(8, 8), (33, 1), (100, 10), (777, 32)])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 1e-8])
+@pytest.mark.parametrize("spread", [None, 0.03])
+def test_fast_voltage(kmc, L, Z, electrodes, dt, spread):
+    dev = _dev(R=45, L=L, Z=Z, electrodes=electrodes, k_e=0.2 / dt if electrodes else 0.0, rho_e=0.4, dt=dt)
+    Ea = None if spread is None else np.maximum(np.random.default_rng(L).normal(0.40, spread, (45, L)), 0.36)
+    n = np.arange(400)
+    V = np.where(n % 97 < 50, 1.0, -1.0) * 0.02 * L * np.abs(np.sin(n / (3.0 + 20.0 * (n > 200))))
+    _check(kmc, dev, V, 0.3, [7, 150, 243], Ea)
+
+
 # rails that share a warp are taken in the order of their ion counts: empty, full
 # and uneven ones, with places beyond the last rail, and a count per rail that must
 # come back at the rail's own index
