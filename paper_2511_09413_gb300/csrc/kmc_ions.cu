@@ -121,11 +121,16 @@ TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_
 // its exponent by |kappa alpha| / (2 L kT).  Exchanges with an electrode alternate
 // in and out as long as the list keeps its entries, so they shift a rail by one at
 // each end and are not counted; where that leaves no room they are.  Room for ten
-// crossings, at most 0.25 (a fifth more draws to look at), at least 0.05.
+// crossings, at most 0.25 (a fifth more draws to look at), at least 0.05.  Where an
+// open rail is so short that not counting its exchanges takes more, up to 0.7: every
+// exchange would use up room that a crossing needs (65,536 x 48 rails 40 % full, an
+// exchange in most steps, 64 steps: 1.59 ms counting them, 0.79 not; 0.93 on the
+// occupancy words).  e^s < 1 + s + s^2 and e^-s > 1 - s there.
 static void ion_slack(SweepArgs &a, bool open)
 {
     const double per = 0.505 * fabs((double)a.ka_f) * (double)a.inv_LkT;
-    const double slack = std::min(0.25, std::max(0.05, 10.0 * per));
+    double slack = std::min(0.25, std::max(0.05, 10.0 * per));
+    if (open && 0.99 * slack < 4.0 * per && 4.1 * per <= 0.7) slack = 4.1 * per;
     a.ion_slack = (float)slack;
     const int fits = per * 1000.0 < 0.99 * slack ? 1000 : (int)floor(0.99 * slack / per);
     a.ion_exchange = open && fits < 4 ? 1 : 0;
