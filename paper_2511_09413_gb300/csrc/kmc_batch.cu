@@ -131,7 +131,8 @@ int build_items(kmc_batch *b, int warps)
     for (size_t i = 0; i < b->dev.size(); ++i) {
         const kmc_handle *h = b->dev[i];
         const kmc_params &p = h->p;
-        const TileShape t = pick_tile(rails, p.n_rails, p.n_sites, p.electrodes == 1, h->n_tot, h->n_max, acc != 0);
+        const TileShape t = pick_tile(rails, p.n_rails, p.n_sites, p.n_zones, p.electrodes == 1, h->n_tot, h->n_max,
+                                      acc != 0, h->args.P0f_scalar);
         host[i] = h->args;
         devs.push_back(&p);
         shapes.push_back(t);
@@ -537,8 +538,7 @@ int kmc_batch_grad_all(kmc_batch *b, const double *const *dLoss_dJ, const double
             if (!active[(size_t)i]) continue;
             const kmc_handle *h = b->dev[(size_t)i];
             devs.push_back(&h->p);
-            shapes.push_back(pick_grad_tile(rails, h->p.n_rails, h->p.n_sites, h->p.electrodes == 1, h->n_tot,
-                                            h->n_max));
+            shapes.push_back(pick_grad_tile(rails, h->p.n_rails, h->p, h->n_tot, h->n_max));
             inst.push_back(i);
         }
         BatchPlan plan{};

@@ -150,8 +150,8 @@ int pick_launch(kmc_handle *h)
     const kmc_params &p = h->p;
     SweepLaunch l{};
     l.acc = h->accept_req >= 0 ? h->accept_req : (h->args.P0f_scalar >= kAcceptAutoP0 ? 1 : 0);
-    const TileShape t = pick_tile(p.n_rails, p.n_rails, p.n_sites, p.electrodes == 1, h->n_tot, h->n_max,
-                                  l.acc != 0);
+    const TileShape t = pick_tile(p.n_rails, p.n_rails, p.n_sites, p.n_zones, p.electrodes == 1, h->n_tot, h->n_max,
+                                  l.acc != 0, h->args.P0f_scalar);
     l.ions = t.ions;
     l.kind = t.kind;
     l.lpr = t.lpr;
@@ -793,7 +793,7 @@ int kmc_grad(kmc_handle *h, const double *dLoss_dJ, const double *dLoss_dZc, dou
         SweepArgs ga;
         int rc = grad_prepare(h, dLoss_dJ, dLoss_dZc, &ga);
         if (rc) return rc;
-        const TileShape ts = pick_grad_tile(R, R, (int)L, p.electrodes == 1, h->n_tot, h->n_max);
+        const TileShape ts = pick_grad_tile(R, R, p, h->n_tot, h->n_max);
         SweepLaunch l{};
         l.kind = ts.kind;
         l.lpr = ts.lpr;

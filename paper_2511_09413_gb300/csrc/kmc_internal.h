@@ -207,9 +207,9 @@ cudaError_t ion_set_smem_limits();
 // gate (may be null): a device flag; with a nonzero one the launch does nothing
 cudaError_t ion_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate, cudaStream_t s);
 // The tile for a device: rails (of all devices that share its launches), sites,
-// electrodes, ions in all of the device's n_rails and at most n_max on a rail,
-// accept path.
-TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max, bool acc);
+// zones, electrodes, ions in all of the device's n_rails and at most n_max on a rail,
+// accept path, hop probability.
+TileShape pick_tile(int64_t rails, int64_t n_rails, int L, int Z, bool open, int64_t n_tot, int64_t n_max, bool acc, double P0);
 // filling of the sites up to which the ion lists are the better tile
 float tile_max_fill(bool acc);
 // sets a.rcap and a.iy for the tile; shared memory of a CTA of `warps` warps
@@ -220,7 +220,7 @@ cudaError_t ion_batch_launch(const BatchArgs &b, int kind, int grid, int warps, 
                              cudaStream_t s);
 int ion_batch_ctas_per_sm(int kind, int mode, int warps, size_t smem);
 // the same for the gradient pass
-TileShape pick_grad_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max);
+TileShape pick_grad_tile(int64_t rails, int64_t n_rails, const kmc_params &p, int64_t n_tot, int64_t n_max);
 // shared memory of a CTA at most, and of an SM, for the gradient pass
 void grad_smem_limits(size_t *most, size_t *total, bool ions);
 constexpr int kGradSmem = 226 * 1024;   // dynamic shared memory of a gradient CTA at most

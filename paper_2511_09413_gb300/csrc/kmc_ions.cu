@@ -91,11 +91,43 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
 // 6.0e11 on 4).
 float tile_max_fill(bool acc) { return acc ? 0.7f : 0.5f; }
 
-TileShape pick_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max, bool acc)
+// Many rails of few sites and few zones.  The words put a rail of up to 32 sites on one
+// lane and of up to 64 on two, where the lists take four and repeat a warp's fixed work
+// two to eight times as often; zones bring the two together, as a warp evaluates those
+// of all its rails.  65,536 rails, 64 steps, times of the lists over those of the words:
+// with the accept path 1.7 to 0.9 at 8 sites (1 to 8 zones), open 1.6, 1.5, 1.3, 0.99 and
+// 0.54 at 16 sites (1, 2, 4, 7 and 10 zones), closed 1.3, 1.2 and 0.98 (1, 2, 4), open 1.1,
+// 1.1 and 0.97 at 48; without it open 2.0, 1.4, 1.05 and 0.65 at 16 (1, 4, 8, 10), 1.5 to 1.0 at
+// 24 and 32 (1), 1.05 to 0.85 at 48 and 64, and closed below 1 at all.  With fewer rails the words leave SMs idle:
+// from 24,000 on 1.1 to 1.5 at up to 16 sites and two zones, from 4,000 on 1.1 to 1.4 at 8
+// closed ones with the accept path.
+static bool words_for_few_sites(int64_t rails, int L, int Z, bool open, bool acc)
+{
+    int most = 0;       // zones
+    if (L > 64) return false;
+    if (rails >= 40000)
+        most = acc ? (open ? (L < 16 ? 6 : L <= 32 ? 4 : 2) : (L < 16 ? 7 : L <= 32 ? 2 : 0))
+                   : (open ? (L < 24 ? 8 : L <= 32 ? 2 : 0) : 0);
+    else if (acc && !open && L < 16 && rails >= 4000) most = 3;
+    else if (!acc && open && L < 24 && rails >= 20000) most = 2;
+    return Z <= most;
+}
+
+// Without the accept path although a hop is likely (a caller's choice): on the lists
+// every move costs the steps drawn ahead, so they win on few rails only (16,384 x 512
+// closed 1.05 times the words' time at P0 = 0.17, 0.85 at 0.07; open 1.6 and 1.2, 1.04 at
+// 0.02; 300 x 100 0.4).
+static bool words_for_likely_hops(int64_t rails, bool open, double P0)
+{
+    return rails >= 4000 && P0 > (open ? 1.0 / 64.0 : 1.0 / 8.0);
+}
+
+TileShape pick_tile(int64_t rails, int64_t n_rails, int L, int Z, bool open, int64_t n_tot, int64_t n_max, bool acc, double P0)
 {
     TileShape t{};
     const double mean = (double)n_tot / (double)n_rails;
-    if (L >= 8 && mean <= tile_max_fill(acc) * L) {
+    if (L >= 8 && mean <= tile_max_fill(acc) * L && !words_for_few_sites(rails, L, Z, open, acc) &&
+        (acc || !words_for_likely_hops(rails, open, P0))) {
         int P = 32;
         while (P > 4) {
             const int64_t warps = rails * (P / 2) / 32;
@@ -197,9 +229,33 @@ int ion_cta_warps(const SweepArgs &a, int kind, int64_t warps)
 // its sums are formed once for 8 rails (65,536 x 512 rails: 56 us a step on 4
 // lanes, 70 on 8, 91 on 16, 155 on 32).  More lanes only where fewer than 1,200
 // warps would be left (4,096 rails: 9.0 us on 4, 7.3 on 8, 6.7 on 16, 11 on 32).
-TileShape pick_grad_tile(int64_t rails, int64_t n_rails, int L, bool open, int64_t n_tot, int64_t n_max)
+//
+// The words take fewer lanes for a rail of few sites, so their warps repeat the fixed
+// work less often; the lists evaluate fewer zones (only where an ion crossed a
+// boundary).  Lists' time over the words', 64 steps at 20 % filling:
+//  * 4,000 rails (16 and 32 lanes on the lists): 1.05 to 1.4 where the words' lanes take
+//    a rail's zones at once, 0.4 to 0.97 where they don't (up to 256 sites);
+//  * 65,536: closed 1.9, 1.4, 1.05, 0.8 at 32 sites (1, 2, 4, 7 zones), 1.3, 1.3, 0.95 at 64 (1, 2, 4);
+//    open 2.3, 1.7, 1.3, 0.97 at 32 and 1.4, 1.4, 1.15 at 64; 24,000: a few per cent to a third less;
+//  * open rails of up to 16 zones, when their warps' shared memory makes more than one
+//    wave: 1.0 to 1.4 at up to 64 sites (10 zones), 0.95 to 1.3 at 128 (16), in one wave 0.75 to 0.9.
+static bool words_for_gradient(int64_t rails, int L, int Z, bool open, int waves)
+{
+    int wpl = 1;
+    const int lpr = sweep_pick_lpr(L, &wpl);
+    if (rails < 1200 || L > 256) return false;
+    if (rails < 9600) return Z <= lpr;
+    if (rails < 16000 || L > 128) return false;
+    if (open && waves > 1 && Z <= (L <= 64 ? 10 : 16)) return true;
+    if (L <= 32) return Z <= (rails >= 40000 ? 4 : 3);
+    return L <= 64 && Z <= (rails >= 40000 ? 2 : 1);
+}
+
+TileShape pick_grad_tile(int64_t rails, int64_t n_rails, const kmc_params &p, int64_t n_tot, int64_t n_max)
 {
     TileShape t{};
+    const int L = p.n_sites;
+    const bool open = p.electrodes == 1;
     if (L >= 8 && (double)n_tot <= tile_max_fill(true) * (double)n_rails * (double)L) {
         int P = 32;
         while (P > 4 && rails * (P / 2) / 32 >= 1200 && ion_rows(P / 2, L, open, n_max, 64) > 0) P >>= 1;
@@ -207,7 +263,18 @@ TileShape pick_grad_tile(int64_t rails, int64_t n_rails, int L, bool open, int64
         t.lpr = P;
         t.rcap = ion_rows(P, L, open, n_max, 64);
         t.kind = kWordKinds + 2 * (P == 4 ? 0 : P == 8 ? 1 : P == 16 ? 2 : 3) + (open ? 1 : 0);
-        return t;
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        sms = std::max(1, sms);
+        size_t most = 0, total = 0;
+        grad_smem_limits(&most, &total, true);
+        const int w = grad_warps(t, p, most, total, rails, sms);
+        SweepArgs a;
+        const int64_t resident = (int64_t)w * std::max<int>(1, std::min<int>((int)(total / (grad_tile_args(a, t, p, w) + 1024)), kGradWarps / w));
+        const int waves = (rails * P / 32 + sms * resident - 1) / (sms * resident) > 1 ? 2 : 1;
+        if (!words_for_gradient(rails, L, p.n_zones, open, waves)) return t;
+        t = TileShape{};
     }
     t.lpr = sweep_pick_lpr(L, &t.wpl);
     t.kind = sweep_kind(t.lpr, t.wpl);

@@ -261,7 +261,7 @@ extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t 
         return l;
     };
     // a quarter of the sites full, but room for any number of ions
-    const TileShape lists = pick_tile(R, R, L, p->electrodes == 1, (int64_t)R * L / 4, L, acc);
+    const TileShape lists = pick_tile(R, R, L, Z, p->electrodes == 1, (int64_t)R * L / 4, L, acc, P0);
     const SweepLaunch li = shape(lists);
     TileShape wt{};
     wt.lpr = sweep_pick_lpr(L, &wt.wpl);

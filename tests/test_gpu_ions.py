@@ -60,6 +60,17 @@ def test_shapes_of_the_lists(kmc, R, L, electrodes, dt):
     _check(kmc, dev, V, 0.25, [n // 3, n - n // 3])
 
 
+# either side of the lines between the occupancy words and the lists for few sites and
+# zones on many rails
+@pytest.mark.parametrize("R,L,Z", [(40001, 16, 2), (40001, 16, 3), (40001, 33, 2), (40001, 33, 3), (40001, 23, 8),
+                                   (40001, 23, 9), (4001, 12, 3), (20001, 17, 2)])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_few_sites_on_many_rails(kmc, R, L, Z, electrodes, dt):
+    dev = _dev(R=R, L=L, Z=Z, electrodes=electrodes, k_e=1.0 / dt if electrodes else 0.0, rho_e=0.3, dt=dt)
+    _check(kmc, dev, np.where(np.arange(24) % 6 < 3, 1.0, -0.5), 0.3, [9, 15])
+
+
 # more than 32 entries a lane: CTAs of up to 20 warps, in one wave and in several,
 # each with a last CTA that is not full
 @pytest.mark.parametrize("R,L,fill", [(2500, 2048, 0.5), (5001, 1100, 0.25)])

@@ -43,3 +43,10 @@ def test_gradient_on_lists(kmc, R, L, Z, fill, electrodes):
         assert np.all(np.abs(g - ref["grad"]) <= 1e-11 * scale + 1e-10 * np.abs(ref["grad"]))
         np.testing.assert_allclose(se, ref["stderr"], rtol=1e-8)
     sim.close()
+
+
+# either side of the lines between the occupancy words and the lists
+@pytest.mark.parametrize("R,L,Z", [(5001, 100, 4), (5001, 100, 5), (20001, 30, 3), (20001, 30, 4), (40001, 60, 10)])
+@pytest.mark.parametrize("electrodes", [0, 1])
+def test_gradient_of_few_sites_on_many_rails(kmc, R, L, Z, electrodes):
+    test_gradient_on_lists(kmc, R, L, Z, 0.2, electrodes)
