@@ -377,8 +377,9 @@ def run_kmc(args):
             "e2e": {"value": e2e_value, "unit": UNIT, "steps": args.steps,
                     "h2d_bytes_per_step": int(Vpin.nbytes),
                     "d2h_bytes_per_step": int(Jpin.nbytes + Zpin.nbytes)},
-            # per timed step: one launch of the sweep and one of zone_scan_kernel
-            "gpu_launches": 2 * args.steps,
+            # per timed step: the sweep and zone_scan_kernel; where a launch looks at the
+            # rails first, also that look and the other tile's launch, which returns at once
+            "gpu_launches": (4 if R >= 1200 and float(R) * L * chunk >= 2e9 else 2) * args.steps,
             "counters": {"philox_blocks_per_site_update": draws / su_per_step,
                          "fp64_decisions": int(cnt1[1] - cnt0[1]),
                          "moves": int(cnt1[2] - cnt0[2])},

@@ -148,31 +148,38 @@ int validate(const kmc_params *p, const double *V, int64_t n_total, const uint8_
 int pick_launch(kmc_handle *h)
 {
     const kmc_params &p = h->p;
-    SweepLaunch l{};
-    l.acc = h->accept_req >= 0 ? h->accept_req : (h->args.P0f_scalar >= kAcceptAutoP0 ? 1 : 0);
+    const int acc = h->accept_req >= 0 ? h->accept_req : (h->args.P0f_scalar >= kAcceptAutoP0 ? 1 : 0);
     const TileShape t = pick_tile(p.n_rails, p.n_rails, p.n_sites, p.n_zones, p.electrodes == 1, h->n_tot, h->n_max,
-                                  l.acc != 0, h->args.P0f_scalar);
-    l.ions = t.ions;
-    l.kind = t.kind;
-    l.lpr = t.lpr;
-    l.wpl = t.wpl;
+                                  acc != 0, h->args.P0f_scalar);
     int flush = h->flush_req > 0 ? h->flush_req : 256;
-    int warps = h->warps_req > 0 ? h->warps_req : 8;
-    warps = std::min(warps, 8);
     int dev = 0, max_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (max_smem <= 0) max_smem = 48 * 1024;
     max_smem = std::min(max_smem, 200 * 1024);
-    auto smem_for = [&](int w) { return tile_args(h->args, t, p, h->P0site != nullptr, w, l.acc != 0); };
-    while (warps > 1 && smem_for(warps) > (size_t)max_smem) warps >>= 1;
-    if (t.ions && h->warps_req <= 0)
-        warps = ion_cta_warps(h->args, t.kind, (p.n_rails * (int64_t)t.lpr + 31) / 32);
-    l.warps = warps;
-    l.smem = smem_for(warps);
-    const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * warps;
-    l.grid = (int)((p.n_rails + rails_per_cta - 1) / rails_per_cta);
-    h->launch = l;
+    auto shape = [&](const TileShape &t) {
+        SweepLaunch l{};
+        l.ions = t.ions;
+        l.kind = t.kind;
+        l.lpr = t.lpr;
+        l.wpl = t.wpl;
+        l.acc = acc;
+        auto smem_for = [&](int w) { return tile_args(h->args, t, p, h->P0site != nullptr, w, acc != 0); };
+        l.warps = std::min(h->warps_req > 0 ? h->warps_req : 8, 8);
+        while (l.warps > 1 && smem_for(l.warps) > (size_t)max_smem) l.warps >>= 1;
+        if (t.ions && h->warps_req <= 0)
+            l.warps = ion_cta_warps(h->args, t.kind, (p.n_rails * (int64_t)t.lpr + 31) / 32);
+        l.smem = smem_for(l.warps);
+        const int64_t rails_per_cta = (int64_t)(32 / l.lpr) * l.warps;
+        l.grid = (int)((p.n_rails + rails_per_cta - 1) / rails_per_cta);
+        return l;
+    };
+    h->launch = shape(t);
+    TileShape w{};
+    w.lpr = sweep_pick_lpr(p.n_sites, &w.wpl);
+    w.kind = sweep_kind(w.lpr, w.wpl);
+    h->words = shape(w);
+    h->words_steps = words_up_to(t, p.n_rails, p.n_sites, p.n_zones, acc != 0);
     h->args.flush = flush;
     return KMC_OK;
 }
@@ -640,8 +647,22 @@ int kmc_step_n(kmc_handle *h, int64_t n_steps)
         const int64_t n = std::min<int64_t>(n_steps, 1 << 30);
         h->args.t0 = h->t;
         h->args.n_steps = (int32_t)n;
-        cudaError_t e = h->launch.ions ? ion_launch(h->args, h->launch, nullptr, h->stream)
-                                       : sweep_launch(h->args, h->launch, nullptr, h->stream);
+        const bool lists = h->launch.ions && n > h->words_steps;
+        // rails fill up, empty and pile up as they run: a launch of about two milliseconds
+        // and more on a device that fills the GPU looks at them first, which takes 13 us with
+        // the empty launch of the other tile (16,384 x 512).  16,384 x 512
+        // rails 40 % full whose ions a field holds at one end: 2.24 ms for 298 steps on the lists,
+        // 0.45 on the words
+        int *gate = nullptr;
+        cudaError_t e = cudaSuccess;
+        if (lists && n >= 64 && (int64_t)h->p.n_rails * h->launch.lpr >= kGateLanes &&
+            (double)h->p.n_rails * h->p.n_sites * (double)n >= 2e9) {
+            gate = (int *)(h->misc + 15);
+            e = tile_gate(h->args, nullptr, h->launch.acc != 0, gate, h->stream);
+        }
+        if (e == cudaSuccess && lists) e = ion_launch(h->args, h->launch, gate, h->stream);
+        if (e == cudaSuccess && (!lists || gate))
+            e = sweep_launch(h->args, h->launch.ions ? h->words : h->launch, gate, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
         e = zone_scan(h->Zc, h->t, (int)n, h->p.n_zones, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "zone-count scan launch");

@@ -65,6 +65,8 @@ struct kmc_handle {
 
     kmc::SweepArgs args{};
     kmc::SweepLaunch launch{};
+    kmc::SweepLaunch words{};                 // of the occupancy words, where launch is of the lists
+    int64_t words_steps = 0;                  // steps of a launch up to which they are used
     int warps_req = 0;
     int flush_req = 0;
     int accept_req = -1;   // accept path: -1 automatic, 0 off, 1 on

@@ -212,6 +212,15 @@ cudaError_t ion_launch(const SweepArgs &a, const SweepLaunch &l, const int *gate
 TileShape pick_tile(int64_t rails, int64_t n_rails, int L, int Z, bool open, int64_t n_tot, int64_t n_max, bool acc, double P0);
 // filling of the sites up to which the ion lists are the better tile
 float tile_max_fill(bool acc);
+// lanes of a launch of the lists from which on the words can be the faster tile: fewer
+// leave SMs idle, and the lists' steps are shorter whatever the rails hold (300 x 100:
+// 0.14 to 0.28 times the words' time at any filling)
+constexpr int64_t kGateLanes = 32 * 1200;
+// *words (if not null) = 1 when the occupancy words are to advance the device as it
+// stands, else 0; dst (if not null) receives the arguments
+cudaError_t tile_gate(const SweepArgs &a, SweepArgs *dst, bool acc, int *words, cudaStream_t s);
+// steps of a launch up to which the words advance a device that the lists have
+int64_t words_up_to(const TileShape &t, int64_t rails, int L, int Z, bool acc);
 // sets a.rcap and a.iy for the tile; shared memory of a CTA of `warps` warps
 int ion_cta_warps(const SweepArgs &a, int kind, int64_t warps);
 size_t tile_args(SweepArgs &a, const TileShape &t, const kmc_params &p, bool persite, int warps, bool acc);

@@ -81,6 +81,8 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
 // rebuilding to save).  Rails of a few sites have next to no ions, and the words
 // put 32 of them on a warp (4 sites: 2.7e11 -> 1.2e11; 8: 1.1e11 -> 1.6e11).
 //
+// (The handle knows the filling of step 0 only; a long launch looks again, tile_gate.)
+//
 // Few lanes per rail spread a step's fixed work (bounds, refresh, votes) over
 // more ions of a lane and waste less of the last row; they also make fewer
 // warps.  6,000 warps fill the GPU (152 SMs x 32) with something to spare for
@@ -90,6 +92,74 @@ IonLayout ion_layout(int P, int Z, int L, bool open, bool persite, int rcap, boo
 // SMs (32,768 x 128, 26 ions: 3.0e11 on 32 lanes, 4.1e11 on 16, 5.6e11 on 8,
 // 6.0e11 on 4).
 float tile_max_fill(bool acc) { return acc ? 0.7f : 0.5f; }
+
+// The filling at which random rails run equally long on both tiles (16,384 x 512,
+// 65,536 x 100 and 4,000 x 1,000: without the accept path 0.93 to 0.95 times the words' time
+// on the lists at 55 %, 1.01 to 1.02 at 60 %; with it 0.81 to 0.91 at 70 %, 1.01 to 1.13 at
+// 80 %), and the share of blocked ions where they stand in runs: without the accept
+// path 0.86 to 1.03 at up to 0.3 and 1.13 to 1.26 at 0.5; with it 0.79 to 0.89 at 0.75 and up
+// to 1.7 at 0.94.  Rails held together by a field are at 0.9 and more: 2 to 7 times.
+struct TileLine {
+    float fill, blocked;
+};
+static TileLine tile_line(bool acc) { return acc ? TileLine{0.75f, 0.9f} : TileLine{0.58f, 0.35f}; }
+
+// The tile for a device as it stands, from 32 rails spread over it, a warp to each:
+// *words = 1 for the occupancy words, when more than line.fill of their sites are
+// occupied or more than line.blocked of their ions held on both sides, by an ion or a
+// blocking electrode, 0 for the lists.  Both tiles are launched after it and one of
+// them returns at once (2 us); the choice changes no result.  dst (may be null) receives
+// the arguments.
+static __global__ void __launch_bounds__(1024) tile_gate_kernel(const __grid_constant__ SweepArgs a, SweepArgs *dst,
+                                                                TileLine line, int *words)
+{
+    __shared__ int ions, held;
+    if (threadIdx.x == 0) {
+        if (dst) *dst = a;
+        ions = held = 0;
+    }
+    if (!words) return;
+    __syncthreads();
+    const uint8_t *row = a.occ + (int64_t)(threadIdx.x >> 5) * a.R / 32 * a.stride;
+    const int wall = a.electrodes == 1 ? 0 : 1;
+    int n = 0, b = 0;
+    for (int k = (int)(threadIdx.x & 31u); k < a.L; k += 32) {
+        const int left = k > 0 ? row[k - 1] : wall, right = k + 1 < a.L ? row[k + 1] : wall;
+        n += row[k];
+        b += row[k] & left & right;
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    b = __reduce_add_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31u) == 0u) {
+        atomicAdd(&ions, n);
+        atomicAdd(&held, b);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        *words = (float)ions > line.fill * 32.0f * (float)a.L || (float)held > line.blocked * (float)ions ? 1 : 0;
+}
+
+cudaError_t tile_gate(const SweepArgs &a, SweepArgs *dst, bool acc, int *words, cudaStream_t s)
+{
+    tile_gate_kernel<<<1, words ? 1024 : 32, 0, s>>>(a, dst, tile_line(acc), words);
+    return cudaGetLastError();
+}
+
+// Building the lists and writing them back takes as long as a few steps, and without
+// the accept path the least that is drawn is four steps.  Lists' time over the words',
+// 1, 2, 3, 4 and 8 steps without the accept path: 1.3, 1.05, 0.99, 0.92, 0.83 on 1,000 x 300, 1.5, 1.3,
+// 1.13, 1.03, 0.9 on 16,384 x 512 open, 2.8, 2.1, 1.8, 1.5, 1.3 (1.16 for 16, 0.96 for 32) on 65,536 x 1,024 open
+// with a warp to every rail; with it 1.4, 1.2, 1.05, 0.98 on 16,384 x 512, 1.5, 1.25, 1.14, 1.07 on
+// 65,536 x 1,024 open, 0.9 on 1,000 x 300.  With many zones to a lane of the words the lists
+// are faster from the first step on (65,536 x 100, 32 zones: 0.73).
+int64_t words_up_to(const TileShape &t, int64_t rails, int L, int Z, bool acc)
+{
+    int wpl = 1;
+    if (!t.ions || rails < 1000 || Z > 4 * sweep_pick_lpr(L, &wpl)) return 0;
+    const bool own = t.lpr == 32 && rails >= 32768;     // a warp to a rail, several waves
+    if (acc) return L >= 256 && rails >= 10000 ? (own ? 3 : 1) : 0;
+    return own ? 16 : 3;
+}
 
 // Many rails of few sites and few zones.  The words put a rail of up to 32 sites on one
 // lane and of up to 64 on two, where the lists take four and repeat a warp's fixed work

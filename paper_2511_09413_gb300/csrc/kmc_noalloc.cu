@@ -79,32 +79,6 @@ int scratch_for_current_device(unsigned char **out)
 
 bool finite_pos(double x) { return isfinite(x) && x > 0.0; }
 
-// Writes the launch arguments into the scratch array from the kernel's own
-// parameter space, so that no host buffer has to outlive the call (a copy
-// from host memory would read the caller's stack frame when it executes), and
-// chooses the tile: the filling is known only on the device, so both tiles are
-// launched and *words tells which of the two has the device (1: the occupancy
-// words, when more than max_fill of the sites of 32 rails spread over it are
-// occupied; an empty launch costs about 2 us).  One block of 1,024 threads, a
-// warp per sampled rail.  The choice changes no result.
-__global__ void __launch_bounds__(1024) store_args_kernel(const SweepArgs a, SweepArgs *dst, float max_fill,
-                                                          int *words)
-{
-    __shared__ int ions;
-    if (threadIdx.x == 0) {
-        *dst = a;
-        ions = 0;
-    }
-    __syncthreads();
-    const int64_t r = (int64_t)(threadIdx.x >> 5) * a.R / 32;
-    int n = 0;
-    for (int k = (int)(threadIdx.x & 31u); k < a.L; k += 32) n += a.occ[r * a.stride + k];
-    n = __reduce_add_sync(0xffffffffu, n);
-    if ((threadIdx.x & 31u) == 0u) atomicAdd(&ions, n);
-    __syncthreads();
-    if (threadIdx.x == 0) *words = (float)ions > max_fill * 32.0f * (float)a.L ? 1 : 0;
-}
-
 }  // namespace
 
 extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t row_stride,
@@ -262,21 +236,28 @@ extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t 
     };
     // a quarter of the sites full, but room for any number of ions
     const TileShape lists = pick_tile(R, R, L, Z, p->electrodes == 1, (int64_t)R * L / 4, L, acc, P0);
-    const SweepLaunch li = shape(lists);
+    SweepLaunch li = shape(lists);
     TileShape wt{};
     wt.lpr = sweep_pick_lpr(L, &wt.wpl);
     wt.kind = sweep_kind(wt.lpr, wt.wpl);
     const SweepLaunch lw = shape(wt);
-    int *gate = (int *)(misc + 7);
+    // the choice of a tile and the other's launch cost 6 us, which a call of a few steps
+    // does not win back (16,384 x 512 open without the accept path: 101 us with them for one
+    // step and 186 for ten, 76 and 167 on the words alone; with it 279 and 433 for ten); where
+    // the lists win whatever the rails hold there is no choice
+    const bool choose = R * (int64_t)lists.lpr >= kGateLanes;
+    if (n_steps <= words_up_to(lists, R, L, Z, acc) || (choose && n_steps < (acc ? 4 : 12) && Z <= 4 * wt.lpr)) li.ions = 0;
+    int *gate = li.ions && choose ? (int *)(misc + 7) : nullptr;
 
-    store_args_kernel<<<1, 1024, 0, s>>>(a, args_dev, tile_max_fill(acc), gate);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "argument store launch");
+    // the arguments reach the scratch array from the kernel's own parameter space: a
+    // copy from host memory would read this call's stack frame when it executes
+    if ((e = tile_gate(a, args_dev, acc, gate, s)) != cudaSuccess) return cuda_fail(e, "argument store launch");
     int64_t left = n_steps;
     while (left > 0) {
         const int64_t n = std::min<int64_t>(left, 1 << 30);
         a.n_steps = (int32_t)n;
         if (li.ions && (e = ion_launch(a, li, gate, s)) != cudaSuccess) return cuda_fail(e, "sweep launch");
-        if ((e = sweep_launch(a, lw, li.ions ? gate : nullptr, s)) != cudaSuccess)
+        if ((!li.ions || gate) && (e = sweep_launch(a, lw, gate, s)) != cudaSuccess)
             return cuda_fail(e, "sweep launch");
         if ((e = zone_scan(a.Zc, a.t0, (int)n, Z, s)) != cudaSuccess)
             return cuda_fail(e, "zone-count scan launch");

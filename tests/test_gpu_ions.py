@@ -146,6 +146,45 @@ def test_uneven_rails(kmc, R, electrodes, dt):
     sim.close()
 
 
+# launches of a few steps run on the occupancy words, longer ones on the lists
+@pytest.mark.parametrize("R,L,chunks", [(1200, 300, [1, 2, 3, 4, 17, 1]), (10001, 256, [1, 5, 1, 3]),
+                                        (32768, 1024, [1, 16, 3])])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_launches_of_few_steps(kmc, R, L, chunks, electrodes, dt):
+    dev = _dev(R=R, L=L, electrodes=electrodes, k_e=1.0 / dt if electrodes else 0.0, rho_e=0.3, dt=dt)
+    _check(kmc, dev, np.where(np.arange(sum(chunks)) % 6 < 3, 1.0, -0.5), 0.25, chunks)
+
+
+# long launches look at the rails first: ions in one block at an end, rails that are
+# full or empty, random ones, and rails whose filling changes between two launches
+@pytest.mark.parametrize("start", ["block", "uneven", "random", "filling"])
+@pytest.mark.parametrize("dt", [5e-7, 1e-8])
+def test_long_launches_choose_their_tile(kmc, start, dt):
+    R, L, n = 16385, 512, 240
+    open_ = start == "filling"
+    dev = _dev(R=R, L=L, kappa=0.0 if start == "block" else 1.0, electrodes=int(open_), k_e=1.0 / dt, rho_e=1.0, dt=dt)
+    occ0 = np.zeros((R, L), np.uint8)
+    rng = np.random.default_rng(3)
+    if start == "block":
+        occ0[:, :200] = 1
+    elif start == "uneven":
+        occ0[: R // 2] = 1
+    else:
+        occ0[:] = rng.random((R, L)) < (0.5 if open_ else 0.3)
+    V = np.full(2 * n, 10.0)
+    sim = kmc.Sim(dev, V, 2, occ0=occ0)
+    orc = oracle.OracleSim(dev, V, occ0, None)
+    for _ in range(2):
+        sim.step_n(n)
+    Jo, Zo = orc.step_n(2 * n)
+    Jg, Zg = sim.traces()
+    assert np.array_equal(Zg, Zo) and np.array_equal(Jg, Jo)
+    assert np.array_equal(sim.occupancy(), orc.occ)
+    assert np.array_equal(sim.rail_current(), orc.J_rail)
+    sim.close()
+
+
 # a batch chooses its tiles from all rails together: the same devices alone
 # and together give the same results, lists and words side by side
 def test_batch_of_lists_and_words(kmc):

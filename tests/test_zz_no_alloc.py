@@ -77,6 +77,44 @@ def test_no_alloc_sweep_matches_handle_path_on_two_calls(env, electrodes):
     assert not occ_dev[:, L:].any()
 
 
+# both tiles and the choice between them on the device (1,300 rails), the lists alone
+# (90 rails), rails too short for the lists, calls of few steps, and a device that
+# fills up from call to call
+@pytest.mark.parametrize("R", [90, 1300])
+@pytest.mark.parametrize("L", [4, 100, 777])
+@pytest.mark.parametrize("fill", [0.35, 0.65, 0.9])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_no_alloc_tiles_match_the_oracle(env, R, L, fill, electrodes, dt):
+    import oracle
+    torch, kmc = env
+    dev = dict(_device(electrodes), R=R, L=L, Z=min(L, 10), dt=dt, k_e=0.5 / dt if electrodes else 0.0,
+               rho_e=0.95 if electrodes else 0.0)
+    Z, calls = dev["Z"], [40, 3, 60, 1]
+    V = W.triangle_protocol(3.0, 40, 4)[: sum(calls)]
+    occ0 = W.random_occupancy(R, L, fill, seed=11)
+    orc = oracle.OracleSim(dev, V, occ0, None)
+    Jo, Zo = orc.step_n(sum(calls))
+    stride = (L + 15) // 16 * 16
+    occ_dev = torch.zeros((R, stride), dtype=torch.uint8, device="cuda")
+    occ_dev[:, :L] = torch.from_numpy(occ0).cuda()
+    V_dev = torch.from_numpy(np.ascontiguousarray(V)).cuda()
+    N0_dev = torch.from_numpy(occ0.sum(axis=1).astype(np.int32)).cuda()
+    J_dev = torch.full((sum(calls),), -7, dtype=torch.int64, device="cuda")
+    Zc_dev = torch.full((sum(calls), Z), -7, dtype=torch.int64, device="cuda")
+    p = kmc.params_from_device(dev, init_mode=2)
+    t = 0
+    for n in calls:
+        kmc.kmc_sweep_noalloc(p, occ_dev.data_ptr(), stride, N0_dev.data_ptr(), V_dev[t:].data_ptr(), t, n,
+                              J_dev[t:].data_ptr(), Zc_dev[t:].data_ptr(), torch.cuda.current_stream().cuda_stream)
+        t += n
+    torch.cuda.synchronize()
+    assert np.array_equal(J_dev.cpu().numpy(), Jo)
+    assert np.array_equal(Zc_dev.cpu().numpy(), Zo)
+    assert np.array_equal(occ_dev[:, :L].cpu().numpy(), orc.occ)
+    assert not occ_dev[:, L:].any()
+
+
 def test_no_alloc_rejects_sizes_beyond_its_scratch(env):
     torch, kmc = env
     dev = _device(0)
