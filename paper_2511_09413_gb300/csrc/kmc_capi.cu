@@ -308,8 +308,10 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
     const size_t occ_bytes = (size_t)(R * h->stride);
     h->occ = (uint8_t *)h->alloc(occ_bytes);
     h->V = (double *)h->alloc(sizeof(double) * (size_t)std::max<int64_t>(n_total, 1));
-    // the ion counts, and for the devices that fill the GPU the rails' order by them,
-    // formed with two words per count behind misc
+    // the ion counts and the rails' order by them, formed with two words per count behind
+    // misc.  Rails share a warp from 2,400 rails on (gradient pass) and 4,800 (sweep), in a
+    // batch of as many also those of smaller devices; below 1,024 rails there are too few
+    // warps for the two launches to pay
     const bool ordered = R >= 1024;
     h->N0 = (int32_t *)h->alloc(sizeof(int32_t) * (size_t)(ordered ? 2 * R : R));
     h->K = (DevConst *)h->alloc(sizeof(DevConst));
@@ -357,13 +359,13 @@ int create_impl(const kmc_params *params, const double *V, int64_t n_total, cons
         if (rc) return rc;
     }
     unsigned long long *bad = h->misc + 5;
-    int32_t *const bins = ordered ? (int32_t *)(h->misc + 16) : nullptr;
-    CK(setup_row_counts(h->occ, h->stride, (int32_t)R, (int32_t)L, h->N0, bad, h->misc + 8,
-                        bins, s),
+    unsigned long long *const stats = h->misc + 8;
+    CK(setup_row_counts(h->occ, h->stride, (int32_t)R, (int32_t)L, h->N0, bad, ordered ? nullptr : stats, s),
        "row counts");
     if (ordered) {
+        int32_t *const bins = (int32_t *)(h->misc + 16);
         h->order = h->N0 + R;
-        CK(setup_order(h->N0, (int32_t)R, (int32_t)L, bins, bins + L + 1, h->order, s), "rail order");
+        CK(setup_order(h->N0, (int32_t)R, (int32_t)L, bins, bins + L + 1, h->order, stats, s), "rail order");
     }
     CK(setup_background(h->N0, (int32_t)R, (int32_t)L, (int32_t)Z, h->K, h->bgd, s), "background");
     CK(cudaMemcpyAsync(h->occ_init, h->occ, occ_bytes, cudaMemcpyDeviceToDevice, s), "checkpoint");

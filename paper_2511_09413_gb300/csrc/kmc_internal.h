@@ -281,14 +281,14 @@ cudaError_t setup_p0_classes(const float *P0f, const float2 *bnd, int64_t R, int
 cudaError_t setup_p0_float(const double *P0, int64_t n, float *out, cudaStream_t s);
 // ions of each rail; with stats, also their total (stats[0]) and the largest (stats[1])
 cudaError_t setup_row_counts(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
-                             int32_t *N0, unsigned long long *bad, unsigned long long *stats,
-                             int32_t *bins, cudaStream_t s);
+                             int32_t *N0, unsigned long long *bad, unsigned long long *stats, cudaStream_t s);
 // bgd[r][z] = (N0[r] w_z / L in the oracle's FP64 order, D'_z): the background
 // of zone z of rail r and its part of Q_z - Qbar (S2.1.8 reading)
 cudaError_t setup_background(const int32_t *N0, int32_t R, int32_t L, int32_t Z, const DevConst *K,
                              double2 *bgd, cudaStream_t s);
-cudaError_t setup_order(const int32_t *N0, int32_t R, int32_t L, const int32_t *bins, int32_t *next, int32_t *order,
-                        cudaStream_t s);
+// the rails by falling ion count, and the stats of setup_row_counts; bins, next: L + 1 zeros each
+cudaError_t setup_order(const int32_t *N0, int32_t R, int32_t L, int32_t *bins, int32_t *next, int32_t *order,
+                        unsigned long long *stats, cudaStream_t s);
 cudaError_t setup_init_bernoulli(const kmc_params &p, uint8_t *occ, int64_t stride,
                                  cudaStream_t s);
 // mode 0: count init keys <= key_bound; mode 1: keys == key_bound with linear index <= idx_bound

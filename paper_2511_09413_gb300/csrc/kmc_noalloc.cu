@@ -147,7 +147,7 @@ extern "C" int kmc_sweep_noalloc(const kmc_params *p, uint8_t *occ_dev, int64_t 
     if ((e = setup_constants(*p, K, s)) != cudaSuccess) return cuda_fail(e, "constants launch");
     const int32_t *N0 = N0_dev_or_null;
     if (!N0) {
-        if ((e = setup_row_counts(occ_dev, row_stride, R, L, N0s, misc + 5, nullptr, nullptr, s)) != cudaSuccess)
+        if ((e = setup_row_counts(occ_dev, row_stride, R, L, N0s, misc + 5, nullptr, s)) != cudaSuccess)
             return cuda_fail(e, "row counts launch");
         N0 = N0s;
     }

@@ -143,7 +143,7 @@ __global__ void p0_classes_kernel(const float *P0f, const float2 *bnd, int64_t R
 
 // One warp per rail: ion count, and a count of bytes that are not 0 or 1.
 __global__ void row_counts_kernel(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
-                                  int32_t *N0, unsigned long long *bad, unsigned long long *stats, int32_t *bins)
+                                  int32_t *N0, unsigned long long *bad, unsigned long long *stats)
 {
     const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -158,7 +158,6 @@ __global__ void row_counts_kernel(const uint8_t *occ, int64_t stride, int32_t R,
     b = __reduce_add_sync(0xffffffffu, b);
     if (lane == 0) {
         N0[r] = c;
-        if (bins) atomicAdd(bins + c, 1);
         if (stats) {
             atomicAdd(stats, (unsigned long long)c);
             atomicMax(stats + 1, (unsigned long long)c);
@@ -167,15 +166,34 @@ __global__ void row_counts_kernel(const uint8_t *occ, int64_t stride, int32_t R,
     }
 }
 
-// The rails by falling ion count, from the number of rails of each count (bins, which
-// row_counts_kernel forms): every block sums up the bins before each count, and a
-// rail takes the next place of its own.  Rails of equal counts come in any order (no
-// result depends on it).
-__global__ void __launch_bounds__(1024) order_kernel(const int32_t *N0, int32_t R, int32_t L, const int32_t *bins,
-                                                     int32_t *next, int32_t *order)
+// bins[n]: rails of n ions.  Counted by block first: most rails share a few counts, and
+// an atomic operation to memory from every rail took 60 us on 65,536 rails.
+__global__ void __launch_bounds__(1024) bins_kernel(const int32_t *N0, int32_t R, int32_t L, int32_t *bins)
 {
-    __shared__ int32_t first[KMC_MAX_SITES + 1], sums[32];
+    __shared__ int32_t own[KMC_MAX_SITES + 1];
+    for (int i = threadIdx.x; i <= L; i += blockDim.x) own[i] = 0;
+    __syncthreads();
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < R) atomicAdd(&own[N0[r]], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i <= L; i += blockDim.x)
+        if (own[i] != 0) atomicAdd(bins + i, own[i]);
+}
+
+// The rails by falling ion count, from the number of rails of each count (bins): every
+// block sums up the bins before each count, and its rails take the next places of their
+// own (next, one atomic operation for each count).  Rails of equal counts come in any order
+// (no result depends on it).  stats: ions in all, and on the fullest rail.
+__global__ void __launch_bounds__(1024) order_kernel(const int32_t *N0, int32_t R, int32_t L, const int32_t *bins,
+                                                     int32_t *next, int32_t *order, unsigned long long *stats)
+{
+    __shared__ int32_t first[KMC_MAX_SITES + 1], own[KMC_MAX_SITES + 1], sums[32], most;
+    __shared__ unsigned long long ions;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        ions = 0;
+        most = 0;
+    }
     int32_t carry = 0;
     for (int32_t b0 = 0; b0 <= L; b0 += 1024) {
         const int32_t i = b0 + (int32_t)threadIdx.x, n = i <= L ? bins[L - i] : 0;
@@ -192,14 +210,29 @@ __global__ void __launch_bounds__(1024) order_kernel(const int32_t *N0, int32_t 
             if (lane >= off) s += u;
         }
         const int32_t before = w > 0 ? __shfl_sync(0xffffffffu, s, w - 1) : 0;
-        if (i <= L) first[L - i] = carry + before + v - n;
+        if (i <= L) {
+            first[L - i] = carry + before + v - n;
+            own[L - i] = 0;
+        }
+        if (blockIdx.x == 0 && n > 0) {
+            atomicAdd(&ions, (unsigned long long)n * (unsigned long long)(L - i));
+            atomicMax(&most, L - i);
+        }
         carry += __shfl_sync(0xffffffffu, s, 31);
         __syncthreads();
     }
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < R) {
-        const int32_t n = N0[r];
-        order[first[n] + atomicAdd(next + n, 1)] = (int32_t)r;
+    const int32_t n = r < R ? N0[r] : 0;
+    int32_t place = 0;
+    if (r < R) place = atomicAdd(&own[n], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i <= L; i += blockDim.x)
+        if (own[i] != 0) first[i] += atomicAdd(next + i, own[i]);
+    __syncthreads();
+    if (r < R) order[first[n] + place] = (int32_t)r;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        stats[0] = ions;
+        stats[1] = (unsigned long long)most;
     }
 }
 
@@ -365,19 +398,20 @@ cudaError_t setup_background(const int32_t *N0, int32_t R, int32_t L, int32_t Z,
 }
 
 cudaError_t setup_row_counts(const uint8_t *occ, int64_t stride, int32_t R, int32_t L,
-                             int32_t *N0, unsigned long long *bad, unsigned long long *stats,
-                             int32_t *bins, cudaStream_t s)
+                             int32_t *N0, unsigned long long *bad, unsigned long long *stats, cudaStream_t s)
 {
     const int warps = 8;
     row_counts_kernel<<<(unsigned)((R + warps - 1) / warps), warps * 32, 0, s>>>(occ, stride, R, L,
-                                                                                N0, bad, stats, bins);
+                                                                                N0, bad, stats);
     return cudaGetLastError();
 }
 
-cudaError_t setup_order(const int32_t *N0, int32_t R, int32_t L, const int32_t *bins, int32_t *next, int32_t *order,
-                        cudaStream_t s)
+cudaError_t setup_order(const int32_t *N0, int32_t R, int32_t L, int32_t *bins, int32_t *next, int32_t *order,
+                        unsigned long long *stats, cudaStream_t s)
 {
-    order_kernel<<<(unsigned)(((int64_t)R + 1023) / 1024), 1024, 0, s>>>(N0, R, L, bins, next, order);
+    const unsigned blocks = (unsigned)(((int64_t)R + 1023) / 1024);
+    bins_kernel<<<blocks, 1024, 0, s>>>(N0, R, L, bins);
+    order_kernel<<<blocks, 1024, 0, s>>>(N0, R, L, bins, next, order, stats);
     return cudaGetLastError();
 }
 
