@@ -159,8 +159,14 @@ int kmc_set_voltage(kmc_handle *h, int64_t first_step, int64_t count, const doub
  * report the total number logged in *n_total (synchronizes). */
 int kmc_near_threshold_log(kmc_handle *h, kmc_log_entry *out, int64_t cap, int64_t *n_total);
 
-/* Device counters since creation: [0] Philox blocks drawn, [1] decisions
- * resolved by the exact FP64 path, [2] accepted moves (synchronizes). */
+/* Device counters since creation (synchronizes): [0] draws, [1] decisions
+ * resolved in FP64, [2] accepted moves.  The first two measure work, depend on
+ * the kernel that ran (kmc_set_accept_path, sizes, filling and the length of
+ * the launches choose it) and are no results.  A draw is one Philox block: on
+ * occupancy words of each ion with a free neighbour, or at an electrode, in
+ * each step; on ion lists of each list entry in each step, which counts
+ * blocked ions and the empty end sites of open rails, and leaves out what is
+ * drawn a second time or for steps that are then drawn again. */
 int kmc_counters(kmc_handle *h, uint64_t out[3]);
 
 /* Launch shape: warps per CTA (1..32, 0 = automatic) and steps between the

@@ -73,7 +73,7 @@ struct SweepArgs {
     kmc_log_entry *log;
     unsigned long long *log_count;
     int64_t log_cap;
-    unsigned long long *counters; // [3] philox blocks, exact decisions, moves
+    unsigned long long *counters; // [3] draws, FP64 decisions, moves (kmc_counters)
     long long *Jr;                // [R] per-rail net leftward crossings, accumulated, or null
     int32_t bnd[kMaxZones + 1];   // zone boundaries floor(z L / Z)
     int32_t wsum[kMaxZones + 1];  // w_{z-1} + w_z (w_{-1} = w_Z = 0)
@@ -233,7 +233,7 @@ TileShape pick_grad_tile(int64_t rails, int64_t n_rails, const kmc_params &p, in
 // shared memory of a CTA at most, and of an SM, for the gradient pass
 void grad_smem_limits(size_t *most, size_t *total, bool ions);
 constexpr int kGradSmem = 226 * 1024;   // dynamic shared memory of a gradient CTA at most
-constexpr int kGradWarps = 20;          // warps of a gradient CTA at most (102 registers)
+constexpr int kGradWarps = 20;          // warps of a gradient CTA at most (96 registers)
 cudaError_t ion_batch_set_smem_limits();
 cudaError_t ion_grad_set_smem_limits();
 int ion_grad_ctas_per_sm(int kind, int warps, size_t smem);

@@ -14,7 +14,7 @@ namespace {
 // Gradient passes (as sweep_grad_kernel and sweep_batch_grad_kernel), 64 rows of
 // bits.  Shared memory, not registers, limits the warps of an SM (on 4 lanes per
 // rail, 8 rails' lists, bounds and score factors are about 13 KB a warp), so a CTA
-// has up to 20 warps of 102 registers.
+// has up to 20 warps of 96 registers.
 template <int P, bool OPEN>
 __global__ void __launch_bounds__(32 * kGradWarps, 1) ion_grad_kernel(const __grid_constant__ SweepArgs a)
 {
