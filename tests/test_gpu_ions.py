@@ -71,6 +71,18 @@ def test_few_sites_on_many_rails(kmc, R, L, Z, electrodes, dt):
     _check(kmc, dev, np.where(np.arange(24) % 6 < 3, 1.0, -0.5), 0.3, [9, 15])
 
 
+# per-site barriers where several rails share a warp (4, 8 and 16 lanes a rail), with
+# and without classes of sites in the bounds' rows
+@pytest.mark.parametrize("R,L", [(49153, 64), (19201, 100), (12289, 300), (6001, 500)])
+@pytest.mark.parametrize("Z", [10, 32])
+@pytest.mark.parametrize("electrodes", [0, 1])
+@pytest.mark.parametrize("dt", [5e-7, 2e-8])
+def test_per_site_barriers_on_few_lanes(kmc, R, L, Z, electrodes, dt):
+    dev = _dev(R=R, L=L, Z=Z, electrodes=electrodes, k_e=1.0 / dt if electrodes else 0.0, rho_e=0.3, dt=dt)
+    Ea = np.maximum(np.random.default_rng(L).normal(0.40, 0.02, (R, L)), 0.35)
+    _check(kmc, dev, np.where(np.arange(20) % 6 < 3, 1.0, -0.5), 0.25, [5, 15], Ea)
+
+
 # more than 32 entries a lane: CTAs of up to 20 warps, in one wave and in several,
 # each with a last CTA that is not full
 @pytest.mark.parametrize("R,L,fill", [(2500, 2048, 0.5), (5001, 1100, 0.25)])
