@@ -50,6 +50,9 @@ BYTES_PER_SITE_UPDATE = 2.0        # uint8 read + write per site and step
 # 32x32->64 widening multiply takes two of the pipe's slots, a low half one:
 # 16 x 2 + 2 = 34.
 PHILOX_IMAD_SLOTS = 34
+# The ion lists look the site's part of rounds 1 and 2 up, one widening multiply
+# each, so a draw of theirs issues 14 x 2 + 2 = 30.
+LIST_IMAD_SLOTS = 30
 IMAD_PER_SM_PER_CLK = 64           # 32-bit integer multiply-add lanes per SM per clock
 SMS = 152
 SM_MAX_MHZ = 2070.0
@@ -363,8 +366,12 @@ def run_kmc(args):
                          "traffic": _traffic_per_launch(R, chunk),
                          "traffic_unit": "DRAM bytes per launch (ncu, scaled by rails)",
                          "peak_basis": "%d SMs x %d IMAD lanes/clk x %.0f MHz / %d IMAD issue slots "
-                                       "per block" % (SMS, IMAD_PER_SM_PER_CLK, sm_max,
-                                                      PHILOX_IMAD_SLOTS),
+                                       "per full block; achieved counts a draw of every list entry "
+                                       "as a full block" % (SMS, IMAD_PER_SM_PER_CLK, sm_max,
+                                                            PHILOX_IMAD_SLOTS),
+                         "issued_frac": achieved / alu_peak * LIST_IMAD_SLOTS / PHILOX_IMAD_SLOTS,
+                         "issued_basis": "%d slots a draw on ion lists, which look two of the "
+                                         "block's products up" % LIST_IMAD_SLOTS,
                          "philox_only_probe": {"achieved": probe, "frac_of_peak": probe / alu_peak,
                                                "sweep_frac_of_probe": achieved / probe,
                                                "basis": "kmc_philox_probe: the draw loop's Philox "
