@@ -165,21 +165,20 @@ int64_t words_up_to(const TileShape &t, int64_t rails, int L, int Z, bool acc)
 // lane and of up to 64 on two, where the lists take four and repeat a warp's fixed work
 // two to eight times as often; zones bring the two together, as a warp evaluates those
 // of all its rails.  65,536 rails, 64 steps, times of the lists over those of the words:
-// with the accept path 1.7 to 0.9 at 8 sites (1 to 8 zones), open 1.6, 1.5, 1.3, 0.99 and
-// 0.54 at 16 sites (1, 2, 4, 7 and 10 zones), closed 1.3, 1.2 and 0.98 (1, 2, 4), open 1.1,
-// 1.1 and 0.97 at 48; without it open 2.0, 1.4, 1.05 and 0.65 at 16 (1, 4, 8, 10), 1.5 to 1.0 at
-// 24 and 32 (1), 1.05 to 0.85 at 48 and 64, and closed below 1 at all.  With fewer rails the words leave SMs idle:
-// from 24,000 on 1.1 to 1.5 at up to 16 sites and two zones, from 4,000 on 1.1 to 1.4 at 8
-// closed ones with the accept path.
+// closed with the accept path 1.7, 1.6, 1.4, 1.3 and 0.9 at 8 sites (1, 2, 4, 7 and 8 zones), 1.3, 1.2
+// and 0.98 at 16 (1, 2, 4); open without it 2.0, 1.4, 1.05 and 0.65 at 16 (1, 4, 8, 10; 40 % full 2.2, 1.9,
+// 1.5 and 0.94), 1.5 to 1.0
+// at 24 and 32 (1), 1.05 to 0.85 at 48 and 64; closed without it below 1 at all; open with it
+// 1.6, 1.3 and 0.54 at 16 (1, 4, 10) under a slow voltage, but 0.7 and 0.4 under one that
+// moves by 8 mV a step, whose draws the words' bands of 32 steps leave to their slow path:
+// these stay on the lists.  With fewer rails the words leave SMs idle: from 24,000 on 1.1
+// to 1.5 at up to 16 sites and two zones, from 4,000 on 1.1 to 1.4 at 8 closed ones with the
+// accept path.
 static bool words_for_few_sites(int64_t rails, int L, int Z, bool open, bool acc)
 {
     int most = 0;       // zones
-    if (L > 64) return false;
-    if (rails >= 40000)
-        most = acc ? (open ? (L < 16 ? 6 : L <= 32 ? 4 : 2) : (L < 16 ? 7 : L <= 32 ? 2 : 0))
-                   : (open ? (L < 24 ? 8 : L <= 32 ? 2 : 0) : 0);
-    else if (acc && !open && L < 16 && rails >= 4000) most = 3;
-    else if (!acc && open && L < 24 && rails >= 20000) most = 2;
+    if (acc && !open) most = rails >= 40000 ? (L < 16 ? 7 : L <= 32 ? 2 : 0) : rails >= 4000 && L < 16 ? 3 : 0;
+    if (!acc && open) most = rails >= 40000 ? (L < 24 ? 9 : L <= 32 ? 2 : 0) : rails >= 20000 && L < 24 ? 2 : 0;
     return Z <= most;
 }
 
@@ -302,23 +301,19 @@ int ion_cta_warps(const SweepArgs &a, int kind, int64_t warps)
 //
 // The words take fewer lanes for a rail of few sites, so their warps repeat the fixed
 // work less often; the lists evaluate fewer zones (only where an ion crossed a
-// boundary).  Lists' time over the words', 64 steps at 20 % filling:
-//  * 4,000 rails (16 and 32 lanes on the lists): 1.05 to 1.4 where the words' lanes take
-//    a rail's zones at once, 0.4 to 0.97 where they don't (up to 256 sites);
-//  * 65,536: closed 1.9, 1.4, 1.05, 0.8 at 32 sites (1, 2, 4, 7 zones), 1.3, 1.3, 0.95 at 64 (1, 2, 4);
-//    open 2.3, 1.7, 1.3, 0.97 at 32 and 1.4, 1.4, 1.15 at 64; 24,000: a few per cent to a third less;
-//  * open rails of up to 16 zones, when their warps' shared memory makes more than one
-//    wave: 1.0 to 1.4 at up to 64 sites (10 zones), 0.95 to 1.3 at 128 (16), in one wave 0.75 to 0.9.
-static bool words_for_gradient(int64_t rails, int L, int Z, bool open, int waves)
+// boundary), and a voltage that moves does not widen their bounds as much.  Lists' time
+// over the words', 64 steps at 20 % filling under a slow voltage: 65,536 rails closed 1.9,
+// 1.4, 1.05 and 0.8 at 32 sites (1, 2, 4 and 7 zones), 1.3, 1.3 and 0.95 at 64 (1, 2, 4), open 2.3, 1.7, 1.3
+// and 0.97 at 32 and 1.4, 1.4, 1.15 at 64; 24,000 rails closed 1.4, 1.15 and 0.83 at 32 (1, 2, 4), open 1.5, 1.3
+// and 0.95; open rails whose lists make two waves by their shared memory (10 zones) 1.3 at
+// up to 32 sites and 1.0 to 1.4 at 64, in one wave (7 zones) 0.75.  On fewer rails, and on
+// longer ones, each side wins somewhere (1,500 to 4,000 rails of one zone: 0.6 to 1.3 by
+// filling and voltage): they stay on the lists.
+static bool words_for_gradient(int64_t rails, int L, int Z, bool open, int64_t waves)
 {
-    int wpl = 1;
-    const int lpr = sweep_pick_lpr(L, &wpl);
-    if (rails < 1200 || L > 256) return false;
-    if (rails < 9600) return Z <= lpr;
-    if (rails < 16000 || L > 128) return false;
-    if (open && waves > 1 && Z <= (L <= 64 ? 10 : 16)) return true;
-    if (L <= 32) return Z <= (rails >= 40000 ? 4 : 3);
-    return L <= 64 && Z <= (rails >= 40000 ? 2 : 1);
+    if (rails < 16000 || L > 64) return false;
+    if (open && waves > 1 && (rails < 40000 || L > 32) && Z <= 10) return true;
+    return Z <= (rails >= 40000 ? (L <= 32 ? 4 : 2) : (L <= 32 ? 3 : 0));
 }
 
 TileShape pick_grad_tile(int64_t rails, int64_t n_rails, const kmc_params &p, int64_t n_tot, int64_t n_max)
@@ -342,7 +337,7 @@ TileShape pick_grad_tile(int64_t rails, int64_t n_rails, const kmc_params &p, in
         const int w = grad_warps(t, p, most, total, rails, sms);
         SweepArgs a;
         const int64_t resident = (int64_t)w * std::max<int>(1, std::min<int>((int)(total / (grad_tile_args(a, t, p, w) + 1024)), kGradWarps / w));
-        const int waves = (rails * P / 32 + sms * resident - 1) / (sms * resident) > 1 ? 2 : 1;
+        const int64_t waves = (rails * P / 32 + sms * resident - 1) / (sms * resident);
         if (!words_for_gradient(rails, L, p.n_zones, open, waves)) return t;
         t = TileShape{};
     }
