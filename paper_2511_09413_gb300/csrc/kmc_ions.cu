@@ -166,14 +166,13 @@ int64_t words_up_to(const TileShape &t, int64_t rails, int L, int Z, bool acc)
 // two to eight times as often; zones bring the two together, as a warp evaluates those
 // of all its rails.  65,536 rails, 64 steps, times of the lists over those of the words:
 // closed with the accept path 1.7, 1.6, 1.4, 1.3 and 0.9 at 8 sites (1, 2, 4, 7 and 8 zones), 1.3, 1.2
-// and 0.98 at 16 (1, 2, 4); open without it 2.0, 1.4, 1.05 and 0.65 at 16 (1, 4, 8, 10; 40 % full 2.2, 1.9,
-// 1.5 and 0.94), 1.5 to 1.0
-// at 24 and 32 (1), 1.05 to 0.85 at 48 and 64; closed without it below 1 at all; open with it
-// 1.6, 1.3 and 0.54 at 16 (1, 4, 10) under a slow voltage, but 0.7 and 0.4 under one that
-// moves by 8 mV a step, whose draws the words' bands of 32 steps leave to their slow path:
-// these stay on the lists.  With fewer rails the words leave SMs idle: from 24,000 on 1.1
-// to 1.5 at up to 16 sites and two zones, from 4,000 on 1.1 to 1.4 at 8 closed ones with the
-// accept path.
+// and 0.98 at 16 (1, 2, 4); open without it 2.0, 1.4, 1.05 and 0.65 at 16 (1, 4, 8, 10; 40 % full
+// 2.2, 1.9, 1.5 and 0.94), 1.5 to 1.0 at 24 and 32 (1), 1.05 to 0.85 at 48 and 64; closed
+// without it below 1 at all; open with it 1.6, 1.3 and 0.54 at 16 (1, 4, 10) under a slow
+// voltage, but 0.7 and 0.4 under one that moves by 8 mV a step, whose draws the words' bands
+// of 32 steps leave to their slow path: these stay on the lists.  With fewer rails the words
+// leave SMs idle: from 24,000 on 1.1 to 1.5 at up to 16 sites and two zones, from 4,000 on 1.1
+// to 1.4 at 8 closed ones with the accept path.
 static bool words_for_few_sites(int64_t rails, int L, int Z, bool open, bool acc)
 {
     int most = 0;       // zones

@@ -10,7 +10,7 @@
 // when an ion moves (no popcount scan, free-neighbour masks or compaction of
 // candidates): every lane draws for its next ion in every iteration.  Ions
 // with both neighbours occupied draw in vain, so fuller rails stay with the
-// occupancy words (pick_tile).
+// occupancy words (pick_tile, tile_gate).
 //
 //  * Zone sums.  The number of ions below each zone boundary, P_b, and
 //    F = sum_b P_b w_b are updated when an ion crosses a boundary, and the

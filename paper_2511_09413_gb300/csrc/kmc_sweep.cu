@@ -1,8 +1,8 @@
 // kmc_sweep.cu -- the per-time-step sweep over every rail and site
 // (arXiv 2511.09413, Supplementary S2.1.2 - S2.1.7) on occupancy words,
-// hand-written for sm_103a.  It advances the fuller rails and those of less than
-// 8 sites; the others run on ion lists (kmc_ions.cuh; pick_tile has the line
-// between them and both sides' rates).
+// hand-written for sm_103a.  It advances the fuller rails, those of few sites and
+// launches of a few steps; the others run on ion lists (kmc_ions.cuh; kmc_ions.cu
+// has the lines between them and both sides' times).
 //
 // Design (GB300):
 //  * A rail lives in registers as a bitmask: lane l of a rail's lane segment
